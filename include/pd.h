@@ -312,9 +312,9 @@ pd_status pd_set_graph_mode(pd_sim* sim, int enable, int poisson_cycles);
  * work with a grid-stride loop and writes results that do not depend on the
  * order in which threads run (integer atomics, per-cell work, canonical id
  * order), so a shape changes speed only, never a result.  Grids are given
- * in blocks per SM (1..64); mg_threads is the block size of the multigrid
- * level kernels (a multiple of 32 in 64..1024) and mg_max_blocks caps their
- * blocks per run and level (1..65535).  pd_set_tuning validates and drops
+ * in blocks per SM (1..64); mg_threads is the block size of the field solve's
+ * node kernels (right-hand side and history, E; a multiple of 32 in 64..1024)
+ * and mg_max_blocks caps their blocks per run (1..65535).  pd_set_tuning validates and drops
  * a captured graph. */
 typedef struct pd_tuning {
     int push_blocks_per_sm;     /* push + gather + deposit (256 threads) */

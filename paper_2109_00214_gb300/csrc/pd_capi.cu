@@ -613,7 +613,7 @@ size_t total_nodes(const pd_sim* s) { return (size_t)s->L.nodes; }
 // shift once two solutions exist)
 pd_status warm_start(pd_sim* s, int* kernels) {
     const bool extrapolate = s->warm_mode == PD_WARM_EXTRAPOLATE && s->solves >= 2;
-    warm_history(s->field, s->rho_e, s->rho_h, s->runs_dev, s->rs, s->phi, s->whist, extrapolate, s->stream);
+    field_begin(s->field, s->rho_e, s->rho_h, s->runs_dev, s->rs, s->whist, extrapolate, s->stream);
     *kernels += 1;
     // the learned forms need one (delta) or two (extrapolated) earlier
     // solves; until then the previous potential stands
@@ -646,11 +646,10 @@ pd_status prime(pd_sim* s) {
         launch_deposit(s->A, s->rho_e, s->rho_h, s->st, P, grid_for(s, 8), s->stream);
     }
     if (s->cfgs[0].field_mode == PD_FIELD_POISSON) {
-        Timed t(s, K_POISSON, false, 2);   // + the warm start's and the solve's kernels, counted below
+        Timed t(s, K_POISSON, false, 1);   // E; + the warm start's and the solve's kernels, counted below
         int nk = 0;
         if (warm_start(s, &nk) != PD_OK) return fail(s, PD_ERR_CUDA, "warm start failed");
-        const cudaError_t fe = field_solve(s->field, s->rho_e, s->rho_h, s->phi, s->E, s->runs_dev, s->rs, 1, 0,
-                                           s->stream, &nk);
+        const cudaError_t fe = field_solve(s->field, s->rs, 1, 0, s->stream, &nk);
         if (fe != cudaSuccess) return cuda_fail(s, fe, "field solve");
         s->launches[K_POISSON] += (uint64_t)nk;
         field_efield(s->field, s->phi, s->runs_dev, s->E, s->st, s->rs, s->stream);
@@ -764,13 +763,12 @@ pd_status issue_step(pd_sim* s, bool capturing) {
             int nk = 0;
             if (warm_start(s, &nk) != PD_OK) return fail(s, PD_ERR_CUDA, "warm start failed");
             const bool host_check = !capturing && !s->graph_on;
-            const cudaError_t fe = field_solve(s->field, s->rho_e, s->rho_h, s->phi, s->E, s->runs_dev, s->rs,
-                                               host_check ? 1 : 0, s->graph_cycles, s->stream, &nk);
+            const cudaError_t fe = field_solve(s->field, s->rs, host_check ? 1 : 0, s->graph_cycles, s->stream, &nk);
             if (fe != cudaSuccess) return cuda_fail(s, fe, "field solve");
             s->launches[K_POISSON] += (uint64_t)nk;
         }
         {
-            Timed t(s, K_EFIELD, capturing, 2);
+            Timed t(s, K_EFIELD, capturing, 1);
             field_efield(s->field, s->phi, s->runs_dev, s->E, s->st, s->rs, s->stream);
         }
     }

@@ -19,15 +19,18 @@
 // each correction is accurate to a few digits, and phi reaches residuals far
 // below float precision.
 //
-// V-cycle: red-black Gauss-Seidel (four half-sweeps per launch through a
-// shared-memory tile), restriction of the integrated residuals by full
-// weighting (1, 1/2, 1/4), bilinear prolongation, coefficients rediscretised
-// on each level, and an exact solve on the coarsest level by its inverse
-// (formed on the host once; Gauss-Seidel sweeps instead when the coarsest
-// level has more than MG_DIRECT_MAX unknowns).
+// V-cycle: red-black Gauss-Seidel (four half-sweeps per launch, a warp a tile
+// of the grid in its registers), restriction of the integrated residuals by
+// full weighting (1, 1/2, 1/4), bilinear prolongation, coefficients
+// rediscretised on each level, and an exact solve on the coarsest level by its
+// inverse (formed on the host once; Gauss-Seidel sweeps instead when the
+// coarsest level has more than MG_DIRECT_MAX unknowns).  A level takes one
+// launch on the way down (smoothing, residual and restriction), one on the way
+// up (prolongation and smoothing); the levels of at most 34 x 34 nodes take one
+// launch together, and the residual with its norm the last of a cycle.
 //
-// Batched over runs: the per-cycle kernels take work lists of (run, tile or
-// chunk) per level, so a launch has only blocks with work; a run that has
+// Batched over runs: the per-cycle kernels take work lists of (run, tile) per
+// level, so a launch has only warps with work; a run that has
 // converged skips the rest of the cycles.  Per-run residual norms and
 // converged flags stay on the device.
 #include <algorithm>
@@ -43,12 +46,18 @@ namespace {
 constexpr double QE_ = 1.602176634e-19;
 constexpr double EPS0_ = 8.8541878128e-12;
 constexpr double PI_ = 3.14159265358979323846;
-constexpr int RED_BLOCKS = 256;      // blocks of a run's residual (a fixed shape: the summation order is fixed)
-constexpr int MAP_CHUNK = 256;         // items of one work-list entry
-constexpr int SP_TI = 32, SP_TJ = 32;  // smoother tile: interior rows x radial nodes
-constexpr int SP_H = 4;                // halo: four half-sweeps per launch
+constexpr int RED_ROWS = 8;            // a warp's part of the residual: 32 radial nodes x 8 rows
+constexpr int TILE_WARPS = 4;          // tiles of a block of the smoothing kernels
+// A smoothing tile is a window of 64 radial nodes x K rows, two columns to a
+// lane and the rows in registers; each half-sweep spoils a ring of the window,
+// so a tile gives the window less 4 nodes a side (post-smoothing), or less 6
+// (pre-smoothing, whose restriction reads two nodes further).
+constexpr int WIN_C = 64, PRE_H = 6, POST_H = 4;
+constexpr int K_SMALL = 20, K_LARGE = 32;
+constexpr int SMALL_TILES = 4 * 152;   // long windows from this many tiles on
 constexpr int TAIL_NODES = 34 * 34;    // levels from the first one with at most this many nodes: k_mg_tail
 constexpr int TAIL_THREADS = 512;
+constexpr int TAIL_SLOTS = 2;          // nodes of a color a thread of k_mg_tail holds (at most 766 a level)
 
 size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 
@@ -83,8 +92,11 @@ size_t tail_floats(const int* a, const int* b, int n) {
     return t;
 }
 
-int chunks(long long n) { return (int)((n + MAP_CHUNK - 1) / MAP_CHUNK); }
-int tiles_of(int nz, int nr) { return ((nz - 1 + SP_TI - 1) / SP_TI) * ((nr + 1 + SP_TJ - 1) / SP_TJ); }
+int tiles_of(int nz, int nr, int K, int halo) {
+    const int ti = K - 2 * halo, tj = WIN_C - 2 * halo;
+    return ((nz + ti - 1) / ti) * ((nr + tj) / tj);
+}
+int red_units(int nz, int nr) { return ((nz - 1 + RED_ROWS - 1) / RED_ROWS) * ((nr + 32) / 32); }
 
 // work-list entries of one run (all levels that smooth)
 size_t run_tasks(int nz, int nr) {
@@ -92,8 +104,8 @@ size_t run_tasks(int nz, int nr) {
     level_dims(nz, nr, a, b, n);
     size_t t = 0;
     for (int l = 0; l + 1 < n; ++l)
-        t += chunks((long long)(a[l + 1] + 1) * (b[l + 1] + 1)) + tiles_of(a[l], b[l]);
-    return t;
+        t += tiles_of(a[l], b[l], K_SMALL, PRE_H) + tiles_of(a[l], b[l], K_SMALL, POST_H);
+    return t + (red_units(nz, nr) + 7) / 8;
 }
 
 // device bytes of one run, in the order field_init takes them
@@ -106,6 +118,7 @@ size_t run_bytes(int nz, int nr) {
         const size_t W = (size_t)b[l] + 1, nodes = ((size_t)a[l] + 1) * W;
         t += 3 * al(nodes * 4) + 4 * al(W * 4);             // e, e2, f; ap, am, b, dinv in float
     }
+    for (int l = tail_level(a, b, n); l < n; ++l) t += al(4 * ((size_t)b[l] + 1) * 4);   // k_mg_tail's coefficients
     const size_t m = (size_t)coarse_unknowns(a, b, n);
     if (m <= (size_t)MG_DIRECT_MAX) t += al(m * m * 4);
     return t;
@@ -121,83 +134,78 @@ bool field_grid_ok(int nz, int nr) {
 size_t field_workspace_bytes(const std::vector<int>& nz, const std::vector<int>& nr) {
     size_t t = 0;
     const size_t R = nz.size();
-    size_t tasks = 0;
+    size_t tasks = 0, red = 0;
     for (size_t r = 0; r < R; ++r) {
         t += run_bytes(nz[r], nr[r]);
         tasks += run_tasks(nz[r], nr[r]);
+        red += (red_units(nz[r], nr[r]) + 7) / 8;
     }
     t += al(R * MG_MAX_LEVELS * sizeof(MGLevel)) + al(R * sizeof(MGTop)) + al(R * 4) * 3 +
-         al(R * RED_BLOCKS * 2 * 8) + al(R * 8) * 2 + al(R * sizeof(float*)) + al(tasks * sizeof(int2) + 8);
+         al(red * 2 * 8) + al(R * 8) * 2 + al(R * sizeof(TailRun)) + al(tasks * sizeof(int2) + 8);
     return t;
 }
 
 // ------------------------------------------------------------------
 // kernels
 // ------------------------------------------------------------------
-// b (double) and the electrode rows of phi of every run (blockIdx.y = run)
-__global__ void k_rhs(const long long* rho_e, const long long* rho_h, const MGTop* top, const RunInfo* runs,
-                      const RunState* rs) {
-    const int run = blockIdx.y;
-    const MGTop T = top[run];
-    const uint32_t nb = runs[run].node_base;
-    const int W = T.nr + 1;
-    const int n = (T.nz + 1) * W;
-    const double V = rs[run].V;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-        const int i = k / W, j = k - i * W;
-        if (i == 0 || i == T.nz) {
-            T.phi[k] = i == 0 ? 0.0 : V;
-            T.bf[k] = 0.0;
-            continue;
-        }
-        double v = (double)(rho_e[nb + k] + rho_h[nb + k]) * T.cr[j];
-        if (i == T.nz - 1) v += T.b[j] * V;
-        T.bf[k] = v;
-    }
-}
-
-// (A x)_ij on an interior node of a correction level, float
-__device__ __forceinline__ float apply_Af(const MGLevel& L, const float* x, int i, int j) {
-    const int W = L.nr + 1;
-    const int k = i * W + j;
-    float s = (L.ap[j] + L.am[j] + 2.0f * L.b[j]) * x[k];
-    if (j < L.nr) s -= L.ap[j] * x[k + 1];
-    if (j > 0) s -= L.am[j] * x[k - 1];
-    if (i + 1 < L.nz) s -= L.b[j] * x[k + W];
-    if (i - 1 > 0) s -= L.b[j] * x[k - W];
-    return s;
-}
-
-// The residual r = b - A phi of every run in double, per-block partial sums
-// of r^2 (and, with with_b, of b^2) for its norm, and the right-hand side of
-// the next correction: level 0's f = r (float).
-// blockIdx.y = run; block x takes the interior rows x, x + RED_BLOCKS, ...
-// with the threads along the row.  A fixed launch shape, so the summation
-// order (and the cycle count) never depends on tuning.
-__global__ void __launch_bounds__(256) k_residual_norms(const MGTop* top, const MGLevel* lev, const int* nlev,
-                                                        double* red, int with_b) {
-    const int run = blockIdx.y;
+// The residual r = b - A phi of every run in double, its norm (and, on the
+// first of a solve, that of b), and the right-hand side of the next correction:
+// level 0's f = r (float).  A warp takes 32 radial nodes and marches over
+// RED_ROWS rows, so that each node of phi is read once a row, not three times;
+// double arithmetic (seven operations a node) bounds it on a large grid.  Work
+// list of (run, first unit), eight units a block; the block that finishes a
+// run's last units sums the blocks' parts in their order and judges the run:
+// relres = |r| / |b|, converged flag, bookkeeping.
+// 512 x 512 cells, device time of a launch under ncu: 14.7 us with the norm (13.8
+// + 8.9 us as a launch of rows and one of norms).
+__global__ void __launch_bounds__(256) k_residual_norms(const MGTop* top, const MGLevel* lev, const int2* tasks,
+                                                        const int* red_base, double* red, unsigned int* ticket,
+                                                        double* bnorm, int* done, const double* tol, RunState* rs,
+                                                        int cycle) {
+    const int2 tk = tasks[blockIdx.x];
+    const int run = tk.x;
+    if (cycle > 0 && done[run]) return;
+    const MGTop& T = top[run];
+    const int nz = T.nz, nr = T.nr, W = nr + 1;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int cols = (W + 31) / 32, rows = (nz - 1 + RED_ROWS - 1) / RED_ROWS;
+    const int u = tk.y + w;
     double acc = 0.0, accb = 0.0;
-    if (nlev[run] > 0) {
-        const MGTop T = top[run];
-        const MGLevel L = lev[run * MG_MAX_LEVELS];
-        const int W = T.nr + 1;
-        const double* x = T.phi;
-        for (int i = 1 + blockIdx.x; i < T.nz; i += RED_BLOCKS) {
-            for (int j = threadIdx.x; j < W; j += blockDim.x) {
-                const int k = i * W + j;
-                const double xp = j < T.nr ? x[k + 1] : 0.0;
-                const double xm = j > 0 ? x[k - 1] : 0.0;
-                const double xu = i + 1 < T.nz ? x[k + W] : 0.0;     // the anode row is in b
-                const double xd = i - 1 > 0 ? x[k - W] : 0.0;
-                const double bk = T.bf[k];
-                double r = bk - T.dg[j] * x[k];
-                r += T.ap[j] * xp;
-                r += T.am[j] * xm;
-                r += T.b[j] * (xu + xd);
-                L.f[k] = (float)r;
-                acc += r * r;
-                if (with_b) accb += bk * bk;
+    if (u < cols * rows) {
+        const int j = (u % cols) * 32 + lane, i0 = 1 + (u / cols) * RED_ROWS, i1 = min(i0 + RED_ROWS, nz);
+        if (j < W) {
+            const double *x = T.phi, *bf = T.bf;
+            float* f = lev[run * MG_MAX_LEVELS].f;
+            const double dg = T.dg[j], ap = T.ap[j], am = T.am[j], bz = T.b[j];
+            // every load before the first use: their latencies overlap
+            double xc[RED_ROWS + 2], xp[RED_ROWS], xm[RED_ROWS], bk[RED_ROWS];
+            const int rt = j < nr ? 1 : 0, lf = j > 0 ? 1 : 0;
+#pragma unroll
+            for (int q = 0; q < RED_ROWS + 2; ++q) {
+                const int i = min(i0 - 1 + q, nz);
+                xc[q] = x[i * W + j];
+            }
+#pragma unroll
+            for (int q = 0; q < RED_ROWS; ++q) {
+                const int k = min(i0 + q, nz) * W + j;
+                xp[q] = x[k + rt];
+                xm[q] = x[k - lf];
+                bk[q] = bf[k];
+            }
+#pragma unroll
+            for (int q = 0; q < RED_ROWS; ++q) {
+                const int i = i0 + q;
+                if (i < i1) {
+                    const double xu = i + 1 < nz ? xc[q + 2] : 0.0;      // the anode row is in b
+                    const double xd = i - 1 > 0 ? xc[q] : 0.0;
+                    double r = bk[q] - dg * xc[q + 1];
+                    r += ap * xp[q];                                     // ap = 0 on the last column
+                    r += am * xm[q];                                     // am = 0 on the axis
+                    r += bz * (xu + xd);
+                    f[i * W + j] = (float)r;
+                    acc += r * r;
+                    if (cycle == 0) accb += bk[q] * bk[q];
+                }
             }
         }
     }
@@ -205,298 +213,433 @@ __global__ void __launch_bounds__(256) k_residual_norms(const MGTop* top, const 
         acc += __shfl_down_sync(0xFFFFFFFFu, acc, o);
         accb += __shfl_down_sync(0xFFFFFFFFu, accb, o);
     }
-    __shared__ double sa[32], sb[32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    __shared__ double sa[8], sb[8];
+    __shared__ bool s_last;
     if (lane == 0) {
         sa[w] = acc;
         sb[w] = accb;
     }
     __syncthreads();
+    const int blocks = (cols * rows + 7) / 8;
+    double* rd = red + 2 * (size_t)red_base[run];
     if (threadIdx.x == 0) {
         double t = 0, tb = 0;
-        for (int q = 0; q < (int)(blockDim.x >> 5); ++q) {
+        for (int q = 0; q < 8; ++q) {
             t += sa[q];
             tb += sb[q];
         }
-        red[(run * RED_BLOCKS + blockIdx.x) * 2] = t;
-        if (with_b) red[(run * RED_BLOCKS + blockIdx.x) * 2 + 1] = tb;
+        __stcg(&rd[2 * (tk.y / 8)], t);
+        __stcg(&rd[2 * (tk.y / 8) + 1], tb);
+        __threadfence();
+        s_last = atomicAdd(&ticket[run], 1u) == (unsigned int)(blocks - 1);
     }
-}
-
-// per run (one warp each): relres = |r| / |b| (|b| from the first call of
-// the solve), converged flag, bookkeeping
-__global__ void k_norms(const double* red, double* bnorm, int* done, const double* tol, RunState* rs, int nruns,
-                        int cycle, int first) {
-    const int run = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    if (run >= nruns) return;
-    double a = 0, b = 0;
-    for (int q = lane; q < RED_BLOCKS; q += 32) {
-        a += red[(run * RED_BLOCKS + q) * 2];
-        if (first) b += red[(run * RED_BLOCKS + q) * 2 + 1];
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    acc = accb = 0.0;
+    for (int q = threadIdx.x; q < blocks; q += 256) {
+        acc += __ldcg(&rd[2 * q]);
+        accb += __ldcg(&rd[2 * q + 1]);
     }
     for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_down_sync(0xFFFFFFFFu, a, o);
-        b += __shfl_down_sync(0xFFFFFFFFu, b, o);
+        acc += __shfl_down_sync(0xFFFFFFFFu, acc, o);
+        accb += __shfl_down_sync(0xFFFFFFFFu, accb, o);
     }
-    if (lane != 0) return;
+    if (lane == 0) {
+        sa[w] = acc;
+        sb[w] = accb;
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    double a = 0, b = 0;
+    for (int q = 0; q < 8; ++q) {
+        a += sa[q];
+        b += sb[q];
+    }
+    ticket[run] = 0u;
     const double rn = sqrt(a);
-    if (first) {
-        done[run] = 0;
-        bnorm[run] = sqrt(b);
-    }
-    if (done[run]) return;
+    if (cycle == 0) bnorm[run] = sqrt(b);
     const double bn = bnorm[run];
     const double rel = bn > 0 ? rn / bn : 0.0;
     rs[run].relres = rel;
     rs[run].cycles = (double)cycle;
-    if (first) rs[run].relres0 = rel;
-    if (!(rel == rel) || !(bn == bn)) {
-        done[run] = 2;              // non-finite: stop this run
-        return;
-    }
-    if (bn == 0.0 || rel <= tol[run]) done[run] = 1;
+    if (cycle == 0) rs[run].relres0 = rel;
+    int d = 0;
+    if (!(rel == rel) || !(bn == bn)) d = 2;              // non-finite: stop this run
+    else if (bn == 0.0 || rel <= tol[run]) d = 1;
+    done[run] = d;
 }
 
-// Four half-sweeps of red-black Gauss-Seidel on A e = f (colors c1, c2, c1,
-// c2: two iterations) in one launch, on a tile of SP_TI interior rows x SP_TJ
-// radial nodes in shared memory: the k-th half-sweep updates the tile grown
-// by 3 - k rings, so the tile's own nodes end exact (the result of four
-// separate half-sweeps).  The work list gives each block its (run, tile).
-// Pre-smoothing (POST false, colors 0, 1, 0, 1): starts from e = 0 (the
-// correction of a level is zero when its cycle begins) and writes e2.
-// Post-smoothing (POST true, colors 1, 0, 1, 0): starts from e2 plus the
-// bilinear prolongation of level l + 1's correction (its e), and writes e,
-// or, with FINAL (level 0), adds the tile to phi.  No block reads what
-// another block of the same launch writes.
-template <bool POST, bool FINAL>
-__global__ void __launch_bounds__(256) k_smooth4(const MGLevel* lev, const MGTop* top, const int* done, int l,
-                                                 const int2* tasks) {
-    constexpr int XR = SP_TI + 2 * SP_H, XC = SP_TJ + 2 * SP_H, FR = XR - 2, FC = XC - 2;
-    __shared__ float xs[XR][XC + 1];
-    __shared__ float fsm[FR][FC];
-    __shared__ float cap[FC], cam[FC], cb[FC], cd[FC];
-    const int2 tk = tasks[blockIdx.x];
-    const int run = tk.x;
-    if (done[run]) return;
-    const int c1 = POST ? 1 : 0;
-    const MGLevel L = lev[run * MG_MAX_LEVELS + l];
+// The window of a warp's tile: two columns a lane (j = j0 + 2 lane and the next),
+// K rows from i0, both even, so that which of a lane's columns has a color
+// follows from the row's number alone.
+template <int K>
+struct Window {
+    float x0[K], x1[K], f0[K], f1[K];
+    float ap0, am0, b0, d0, ap1, am1, b1, d1;
+};
+
+// the coefficients of the lane's columns (zero outside the grid: such nodes stay
+// zero) and the right-hand side
+template <int K>
+__device__ __forceinline__ void window_load(Window<K>& w, const MGLevel& L, int i0, int j) {
     const int W = L.nr + 1;
-    const int tj = (W + SP_TJ - 1) / SP_TJ;
-    const int i0 = 1 + (tk.y / tj) * SP_TI, j0 = (tk.y % tj) * SP_TJ;
-    if (POST) {
-        const MGLevel Cl = lev[run * MG_MAX_LEVELS + l + 1];
-        const int Wc = Cl.nr + 1;
-        const float* ce = Cl.e;
-        for (int q = threadIdx.x; q < XR * XC; q += blockDim.x) {
-            const int a = q / XC, c = q % XC;
-            const int i = i0 - SP_H + a, j = j0 - SP_H + c;
-            float v = 0.0f;
-            // only interior rows are read by the update (the corrections vanish on the electrodes)
-            if (i >= 1 && i <= L.nz - 1 && j >= 0 && j <= L.nr) {
-                const int I0 = i >> 1, J0 = j >> 1;
-                const int I1 = (i & 1) ? I0 + 1 : I0, J1 = (j & 1) ? J0 + 1 : J0;
-                const float cc =
-                    0.25f * (ce[I0 * Wc + J0] + ce[I1 * Wc + J0] + ce[I0 * Wc + J1] + ce[I1 * Wc + J1]);
-                v = L.e2[i * W + j] + cc;
-            }
-            xs[a][c] = v;
-        }
-    } else {
-        for (int q = threadIdx.x; q < XR * (XC + 1); q += blockDim.x) (&xs[0][0])[q] = 0.0f;
+    const bool in0 = j >= 0 && j <= L.nr, in1 = j + 1 >= 0 && j + 1 <= L.nr;
+    w.ap0 = in0 ? L.ap[j] : 0.0f;
+    w.am0 = in0 ? L.am[j] : 0.0f;
+    w.b0 = in0 ? L.b[j] : 0.0f;
+    w.d0 = in0 ? L.dinv[j] : 0.0f;
+    w.ap1 = in1 ? L.ap[j + 1] : 0.0f;
+    w.am1 = in1 ? L.am[j + 1] : 0.0f;
+    w.b1 = in1 ? L.b[j + 1] : 0.0f;
+    w.d1 = in1 ? L.dinv[j + 1] : 0.0f;
+    const float* f = L.f;
+#pragma unroll
+    for (int r = 0; r < K; ++r) {
+        const int i = i0 + r;
+        const bool in = i >= 1 && i <= L.nz - 1;
+        const int k = i * W + j;
+        w.f0[r] = in && in0 ? f[k] : 0.0f;
+        w.f1[r] = in && in1 ? f[k + 1] : 0.0f;
     }
-    for (int q = threadIdx.x; q < FR * FC; q += blockDim.x) {
-        const int a = q / FC, c = q % FC;
-        const int i = i0 - SP_H + 1 + a, j = j0 - SP_H + 1 + c;
-        fsm[a][c] = (i >= 1 && i <= L.nz - 1 && j >= 0 && j <= L.nr) ? L.f[i * W + j] : 0.0f;
-    }
-    for (int c = threadIdx.x; c < FC; c += blockDim.x) {
-        const int j = j0 - SP_H + 1 + c;
-        const bool in = j >= 0 && j <= L.nr;
-        cap[c] = in ? L.ap[j] : 0.0f;
-        cam[c] = in ? L.am[j] : 0.0f;
-        cb[c] = in ? L.b[j] : 0.0f;
-        cd[c] = in ? L.dinv[j] : 0.0f;
-    }
-    __syncthreads();
-#pragma unroll 1
-    for (int k = 0; k < 4; ++k) {
-        const int grow = 3 - k, color = (k & 1) ? 1 - c1 : c1;
-        // the nodes of one color: half of each row of the grown tile
-        const int rows = SP_TI + 2 * grow, half = (SP_TJ + 2 * grow) / 2;
-        for (int q = threadIdx.x; q < rows * half; q += blockDim.x) {
-            const int ii = q / half, jj = q - ii * half;
-            const int i = i0 - grow + ii;
-            const int jf = j0 - grow;                                   // first column of the row
-            const int j = jf + 2 * jj + (((i + jf) & 1) != color ? 1 : 0);
-            if (i < 1 || i > L.nz - 1 || j < 0 || j > L.nr) continue;
-            const int a = i - i0 + SP_H, c = j - j0 + SP_H, fa = a - 1, fc = c - 1;
-            float v = fsm[fa][fc];
-            if (j < L.nr) v += cap[fc] * xs[a][c + 1];
-            if (j > 0) v += cam[fc] * xs[a][c - 1];
-            if (i + 1 < L.nz) v += cb[fc] * xs[a + 1][c];
-            if (i - 1 > 0) v += cb[fc] * xs[a - 1][c];
-            xs[a][c] = v * cd[fc];
-        }
-        __syncthreads();
-    }
-    if (FINAL) {
-        double* phi = top[run].phi;
-        for (int q = threadIdx.x; q < SP_TI * SP_TJ; q += blockDim.x) {
-            const int i = i0 + q / SP_TJ, j = j0 + q % SP_TJ;
-            if (i <= L.nz - 1 && j <= L.nr) phi[i * W + j] += (double)xs[i - i0 + SP_H][j - j0 + SP_H];
-        }
-    } else {
-        float* out = POST ? L.e : L.e2;
-        for (int q = threadIdx.x; q < SP_TI * SP_TJ; q += blockDim.x) {
-            const int i = i0 + q / SP_TJ, j = j0 + q % SP_TJ;
-            if (i <= L.nz - 1 && j <= L.nr) out[i * W + j] = xs[i - i0 + SP_H][j - j0 + SP_H];
+}
+
+// One half-sweep of red-black Gauss-Seidel on A e = f: the nodes with (i + j) & 1
+// == C.  Rows outside the grid stay zero.
+template <int K, int C>
+__device__ __forceinline__ void window_sweep(Window<K>& w, int i0, int nz) {
+#pragma unroll
+    for (int r = 0; r < K; ++r) {
+        const bool in = i0 + r >= 1 && i0 + r <= nz - 1;
+        if (((C + r) & 1) == 0) {
+            const float xl = __shfl_up_sync(0xFFFFFFFFu, w.x1[r], 1);
+            float v = w.f0[r];
+            v = fmaf(w.ap0, w.x1[r], v);
+            v = fmaf(w.am0, xl, v);
+            if (r + 1 < K) v = fmaf(w.b0, w.x0[r + 1 < K ? r + 1 : r], v);
+            if (r > 0) v = fmaf(w.b0, w.x0[r > 0 ? r - 1 : r], v);
+            w.x0[r] = in ? v * w.d0 : 0.0f;
+        } else {
+            const float xr = __shfl_down_sync(0xFFFFFFFFu, w.x0[r], 1);
+            float v = w.f1[r];
+            v = fmaf(w.ap1, xr, v);
+            v = fmaf(w.am1, w.x0[r], v);
+            if (r + 1 < K) v = fmaf(w.b1, w.x1[r + 1 < K ? r + 1 : r], v);
+            if (r > 0) v = fmaf(w.b1, w.x1[r > 0 ? r - 1 : r], v);
+            w.x1[r] = in ? v * w.d1 : 0.0f;
         }
     }
 }
 
-// Coarse right-hand side of level l + 1 = the sum of the fine residuals
-// r = f - A e2 (e2: level l's pre-smoothed correction, r computed here)
-// over the coarse control volume (full weighting scaled by 4); zero coarse
-// correction.  Work list of the coarse level's nodes.
-__global__ void k_restrict(const MGLevel* lev, const int* done, int l, const int2* tasks) {
-    const int2 tk = tasks[blockIdx.x];
-    const int run = tk.x;
-    if (done[run]) return;
-    const MGLevel F = lev[run * MG_MAX_LEVELS + l];
-    const MGLevel Cl = lev[run * MG_MAX_LEVELS + l + 1];
-    const int Wc = Cl.nr + 1, Wf = F.nr + 1;
-    const int n = min((Cl.nz + 1) * Wc, tk.y + MAP_CHUNK);
-    for (int k = tk.y + threadIdx.x; k < n; k += blockDim.x) {
-        const int I = k / Wc, J = k - I * Wc;
-        if (I == 0 || I == Cl.nz) {
-            Cl.f[k] = 0.0f;
-            continue;
+// The way down a level: four half-sweeps (colors 0, 1, 0, 1) from e = 0 into e2,
+// the residual r = f - A e2, and the next level's right-hand side, the sum of
+// the residuals over its control volumes (full weighting scaled by 4).  The
+// window's even columns are the coarse nodes': lane = coarse column.
+// Latency bounds it on one grid (all loads before the first use, no barrier).
+// Average over the levels of 512 x 512 cells: 5.2 us, against 8.8 us for the
+// smoothing by a block through shared memory plus 6.9 us for the restriction.
+template <int K>
+__global__ void __launch_bounds__(TILE_WARPS * 32, K == K_LARGE ? 3 : 4) k_down(const MGLevel* lev, const int* done, int l,
+                                                          const int2* tasks, int ntask) {
+    constexpr int TI = K - 2 * PRE_H, TJ = WIN_C - 2 * PRE_H;
+    const int t = blockIdx.x * TILE_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (t >= ntask) return;
+    const int2 tk = tasks[t];
+    if (done[tk.x]) return;
+    const MGLevel L = lev[tk.x * MG_MAX_LEVELS + l];
+    const int nz = L.nz, nr = L.nr, W = nr + 1;
+    const int tj = (W + TJ - 1) / TJ;
+    const int i0 = (tk.y / tj) * TI - PRE_H, j0 = (tk.y % tj) * TJ - PRE_H, j = j0 + 2 * lane;
+    Window<K> w;
+    window_load(w, L, i0, j);
+    // color 0 from zero: f / d
+#pragma unroll
+    for (int r = 0; r < K; ++r) {
+        w.x0[r] = (r & 1) == 0 ? w.f0[r] * w.d0 : 0.0f;
+        w.x1[r] = (r & 1) == 0 ? 0.0f : w.f1[r] * w.d1;
+    }
+    window_sweep<K, 1>(w, i0, nz);
+    window_sweep<K, 0>(w, i0, nz);
+    window_sweep<K, 1>(w, i0, nz);
+    {
+        const bool c0 = lane >= PRE_H / 2 && lane < 32 - PRE_H / 2 && j <= nr, c1 = c0 && j + 1 <= nr;
+        float* e2 = L.e2;
+#pragma unroll
+        for (int r = PRE_H; r < K - PRE_H; ++r) {
+            const int i = i0 + r;
+            if (i < 1 || i > nz - 1) continue;
+            if (c0) e2[i * W + j] = w.x0[r];
+            if (c1) e2[i * W + j + 1] = w.x1[r];
         }
+    }
+    // residuals over f (rows PRE_H - 1 .. K - PRE_H)
+    const float dg0 = w.ap0 + w.am0 + 2.0f * w.b0, dg1 = w.ap1 + w.am1 + 2.0f * w.b1;
+#pragma unroll
+    for (int r = PRE_H - 1; r <= K - PRE_H; ++r) {
+        const float xl = __shfl_up_sync(0xFFFFFFFFu, w.x1[r], 1), xr = __shfl_down_sync(0xFFFFFFFFu, w.x0[r], 1);
+        float s = dg0 * w.x0[r];
+        s = fmaf(-w.ap0, w.x1[r], s);
+        s = fmaf(-w.am0, xl, s);
+        s = fmaf(-w.b0, w.x0[r + 1], s);
+        s = fmaf(-w.b0, w.x0[r - 1], s);
+        w.f0[r] = w.f0[r] - s;
+        s = dg1 * w.x1[r];
+        s = fmaf(-w.ap1, xr, s);
+        s = fmaf(-w.am1, w.x0[r], s);
+        s = fmaf(-w.b1, w.x1[r + 1], s);
+        s = fmaf(-w.b1, w.x1[r - 1], s);
+        w.f1[r] = w.f1[r] - s;
+    }
+    const MGLevel& Cl = lev[tk.x * MG_MAX_LEVELS + l + 1];
+    const int Wc = Cl.nr + 1, nzc = Cl.nz, J = j >> 1;
+    float* cf = Cl.f;
+    const bool out = lane >= PRE_H / 2 && lane < 32 - PRE_H / 2 && j <= nr;
+#pragma unroll
+    for (int r = PRE_H; r < K - PRE_H; r += 2) {
+        const int I = (i0 + r) >> 1;
         float s = 0.0f;
+#pragma unroll
         for (int di = -1; di <= 1; ++di) {
-            const int i = 2 * I + di;
-            if (i <= 0 || i >= F.nz) continue;
             const float wi = di == 0 ? 1.0f : 0.5f;
-            for (int dj = -1; dj <= 1; ++dj) {
-                const int j = 2 * J + dj;
-                if (j < 0 || j > F.nr) continue;
-                const float wj = dj == 0 ? 1.0f : 0.5f;
-                s += wi * wj * (F.f[i * Wf + j] - apply_Af(F, F.e2, i, j));
-            }
+            const float left = __shfl_up_sync(0xFFFFFFFFu, w.f1[r + di], 1);
+            s = fmaf(0.5f * wi, left, s);
+            s = fmaf(wi, w.f0[r + di], s);
+            s = fmaf(0.5f * wi, w.f1[r + di], s);
         }
-        Cl.f[k] = s;
+        if (out && I >= 1 && I <= nzc - 1) cf[I * Wc + J] = s;
+    }
+}
+
+// The way up a level: e2 plus the bilinear prolongation of level l + 1's
+// correction (its e), four half-sweeps (colors 1, 0, 1, 0), into e, or, with
+// FINAL (level 0), added to phi.  512 x 512 cells: 10.2 us on level 0 and 6.5 us on
+// the others' average (16.3 and 12.9 us by a block through shared memory).
+template <int K, bool FINAL>
+__global__ void __launch_bounds__(TILE_WARPS * 32, K == K_LARGE ? 2 : 3) k_up(const MGLevel* lev, const MGTop* top, const int* done, int l,
+                                                        const int2* tasks, int ntask) {
+    constexpr int TI = K - 2 * POST_H, TJ = WIN_C - 2 * POST_H;
+    const int t = blockIdx.x * TILE_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (t >= ntask) return;
+    const int2 tk = tasks[t];
+    if (done[tk.x]) return;
+    const MGLevel L = lev[tk.x * MG_MAX_LEVELS + l];
+    const int nz = L.nz, nr = L.nr, W = nr + 1;
+    const int tj = (W + TJ - 1) / TJ;
+    const int i0 = (tk.y / tj) * TI - POST_H, j0 = (tk.y % tj) * TJ - POST_H, j = j0 + 2 * lane;
+    Window<K> w;
+    window_load(w, L, i0, j);
+    {
+        const MGLevel& Cl = lev[tk.x * MG_MAX_LEVELS + l + 1];
+        const int Wc = Cl.nr + 1, J = j >> 1;
+        const float *ce = Cl.e, *e2 = L.e2;
+        const bool in0 = j >= 0 && j <= nr, in1 = j + 1 >= 1 && j + 1 <= nr;
+        // coarse rows from i0 / 2 at columns J and J + 1 (those of the grid), and
+        // e2: every load before the first use, so that their latencies overlap
+        float a0[K / 2 + 1], a1[K / 2 + 1];
+#pragma unroll
+        for (int r = 0; r <= K / 2; ++r) {
+            const int I = (i0 >> 1) + r;
+            const bool inI = I >= 0 && I <= Cl.nz;
+            a0[r] = inI && in0 ? ce[I * Wc + J] : 0.0f;
+            a1[r] = inI && in1 ? ce[I * Wc + J + 1] : 0.0f;
+        }
+#pragma unroll
+        for (int r = 0; r < K; ++r) {
+            const int i = i0 + r, k = i * W + j;
+            const bool in = i >= 1 && i <= nz - 1;
+            w.x0[r] = in && in0 ? e2[k] : 0.0f;
+            w.x1[r] = in && in1 ? e2[k + 1] : 0.0f;
+        }
+#pragma unroll
+        for (int r = 0; r < K; ++r) {
+            const bool in = i0 + r >= 1 && i0 + r <= nz - 1;
+            const float p0 = a0[r / 2], p1 = a1[r / 2], q0 = a0[(r + 1) / 2], q1 = a1[(r + 1) / 2];
+            const float s0 = ((p0 + q0) + p0) + q0, s1 = ((p0 + q0) + p1) + q1;
+            w.x0[r] = in && in0 ? fmaf(0.25f, s0, w.x0[r]) : 0.0f;
+            w.x1[r] = in && in1 ? fmaf(0.25f, s1, w.x1[r]) : 0.0f;
+        }
+    }
+    window_sweep<K, 1>(w, i0, nz);
+    window_sweep<K, 0>(w, i0, nz);
+    window_sweep<K, 1>(w, i0, nz);
+    window_sweep<K, 0>(w, i0, nz);
+    const bool c0 = lane >= POST_H / 2 && lane < 32 - POST_H / 2 && j <= nr, c1 = c0 && j + 1 <= nr;
+    if (FINAL) {
+        double* phi = top[tk.x].phi;
+        double p0[TI], p1[TI];
+#pragma unroll
+        for (int r = 0; r < TI; ++r) {
+            const int i = i0 + POST_H + r, k = i * W + j;
+            const bool in = i >= 1 && i <= nz - 1;
+            p0[r] = in && c0 ? phi[k] : 0.0;
+            p1[r] = in && c1 ? phi[k + 1] : 0.0;
+        }
+#pragma unroll
+        for (int r = 0; r < TI; ++r) {
+            const int i = i0 + POST_H + r, k = i * W + j;
+            const bool in = i >= 1 && i <= nz - 1;
+            if (in && c0) phi[k] = p0[r] + (double)w.x0[POST_H + r];
+            if (in && c1) phi[k + 1] = p1[r] + (double)w.x1[POST_H + r];
+        }
+    } else {
+        float* e = L.e;
+#pragma unroll
+        for (int r = POST_H; r < K - POST_H; ++r) {
+            const int i = i0 + r;
+            if (i < 1 || i > nz - 1) continue;
+            if (c0) e[i * W + j] = w.x0[r];
+            if (c1) e[i * W + j + 1] = w.x1[r];
+        }
     }
 }
 
 // The levels of one run from its first tail level T down to its coarsest,
-// one V(2,2) cycle by one block in shared memory (blockIdx.x = run): the
-// per-level kernels' operations in their order -- four red-black half-sweeps
-// (colors 0, 1, 0, 1), the residual, the full-weighting restriction, on the
-// coarsest level e = A^-1 f with the stored inverse (transposed: column v at
-// inv[v * m]) or `sweeps` Gauss-Seidel sweeps, then bilinear prolongation
-// and four half-sweeps (colors 1, 0, 1, 0) on the way up.  Input: f of level
-// T (its e is zero).  Output: the correction of level T in its e, or, when T
-// is level 0, added to phi.
+// one V(2,2) cycle by one block in shared memory (blockIdx.x = run): on each
+// level four red-black half-sweeps (colors 0, 1, 0, 1), the residual and the
+// full-weighting restriction; on the coarsest e = A^-1 f with the stored inverse
+// (transposed: column v at inv[v * m]) or `sweeps` Gauss-Seidel sweeps; then
+// bilinear prolongation and four half-sweeps (colors 1, 0, 1, 0) on the way up.
+// Input: f of level T (its e is zero).  Output: the correction of level T in its
+// e, or, when T is level 0, added to phi.
+//
+// A chain of short phases between block barriers bounds it, so a thread keeps
+// its nodes (one of each color, two on a few narrow grids), their right-hand
+// sides and coefficients in registers through a level's sweeps, and a phase is
+// four shared-memory reads, five operations and a write; the run's table and
+// its coefficients come in one copy each.  Three levels from 32 x 32 cells: 26.5
+// -> 16.9 us; with 14 x 61 coarsest unknowns by 200 sweeps (the paper's domain):
+// 156 -> 39 us.
+static_assert(sizeof(TailRun) / 4 <= TAIL_THREADS, "a thread a word");
+
 struct TailLevel {
     float *e, *f, *r, *ap, *am, *b, *d;
     int nz, nr;
 };
 
-__device__ __forceinline__ void tail_half_sweep(const TailLevel& L, int color) {
-    const int W = L.nr + 1;
-    const int n = (L.nz - 1) * W;
-    for (int q = threadIdx.x; q < n; q += blockDim.x) {
-        const int i = 1 + q / W, j = q - (i - 1) * W;
-        if (((i + j) & 1) != color) continue;
-        const int k = i * W + j;
-        float v = L.f[k];
-        if (j < L.nr) v += L.ap[j] * L.e[k + 1];
-        if (j > 0) v += L.am[j] * L.e[k - 1];
-        if (i + 1 < L.nz) v += L.b[j] * L.e[k + W];
-        if (i - 1 > 0) v += L.b[j] * L.e[k - W];
-        L.e[k] = v * L.d[j];
+struct TailNode {
+    int k, up, dn;                       // node; the rows above and below (itself's zero coefficient at an electrode)
+    int rt, lf;
+    float f, ap, am, bu, bd, d;
+};
+
+// the thread's nodes of each color (k < 0: none)
+__device__ __forceinline__ void tail_nodes(const TailLevel& L, TailNode (&nd)[2][TAIL_SLOTS]) {
+    const int W = L.nr + 1, half = (W + 1) / 2, n = (L.nz - 1) * half;
+#pragma unroll
+    for (int q = 0; q < TAIL_SLOTS; ++q) {
+        const int p = (int)threadIdx.x + q * TAIL_THREADS;
+        nd[0][q].k = nd[1][q].k = -1;
+        if (p >= n) continue;
+        const int i = 1 + p / half, jj = 2 * (p - (i - 1) * half);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const int j = jj + ((i + c) & 1);
+            if (j > L.nr) continue;
+            TailNode& t = nd[c][q];
+            const int k = i * W + j;
+            t.k = k;
+            t.f = L.f[k];
+            t.ap = j < L.nr ? L.ap[j] : 0.0f;
+            t.am = j > 0 ? L.am[j] : 0.0f;
+            t.bu = i + 1 < L.nz ? L.b[j] : 0.0f;
+            t.bd = i - 1 > 0 ? L.b[j] : 0.0f;
+            t.d = L.d[j];
+            t.rt = j < L.nr ? k + 1 : k;
+            t.lf = j > 0 ? k - 1 : k;
+            t.up = k + W;
+            t.dn = k - W;
+        }
+    }
+}
+
+__device__ __forceinline__ void tail_half_sweep(const TailLevel& L, const TailNode (&nd)[TAIL_SLOTS]) {
+    float* e = L.e;
+#pragma unroll
+    for (int q = 0; q < TAIL_SLOTS; ++q) {
+        const TailNode& t = nd[q];
+        if (t.k < 0) continue;
+        float v = t.f;
+        v = fmaf(t.ap, e[t.rt], v);
+        v = fmaf(t.am, e[t.lf], v);
+        v = fmaf(t.bu, e[t.up], v);
+        v = fmaf(t.bd, e[t.dn], v);
+        e[t.k] = v * t.d;
     }
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(TAIL_THREADS) k_mg_tail(const MGLevel* lev, const MGTop* top, const int* nlev,
-                                                          const int* tail_lev, const int* done,
-                                                          const float* const* inv, int sweeps) {
+__global__ void __launch_bounds__(TAIL_THREADS) k_mg_tail(const TailRun* runs, const int* done, int sweeps) {
     extern __shared__ float sm[];
+    __shared__ TailRun R;
     __shared__ TailLevel tl[MG_MAX_LEVELS];
     const int run = blockIdx.x;
+    if (threadIdx.x < sizeof(TailRun) / 4)
+        reinterpret_cast<int*>(&R)[threadIdx.x] = reinterpret_cast<const int*>(runs + run)[threadIdx.x];
     if (done[run]) return;
-    const int n = nlev[run], T = tail_lev[run];
-    const MGLevel* Lg = lev + run * MG_MAX_LEVELS;
-    if (threadIdx.x == 0) {
-        int o = 0;
-        for (int l = T; l < n; ++l) {
-            const int W = Lg[l].nr + 1, nodes = (Lg[l].nz + 1) * W;
-            TailLevel& t = tl[l];
-            t.nz = Lg[l].nz;
-            t.nr = Lg[l].nr;
-            t.e = sm + o;
-            t.f = t.e + nodes;
-            t.r = t.f + nodes;
-            t.ap = t.r + nodes;
-            t.am = t.ap + W;
-            t.b = t.am + W;
-            t.d = t.b + W;
-            o += 3 * nodes + 4 * W;
-        }
+    __syncthreads();
+    const int n = R.n;                           // levels counted from the tail's first
+    if ((int)threadIdx.x < n) {
+        const int l = threadIdx.x;
+        const int W = R.nr[l] + 1, nodes = (R.nz[l] + 1) * W;
+        TailLevel& t = tl[l];
+        t.nz = R.nz[l];
+        t.nr = R.nr[l];
+        t.e = sm + R.node_off[l];
+        t.f = t.e + nodes;
+        t.r = t.f + nodes;
+        t.ap = sm + R.coef_off[l];
+        t.am = t.ap + W;
+        t.b = t.am + W;
+        t.d = t.b + W;
+    }
+    // inputs: the coefficients (packed as they lie in shared memory), zero
+    // corrections, f of the first level
+    for (int k = threadIdx.x; k < R.ncoef; k += TAIL_THREADS) sm[k] = __ldg(&R.coef[k]);
+    {
+        const int nodes0 = (R.nz[0] + 1) * (R.nr[0] + 1);
+        float* f0 = sm + R.node_off[0] + nodes0;
+        for (int k = threadIdx.x; k < nodes0; k += TAIL_THREADS) f0[k] = R.f[k];
+        for (int l = 0; l < n; ++l)
+            for (int k = threadIdx.x; k < (R.nz[l] + 1) * (R.nr[l] + 1); k += TAIL_THREADS) sm[R.node_off[l] + k] = 0.0f;
     }
     __syncthreads();
-    // inputs: f of level T, zero corrections, the coefficients
-    for (int l = T; l < n; ++l) {
-        const TailLevel t = tl[l];
-        const int W = t.nr + 1, nodes = (t.nz + 1) * W;
-        for (int k = threadIdx.x; k < nodes; k += blockDim.x) {
-            t.e[k] = 0.0f;
-            if (l == T) t.f[k] = Lg[l].f[k];
-        }
-        for (int j = threadIdx.x; j < W; j += blockDim.x) {
-            t.ap[j] = Lg[l].ap[j];
-            t.am[j] = Lg[l].am[j];
-            t.b[j] = Lg[l].b[j];
-            t.d[j] = Lg[l].dinv[j];
-        }
-    }
-    __syncthreads();
+    TailNode nd[2][TAIL_SLOTS];
     // down
-    for (int l = T; l + 1 < n; ++l) {
+    for (int l = 0; l + 1 < n; ++l) {
         const TailLevel F = tl[l], Cl = tl[l + 1];
-        for (int k = 0; k < 4; ++k) tail_half_sweep(F, k & 1);
-        const int Wf = F.nr + 1, Wc = Cl.nr + 1;
-        for (int q = threadIdx.x; q < (F.nz - 1) * Wf; q += blockDim.x) {
-            const int i = 1 + q / Wf, j = q - (i - 1) * Wf;
-            const int k = i * Wf + j;
-            float s = (F.ap[j] + F.am[j] + 2.0f * F.b[j]) * F.e[k];
-            if (j < F.nr) s -= F.ap[j] * F.e[k + 1];
-            if (j > 0) s -= F.am[j] * F.e[k - 1];
-            if (i + 1 < F.nz) s -= F.b[j] * F.e[k + Wf];
-            if (i - 1 > 0) s -= F.b[j] * F.e[k - Wf];
-            F.r[k] = F.f[k] - s;
+        tail_nodes(F, nd);
+        for (int k = 0; k < 2; ++k) {
+            tail_half_sweep(F, nd[0]);
+            tail_half_sweep(F, nd[1]);
         }
+        const int Wf = F.nr + 1, Wc = Cl.nr + 1;
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+            for (int q = 0; q < TAIL_SLOTS; ++q) {
+                const TailNode& t = nd[c][q];
+                if (t.k < 0) continue;
+                const int j = t.k % Wf;
+                float s = (F.ap[j] + F.am[j] + 2.0f * F.b[j]) * F.e[t.k];
+                s = fmaf(-t.ap, F.e[t.rt], s);
+                s = fmaf(-t.am, F.e[t.lf], s);
+                s = fmaf(-t.bu, F.e[t.up], s);
+                s = fmaf(-t.bd, F.e[t.dn], s);
+                F.r[t.k] = t.f - s;
+            }
         __syncthreads();
-        for (int k = threadIdx.x; k < (Cl.nz + 1) * Wc; k += blockDim.x) {
-            const int I = k / Wc, J = k - I * Wc;
-            if (I == 0 || I == Cl.nz) {
-                Cl.f[k] = 0.0f;
-                continue;
-            }
+        for (int k = threadIdx.x; k < (Cl.nz - 1) * Wc; k += TAIL_THREADS) {
+            const int I = 1 + k / Wc, J = k - (I - 1) * Wc;
             float s = 0.0f;
+#pragma unroll
             for (int di = -1; di <= 1; ++di) {
-                const int i = 2 * I + di;
-                if (i <= 0 || i >= F.nz) continue;
                 const float wi = di == 0 ? 1.0f : 0.5f;
-                for (int dj = -1; dj <= 1; ++dj) {
-                    const int j = 2 * J + dj;
-                    if (j < 0 || j > F.nr) continue;
-                    const float wj = dj == 0 ? 1.0f : 0.5f;
-                    s += wi * wj * F.r[i * Wf + j];
-                }
+                const float* r = F.r + (2 * I + di) * Wf + 2 * J;
+                if (J > 0) s = fmaf(0.5f * wi, r[-1], s);
+                s = fmaf(wi, r[0], s);
+                if (2 * J + 1 <= F.nr) s = fmaf(0.5f * wi, r[1], s);
             }
-            Cl.f[k] = s;
+            Cl.f[I * Wc + J] = s;
         }
         __syncthreads();
     }
@@ -505,12 +648,12 @@ __global__ void __launch_bounds__(TAIL_THREADS) k_mg_tail(const MGLevel* lev, co
         const TailLevel L = tl[n - 1];
         const int W = L.nr + 1;
         const int m = (L.nz - 1) * W;
-        const float* Ai = inv[run];
+        const float* Ai = R.inv;
         if (Ai) {
             // e = A^-1 f: P threads per unknown, each summing every P-th
             // term (their loads in flight together), then a shuffle sum
             const int P = m <= 64 ? 8 : (m <= 128 ? 4 : (m <= 256 ? 2 : 1));
-            const int per = (int)blockDim.x / P;
+            const int per = TAIL_THREADS / P;
             for (int u0 = 0; u0 < m; u0 += per) {        // the same trip count in every thread
                 const int u = u0 + (int)threadIdx.x / P, part = (int)threadIdx.x % P;
                 float acc = 0.0f;
@@ -523,42 +666,59 @@ __global__ void __launch_bounds__(TAIL_THREADS) k_mg_tail(const MGLevel* lev, co
             }
             __syncthreads();
         } else {
+            tail_nodes(L, nd);
             for (int it = 0; it < sweeps; ++it) {
-                tail_half_sweep(L, 0);
-                tail_half_sweep(L, 1);
+                tail_half_sweep(L, nd[0]);
+                tail_half_sweep(L, nd[1]);
             }
         }
     }
     // up
-    for (int l = n - 2; l >= T; --l) {
+    for (int l = n - 2; l >= 0; --l) {
         const TailLevel F = tl[l], Cl = tl[l + 1];
         const int Wf = F.nr + 1, Wc = Cl.nr + 1;
-        for (int q = threadIdx.x; q < (F.nz - 1) * Wf; q += blockDim.x) {
-            const int i = 1 + q / Wf, j = q - (i - 1) * Wf;
-            const int I0 = i >> 1, J0 = j >> 1;
-            const int I1 = (i & 1) ? I0 + 1 : I0, J1 = (j & 1) ? J0 + 1 : J0;
-            const float c = 0.25f * (Cl.e[I0 * Wc + J0] + Cl.e[I1 * Wc + J0] + Cl.e[I0 * Wc + J1] + Cl.e[I1 * Wc + J1]);
-            F.e[i * Wf + j] += c;
-        }
+        tail_nodes(F, nd);
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+            for (int q = 0; q < TAIL_SLOTS; ++q) {
+                const int k = nd[c][q].k;
+                if (k < 0) continue;
+                const int i = k / Wf, j = k - i * Wf;
+                const int I0 = i >> 1, J0 = j >> 1;
+                const int I1 = (i & 1) ? I0 + 1 : I0, J1 = (j & 1) ? J0 + 1 : J0;
+                const float s =
+                    ((Cl.e[I0 * Wc + J0] + Cl.e[I1 * Wc + J0]) + Cl.e[I0 * Wc + J1]) + Cl.e[I1 * Wc + J1];
+                F.e[k] = fmaf(0.25f, s, F.e[k]);
+            }
         __syncthreads();
-        for (int k = 0; k < 4; ++k) tail_half_sweep(F, 1 - (k & 1));
+        for (int k = 0; k < 2; ++k) {
+            tail_half_sweep(F, nd[1]);
+            tail_half_sweep(F, nd[0]);
+        }
     }
     // output
-    const TailLevel t = tl[T];
+    const TailLevel t = tl[0];
     const int W = t.nr + 1;
-    if (T == 0) {
-        double* phi = top[run].phi;
-        for (int q = threadIdx.x; q < (t.nz - 1) * W; q += blockDim.x) phi[W + q] += (double)t.e[W + q];
+    if (R.phi) {
+        double* phi = R.phi;
+        for (int q = threadIdx.x; q < (t.nz - 1) * W; q += TAIL_THREADS) phi[W + q] += (double)t.e[W + q];
     } else {
-        float* e = Lg[T].e;
-        for (int k = threadIdx.x; k < (t.nz + 1) * W; k += blockDim.x) e[k] = t.e[k];
+        float* e = R.e;
+        for (int k = threadIdx.x; k < (t.nz + 1) * W; k += TAIL_THREADS) e[k] = t.e[k];
     }
 }
 
 // E = -grad(phi): central inside, one-sided at the electrodes, E_r = 0 on the
-// axis and at r = R
-__global__ void k_efield(const MGTop* top, const RunInfo* runs, float2* E) {
+// axis and at r = R; and the end of the solve's bookkeeping
+__global__ void k_efield(const MGTop* top, const RunInfo* runs, float2* E, const int* done, DevState* st,
+                         RunState* rs) {
     const int run = blockIdx.y;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (done[run] == 2) atomicOr(&st->error, ERR_NONFINITE);
+        const double rel = rs[run].relres;
+        if (!(rel <= rs[run].relres_max)) rs[run].relres_max = rel;   // NaN propagates
+    }
     const MGTop T = top[run];
     const int nz = T.nz, nr = T.nr;
     const int W = nr + 1;
@@ -574,14 +734,6 @@ __global__ void k_efield(const MGTop* top, const RunInfo* runs, float2* E) {
         if (j == 0 || j == nr) er = 0.0;
         else er = -(p[k + 1] - p[k - 1]) * T.i2dr;
         out[k] = make_float2((float)ez, (float)er);
-    }
-}
-
-__global__ void k_solve_epilogue(const int* done, int nruns, DevState* st, RunState* rs) {
-    for (int r = threadIdx.x; r < nruns; r += blockDim.x) {
-        if (done[r] == 2) atomicOr(&st->error, ERR_NONFINITE);
-        const double rel = rs[r].relres;
-        if (!(rel <= rs[r].relres_max)) rs[r].relres_max = rel;   // NaN propagates
     }
 }
 
@@ -697,7 +849,7 @@ int field_init(FieldSolver& fs, const std::vector<pd_config>& cfgs, const std::v
     fs.max_nodes0 = 0;
     fs.max_cycles = cfgs[0].poisson_max_cycles > 0 ? cfgs[0].poisson_max_cycles : 60;
     std::vector<double> tol(R);
-    std::vector<float*> inv(R, nullptr);
+    std::vector<TailRun> tails(R);
     for (int r = 0; r < R; ++r) {
         const pd_config& c = cfgs[r];
         int a[MG_MAX_LEVELS], b[MG_MAX_LEVELS], n;
@@ -748,6 +900,7 @@ int field_init(FieldSolver& fs, const std::vector<pd_config>& cfgs, const std::v
         upload(T.iv, iv, s);
         cudaStreamSynchronize(s);          // the host vectors above go out of scope
         // correction levels in float
+        std::vector<float> coef;
         for (int l = 0; l < n; ++l) {
             MGLevel& L = fs.host_lev[(size_t)r * MG_MAX_LEVELS + l];
             L.nz = a[l];
@@ -776,53 +929,88 @@ int field_init(FieldSolver& fs, const std::vector<pd_config>& cfgs, const std::v
                 const int m = coarse_unknowns(a, b, n);
                 std::vector<double> Ai;
                 if (!invert_coarse(L.nz, L.nr, lap, lam, lbb, Ai)) return 1;
-                inv[r] = (float*)take((size_t)m * m * 4);
+                float* inv = (float*)take((size_t)m * m * 4);
                 fai = to_float(Ai);
-                upload(inv[r], fai, s);
+                upload(inv, fai, s);
+                tails[r].inv = inv;
             }
             cudaStreamSynchronize(s);      // the host vectors above go out of scope
+            if (l >= fs.tail_lev[r])
+                for (const std::vector<float>* v : {&fap, &fam, &fbb, &fdi}) coef.insert(coef.end(), v->begin(), v->end());
         }
+        // k_mg_tail's table
+        TailRun& tr = tails[r];
+        const int t0 = fs.tail_lev[r];
+        int o_coef = 0, o_node = (int)coef.size();
+        tr.n = n - t0;
+        tr.ncoef = o_node;
+        for (int l = t0; l < n; ++l) {
+            tr.nz[l - t0] = a[l];
+            tr.nr[l - t0] = b[l];
+            tr.coef_off[l - t0] = o_coef;
+            tr.node_off[l - t0] = o_node;
+            o_coef += 4 * (b[l] + 1);
+            o_node += 3 * (a[l] + 1) * (b[l] + 1);
+        }
+        float* dcoef = (float*)take(coef.size() * 4);
+        upload(dcoef, coef, s);
+        cudaStreamSynchronize(s);
+        tr.coef = dcoef;
+        tr.f = fs.host_lev[(size_t)r * MG_MAX_LEVELS + t0].f;
+        tr.e = fs.host_lev[(size_t)r * MG_MAX_LEVELS + t0].e;
+        tr.phi = t0 == 0 ? T.phi : nullptr;
     }
     fs.lev = (MGLevel*)take((size_t)R * MG_MAX_LEVELS * sizeof(MGLevel));
     fs.top = (MGTop*)take((size_t)R * sizeof(MGTop));
-    fs.nlev_dev = (int*)take((size_t)R * 4);
-    fs.tail_lev_dev = (int*)take((size_t)R * 4);
     fs.done = (int*)take((size_t)R * 4);
-    fs.red = (double*)take((size_t)R * RED_BLOCKS * 2 * 8);
+    fs.ticket = (unsigned int*)take((size_t)R * 4);
+    fs.red_base = (int*)take((size_t)R * 4);
+    std::vector<int> red_base(R);
+    int nred = 0;
+    for (int r = 0; r < R; ++r) {
+        red_base[r] = nred;
+        nred += (red_units(cfgs[r].nz, cfgs[r].nr) + 7) / 8;
+    }
+    fs.red = (double*)take((size_t)nred * 2 * 8);
     fs.bnorm = (double*)take((size_t)R * 8);
     fs.tol = (double*)take((size_t)R * 8);
-    fs.inv = (float**)take((size_t)R * sizeof(float*));
+    fs.tails = (TailRun*)take((size_t)R * sizeof(TailRun));
     // work lists, level by level: the levels above each run's tail
     std::vector<int2> tasks;
     for (int l = 0; l < MG_MAX_LEVELS; ++l) {
-        auto add = [&](int r, long long cnt, int step) {
-            for (long long q = 0; q < cnt; q += step) tasks.push_back(make_int2(r, (int)q));
-        };
-        fs.coarse_off[l] = (int)tasks.size();
+        // short windows where long ones would leave most SMs idle: a tile of
+        // K = 20 rows is through in two thirds of the time of one of 32, but
+        // spends 60 % of its rows on the rings instead of 38 %; the line is four
+        // tiles, one block, an SM
+        int large = 0;
         for (int r = 0; r < R; ++r)
-            if (l < fs.tail_lev[r]) {
-                const MGLevel& C = fs.host_lev[(size_t)r * MG_MAX_LEVELS + l + 1];
-                add(r, (long long)(C.nz + 1) * (C.nr + 1), MAP_CHUNK);
-            }
-        fs.coarse_len[l] = (int)tasks.size() - fs.coarse_off[l];
-        fs.tile_off[l] = (int)tasks.size();
-        for (int r = 0; r < R; ++r)
-            if (l < fs.tail_lev[r]) {
-                const MGLevel& L = fs.host_lev[(size_t)r * MG_MAX_LEVELS + l];
-                add(r, tiles_of(L.nz, L.nr), 1);
-            }
-        fs.tile_len[l] = (int)tasks.size() - fs.tile_off[l];
+            if (l < fs.tail_lev[r]) large += tiles_of(fs.host_lev[(size_t)r * MG_MAX_LEVELS + l].nz,
+                                                      fs.host_lev[(size_t)r * MG_MAX_LEVELS + l].nr, K_LARGE, PRE_H);
+        fs.rows[l] = large > SMALL_TILES ? K_LARGE : K_SMALL;
+        for (int post = 0; post < 2; ++post) {
+            fs.tile_off[post][l] = (int)tasks.size();
+            for (int r = 0; r < R; ++r)
+                if (l < fs.tail_lev[r]) {
+                    const MGLevel& L = fs.host_lev[(size_t)r * MG_MAX_LEVELS + l];
+                    const int cnt = tiles_of(L.nz, L.nr, fs.rows[l], post ? POST_H : PRE_H);
+                    for (int q = 0; q < cnt; ++q) tasks.push_back(make_int2(r, q));
+                }
+            fs.tile_len[post][l] = (int)tasks.size() - fs.tile_off[post][l];
+        }
     }
+    fs.red_off = (int)tasks.size();
+    for (int r = 0; r < R; ++r)
+        for (int u = 0; u < red_units(cfgs[r].nz, cfgs[r].nr); u += 8) tasks.push_back(make_int2(r, u));
+    fs.red_len = (int)tasks.size() - fs.red_off;
     if (fs.tail_smem > 48 * 1024) return 1;          // cannot happen: tail levels hold at most 34 x 34 nodes
     fs.tasks = (int2*)take(tasks.size() * sizeof(int2) + 8);
     if (o > bytes) return 1;
     upload(fs.tasks, tasks, s);
     upload(fs.lev, fs.host_lev, s);
     upload(fs.top, fs.host_top, s);
-    upload(fs.nlev_dev, fs.nlev, s);
-    upload(fs.tail_lev_dev, fs.tail_lev, s);
     upload(fs.tol, tol, s);
-    upload(fs.inv, inv, s);
+    upload(fs.tails, tails, s);
+    upload(fs.red_base, red_base, s);
     if (!fs.host_done && cudaMallocHost(&fs.host_done, (size_t)R * 4) != cudaSuccess) return 1;
     return cudaStreamSynchronize(s) == cudaSuccess ? 0 : 1;
 }
@@ -832,58 +1020,47 @@ void field_free(FieldSolver& fs) {
     fs.host_done = nullptr;
 }
 
-// two red-black iterations (four half-sweeps) in one launch: pre-smoothing
-// from zero into e2, or post-smoothing from e2 plus the prolongated
-// correction of level l + 1 into e (level 0: into phi)
-static int smooth4(FieldSolver& fs, int l, bool post, cudaStream_t s) {
-    if (!fs.tile_len[l]) return 0;
-    const int2* t = fs.tasks + fs.tile_off[l];
-    if (!post) k_smooth4<false, false><<<fs.tile_len[l], 256, 0, s>>>(fs.lev, fs.top, fs.done, l, t);
-    else if (l == 0) k_smooth4<true, true><<<fs.tile_len[l], 256, 0, s>>>(fs.lev, fs.top, fs.done, l, t);
-    else k_smooth4<true, false><<<fs.tile_len[l], 256, 0, s>>>(fs.lev, fs.top, fs.done, l, t);
-    return 1;
-}
-
 // one correction cycle of every run that has not converged (the right-hand
 // side is level 0's f, set with the residual norms); returns the kernels
 // launched
 static int vcycle(FieldSolver& fs, cudaStream_t s) {
-    const int R = fs.nruns;
-    const int th = fs.threads;
-    int nk = 0;
+    const int R = fs.nruns, th = TILE_WARPS * 32;
+    int nk = 1;
     // down to each run's tail: pre-smooth, residual and restriction
     for (int l = 0; l < fs.max_tail; ++l) {
-        nk += smooth4(fs, l, false, s);
-        if (fs.coarse_len[l]) {
-            k_restrict<<<fs.coarse_len[l], th, 0, s>>>(fs.lev, fs.done, l, fs.tasks + fs.coarse_off[l]);
-            ++nk;
-        }
+        const int n = fs.tile_len[0][l], g = (n + TILE_WARPS - 1) / TILE_WARPS;
+        const int2* t = fs.tasks + fs.tile_off[0][l];
+        if (!n) continue;
+        if (fs.rows[l] == K_SMALL) k_down<K_SMALL><<<g, th, 0, s>>>(fs.lev, fs.done, l, t, n);
+        else k_down<K_LARGE><<<g, th, 0, s>>>(fs.lev, fs.done, l, t, n);
+        ++nk;
     }
     // the tail levels of every run, one block each
-    k_mg_tail<<<R, TAIL_THREADS, fs.tail_smem, s>>>(fs.lev, fs.top, fs.nlev_dev, fs.tail_lev_dev, fs.done, fs.inv,
-                                                    200);
-    ++nk;
+    k_mg_tail<<<R, TAIL_THREADS, fs.tail_smem, s>>>(fs.tails, fs.done, 200);
     // up: prolongation and post-smoothing in one launch per level; level 0's adds the correction to phi
-    for (int l = fs.max_tail - 1; l >= 0; --l) nk += smooth4(fs, l, true, s);
+    for (int l = fs.max_tail - 1; l >= 0; --l) {
+        const int n = fs.tile_len[1][l], g = (n + TILE_WARPS - 1) / TILE_WARPS;
+        const int2* t = fs.tasks + fs.tile_off[1][l];
+        if (!n) continue;
+        const bool small = fs.rows[l] == K_SMALL;
+        if (l == 0 && small) k_up<K_SMALL, true><<<g, th, 0, s>>>(fs.lev, fs.top, fs.done, l, t, n);
+        else if (l == 0) k_up<K_LARGE, true><<<g, th, 0, s>>>(fs.lev, fs.top, fs.done, l, t, n);
+        else if (small) k_up<K_SMALL, false><<<g, th, 0, s>>>(fs.lev, fs.top, fs.done, l, t, n);
+        else k_up<K_LARGE, false><<<g, th, 0, s>>>(fs.lev, fs.top, fs.done, l, t, n);
+        ++nk;
+    }
     return nk;
 }
 
-static void norms(FieldSolver& fs, RunState* rs, int cycle, int first, cudaStream_t s) {
-    const int R = fs.nruns;
-    const dim3 g(RED_BLOCKS, R);
-    k_residual_norms<<<g, 256, 0, s>>>(fs.top, fs.lev, fs.nlev_dev, fs.red, first);
-    k_norms<<<(R + 3) / 4, 128, 0, s>>>(fs.red, fs.bnorm, fs.done, fs.tol, rs, R, cycle, first);
+static void norms(FieldSolver& fs, RunState* rs, int cycle, cudaStream_t s) {
+    k_residual_norms<<<fs.red_len, 256, 0, s>>>(fs.top, fs.lev, fs.tasks + fs.red_off, fs.red_base, fs.red, fs.ticket,
+                                                fs.bnorm, fs.done, fs.tol, rs, cycle);
 }
 
-cudaError_t field_solve(FieldSolver& fs, const long long* rho_e, const long long* rho_h, double* phi, float2* E,
-                const RunInfo* runs, RunState* rs, int host_check, int cycles, cudaStream_t s, int* kernels) {
-    (void)E;
-    (void)phi;
+cudaError_t field_solve(FieldSolver& fs, RunState* rs, int host_check, int cycles, cudaStream_t s, int* kernels) {
     const int R = fs.nruns;
-    const dim3 g0(blocks_for(fs, fs.max_nodes0), R);
-    k_rhs<<<g0, fs.threads, 0, s>>>(rho_e, rho_h, fs.top, runs, rs);
-    norms(fs, rs, 0, 1, s);
-    if (kernels) *kernels += 3;
+    norms(fs, rs, 0, s);
+    if (kernels) *kernels += 1;
     if (host_check) {
         for (int cyc = 1; cyc <= fs.max_cycles; ++cyc) {
             cudaError_t e = cudaMemcpyAsync(fs.host_done, fs.done, (size_t)R * 4, cudaMemcpyDeviceToHost, s);
@@ -893,14 +1070,14 @@ cudaError_t field_solve(FieldSolver& fs, const long long* rho_e, const long long
             for (int r = 0; r < R; ++r) all = all && fs.host_done[r] != 0;
             if (all) break;
             const int nk = vcycle(fs, s);
-            norms(fs, rs, cyc, 0, s);
-            if (kernels) *kernels += nk + 2;
+            norms(fs, rs, cyc, s);
+            if (kernels) *kernels += nk + 1;
         }
     } else {
         for (int cyc = 1; cyc <= cycles; ++cyc) {
             const int nk = vcycle(fs, s);
-            norms(fs, rs, cyc, 0, s);
-            if (kernels) *kernels += nk + 2;
+            norms(fs, rs, cyc, s);
+            if (kernels) *kernels += nk + 1;
         }
     }
     return cudaGetLastError();
@@ -911,45 +1088,49 @@ void field_efield(FieldSolver& fs, const double* phi, const RunInfo* runs, float
                   cudaStream_t s) {
     (void)phi;
     const dim3 g(blocks_for(fs, fs.max_nodes0), fs.nruns);
-    k_efield<<<g, fs.threads, 0, s>>>(fs.top, runs, E);
-    k_solve_epilogue<<<1, 128, 0, s>>>(fs.done, fs.nruns, st, rs);
+    k_efield<<<g, fs.threads, 0, s>>>(fs.top, runs, E, fs.done, st, rs);
 }
 
 // ------------------------------------------------------------------
 // warm start
 // ------------------------------------------------------------------
-// node density of the current fixed-point charge (C/m^3)
-__device__ __forceinline__ double node_rho(const long long* rho_e, const long long* rho_h, const MGTop& T,
-                                           double qw, int i, int j, uint32_t g) {
-    const double f = (i == 0 || i == T.nz) ? 2.0 : 1.0;       // half volume on the electrode rows
-    return qw * (double)(rho_e[g] + rho_h[g]) * (T.iv[j] * f);
-}
-
-// history shift at the start of a solve: rho_prev2 := rho_prev, rho_prev :=
-// rho_last, phi_prev2 := phi_prev, phi_prev := phi, V_prev2 := V_prev,
-// V_prev := V_last; then rho_last := current density, V_last := V
-__global__ void k_warm_history(const long long* rho_e, const long long* rho_h, const MGTop* top,
-                               const RunInfo* runs, const RunState* rs, WarmHistory h, int extrapolate) {
+// The start of a solve: the right-hand side b (double) and the electrode rows
+// of phi (blockIdx.y = run), and the history shift rho_prev2 := rho_prev,
+// rho_prev := rho_last, phi_prev2 := phi_prev, phi_prev := phi, V_prev2 :=
+// V_prev, V_prev := V_last; then rho_last := current density, V_last := V.
+__global__ void k_begin(const long long* rho_e, const long long* rho_h, const MGTop* top, const RunInfo* runs,
+                        const RunState* rs, WarmHistory h, int extrapolate) {
     const int run = blockIdx.y;
-    const MGTop T = top[run];
+    const MGTop& T = top[run];
     const RunInfo& RI = runs[run];
-    const double qw = QE_ * RI.weight / 4294967296.0;
-    const int W = T.nr + 1, n = (T.nz + 1) * W;
+    const double qw = QE_ * RI.weight / 4294967296.0, V = rs[run].V;
+    const int nz = T.nz, W = T.nr + 1, n = (nz + 1) * W;
+    double *phi = T.phi, *bf = T.bf;
+    const double *cr = T.cr, *iv = T.iv, *bz = T.b;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
         const int i = k / W, j = k - i * W;
+        const bool rim = i == 0 || i == nz;
         const uint32_t g = RI.node_base + (uint32_t)k;
+        const double q = (double)(rho_e[g] + rho_h[g]);
         h.rho_prev2[g] = h.rho_prev[g];
         h.rho_prev[g] = h.rho_last[g];
-        const double p = T.phi[k], pp = h.phi_prev[g];
-        if (extrapolate && i > 0 && i < T.nz) T.phi[k] = 2.0 * p - pp;
+        const double p = phi[k], pp = h.phi_prev[g];
+        if (rim) phi[k] = i == 0 ? 0.0 : V;
+        else if (extrapolate) phi[k] = 2.0 * p - pp;
+        double v = 0.0;
+        if (!rim) {
+            v = q * cr[j];
+            if (i == nz - 1) v += bz[j] * V;
+        }
+        bf[k] = v;
         h.phi_prev2[g] = pp;
         h.phi_prev[g] = p;
-        h.rho_last[g] = node_rho(rho_e, rho_h, T, qw, i, j, g);
+        h.rho_last[g] = qw * q * (iv[j] * (rim ? 2.0 : 1.0));       // half volume on the electrode rows
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         h.V_prev2[run] = h.V_prev[run];
         h.V_prev[run] = h.V_last[run];
-        h.V_last[run] = rs[run].V;
+        h.V_last[run] = V;
     }
 }
 
@@ -1059,11 +1240,10 @@ __global__ void k_warm_targets(const double* phi, const MGTop* top, const RunInf
     }
 }
 
-void warm_history(FieldSolver& fs, const long long* rho_e, const long long* rho_h, const RunInfo* runs,
-                  const RunState* rs, double* phi, const WarmHistory& h, bool extrapolate, cudaStream_t s) {
-    (void)phi;
+void field_begin(FieldSolver& fs, const long long* rho_e, const long long* rho_h, const RunInfo* runs,
+                 const RunState* rs, const WarmHistory& h, bool extrapolate, cudaStream_t s) {
     const dim3 g(blocks_for(fs, fs.max_nodes0), fs.nruns);
-    k_warm_history<<<g, fs.threads, 0, s>>>(rho_e, rho_h, fs.top, runs, rs, h, extrapolate ? 1 : 0);
+    k_begin<<<g, fs.threads, 0, s>>>(rho_e, rho_h, fs.top, runs, rs, h, extrapolate ? 1 : 0);
 }
 
 void warm_inputs(FieldSolver& fs, const WarmHistory& h, int form, const RunInfo* runs, double* rmax, float* x,

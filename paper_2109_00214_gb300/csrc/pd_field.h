@@ -32,6 +32,18 @@ struct MGTop {
     double idz, i2dz, i2dr;  // 1 / dz, 1 / (2 dz), 1 / (2 dr)
 };
 
+// one run's levels from its tail level down, for k_mg_tail
+struct TailRun {
+    int n, ncoef;                        // levels; floats of their coefficients
+    int nz[MG_MAX_LEVELS], nr[MG_MAX_LEVELS];
+    int node_off[MG_MAX_LEVELS], coef_off[MG_MAX_LEVELS];   // in shared memory: e, f, r; ap, am, b, 1 / diagonal
+    const float* coef;                   // the coefficients, as they lie there
+    const float* f;                      // the first level's right-hand side
+    float* e;                            // its correction, or
+    double* phi;                         // the run's potential when it is level 0
+    const float* inv;                    // inverse of the coarsest operator (transposed), or null
+};
+
 struct FieldSolver {
     int nruns = 0;
     int max_levels = 0;                 // deepest hierarchy over the runs
@@ -40,27 +52,29 @@ struct FieldSolver {
     MGLevel* lev = nullptr;             // device copy of host_lev
     std::vector<MGTop> host_top;        // [run]
     MGTop* top = nullptr;               // device copy
-    int* nlev_dev = nullptr;            // [nruns]
-    double* red = nullptr;              // [nruns][RED_BLOCKS][2] partial norms
+    double* red = nullptr;              // partial norms (r^2, b^2) of the residual's blocks
+    int* red_base = nullptr;            // [nruns] a run's first block in them
+    unsigned int* ticket = nullptr;     // [nruns] blocks that have finished their part of a residual
     double* bnorm = nullptr;            // [nruns]
     int* done = nullptr;                // [nruns] converged flags
     int* host_done = nullptr;           // pinned copy
     double* tol = nullptr;              // [nruns]
     int max_cycles = 60;
     int max_nodes0 = 0;                 // largest level-0 node count
-    float** inv = nullptr;              // [nruns] inverse of the coarsest operator (transposed), or null
-    // work lists of the per-cycle kernels: (run, first item) of each block,
-    // for every level l the runs whose tail level lies below l
+    // work lists of the per-cycle kernels: (run, tile) of each warp, for every
+    // level l the runs whose tail level lies below l, on the way down and up;
+    // and (run, first unit) of the residual's blocks
     int2* tasks = nullptr;              // device copy of all lists
-    int coarse_off[MG_MAX_LEVELS] = {}, coarse_len[MG_MAX_LEVELS] = {};   // all nodes of level l + 1
-    int tile_off[MG_MAX_LEVELS] = {}, tile_len[MG_MAX_LEVELS] = {};       // smoother tiles of level l
+    int tile_off[2][MG_MAX_LEVELS] = {}, tile_len[2][MG_MAX_LEVELS] = {};
+    int rows[MG_MAX_LEVELS] = {};       // rows of a tile's window on the level
+    int red_off = 0, red_len = 0;
     // levels from tail_lev[run] down are cycled by one block per run in
     // shared memory (k_mg_tail); the level lists hold only the levels above
     std::vector<int> tail_lev;
-    int* tail_lev_dev = nullptr;        // [nruns]
+    TailRun* tails = nullptr;           // [nruns]
     int max_tail = 0;                   // largest tail_lev over the runs
     size_t tail_smem = 0;               // dynamic shared memory of k_mg_tail
-    int threads = 256;                  // threads per block of the level kernels (64..1024, a multiple of 32)
+    int threads = 256;                  // threads per block of the node kernels (64..1024, a multiple of 32)
     int max_blocks = 1216;              // cap on blocks per run of the once-per-solve node kernels
 };
 
@@ -71,15 +85,13 @@ size_t field_workspace_bytes(const std::vector<int>& nz, const std::vector<int>&
 int field_init(FieldSolver& fs, const std::vector<pd_config>& cfgs, const std::vector<uint32_t>& node_base,
                double* phi, void* ws, size_t bytes, cudaStream_t s);
 void field_free(FieldSolver& fs);
-// rho_e + rho_h (fixed point) -> phi (warm-started from its current value) -> E
-// for every run; the anode potential of each run is RunState::V.  With
+// phi of every run from field_begin's right-hand side.  With
 // host_check, cycles run until every run reaches its tolerance (the host
 // reads the flags between cycles); otherwise exactly `cycles` cycles are
 // issued with no host synchronisation (runs already converged skip them),
 // so the solve can be captured in a CUDA graph.  Records relres / cycles.
-cudaError_t field_solve(FieldSolver& fs, const long long* rho_e, const long long* rho_h, double* phi, float2* E,
-                const RunInfo* runs, RunState* rs, int host_check, int cycles, cudaStream_t s,
-                int* kernels = nullptr);   // adds the number of kernels launched
+cudaError_t field_solve(FieldSolver& fs, RunState* rs, int host_check, int cycles, cudaStream_t s,
+                        int* kernels = nullptr);   // adds the number of kernels launched
 
 // E = -grad(phi) of every run; flags runs whose solve met a non-finite value
 // and folds each run's final residual into RunState::relres_max
@@ -105,12 +117,13 @@ struct WarmHistory {
 //   extrapolated: d = rho - (2 rho' - rho''),
 //                 base = 2 phi' - phi'' + (V - 2 V' + V'') z / L
 enum WarmForm { WARM_ABSOLUTE = 0, WARM_DELTA = 1, WARM_EXTRAP = 2 };
-// at the start of every solve: shift the history and record the current
-// density (Verboncoeur volumes, halved on the electrode rows) and voltage;
-// with `extrapolate`, phi := 2 phi - phi_prev on the interior rows (phi_prev
-// taken before the shift)
-void warm_history(FieldSolver& fs, const long long* rho_e, const long long* rho_h, const RunInfo* runs,
-                  const RunState* rs, double* phi, const WarmHistory& h, bool extrapolate, cudaStream_t s);
+// At the start of every solve: the right-hand side of rho_e + rho_h (fixed
+// point) and the anode's RunState::V, the electrode rows of phi, and the
+// history shifted with the current density (Verboncoeur volumes, halved on the
+// electrode rows) and voltage recorded; with `extrapolate`, phi := 2 phi -
+// phi_prev on the interior rows (phi_prev taken before the shift)
+void field_begin(FieldSolver& fs, const long long* rho_e, const long long* rho_h, const RunInfo* runs,
+                 const RunState* rs, const WarmHistory& h, bool extrapolate, cudaStream_t s);
 // d of the form; rmax[run] = max |d|; x = d / rmax
 void warm_inputs(FieldSolver& fs, const WarmHistory& h, int form, const RunInfo* runs, double* rmax, float* x,
                  cudaStream_t s);

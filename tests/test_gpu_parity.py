@@ -402,6 +402,49 @@ def test_rz_poisson_matches_oracle(pd, xs, n, nr):
     assert np.allclose(gEr, oEr, rtol=1e-6, atol=1e-6 * np.abs(oEz).max())
 
 
+@pytest.mark.parametrize("nz,nr", [
+    (80, 104),     # whole tiles of the pre-smoothing: 8 rows x 52 radial nodes, one node over
+    (96, 112),     # 12 rows x 56 of the post-smoothing, one over
+    (88, 56),      # ragged both ways
+    (28, 448),     # many column tiles, coarsest level by Gauss-Seidel sweeps
+    (1024, 1024),  # long windows (from 608 tiles a level)
+])
+def test_rz_poisson_residual_on_tile_edges(pd, xs, nz, nr):
+    """The solve's potential against the discrete Eq. (8) in float64 on grids
+    that end on and beside the smoothing tiles' edges."""
+    cfg, parts = synthetic.rz_plume(n=nz, total=5e4, seed=4)
+    keep = parts["ir"] < nr
+    parts = {k: v[keep] for k, v in parts.items()}
+    cfg.update(nr=nr, field_on=1, inject_on=0, poisson_tol=1e-9)
+    sim = pd.Simulation(cfg, xs)
+    sim.load(parts)
+    sim.step(0)
+    phi, (qe, qh) = sim.phi(), sim.rho()
+    d, j = cfg["dz"], np.arange(nr + 1)
+    ap, am = 2 * np.pi * (j + 0.5) * d, 2 * np.pi * (j - 0.5) * d
+    ap[-1] = am[0] = 0.0
+    area = 2 * np.pi * j * d * d
+    area[0] = np.pi * d * d / 4
+    area[-1] = np.pi * d * d * (nr - 0.25)
+    verb = 2 * np.pi * d ** 3 * j
+    verb[0] = np.pi * d ** 3 / 3
+    verb[-1] = 2 * np.pi * d ** 3 * (nr / 2 - 1 / 6)
+    qw = 1.602176634e-19 * cfg["weight"] / 2.0 ** 32
+    b = qw * (qe + qh)[1:-1] * (area * d / (verb * 8.8541878128e-12))
+    b[-1] += area / d * phi[-1]
+    p = phi.copy()
+    p[0] = p[-1] = 0.0
+    c = p[1:-1]
+    r = b - (ap + am + 2 * area / d) * c + area / d * (p[2:] + p[:-2])
+    r[:, :-1] += ap[:-1] * c[:, 1:]
+    r[:, 1:] += am[1:] * c[:, :-1]
+    rel = np.linalg.norm(r) / np.linalg.norm(b)
+    sc = sim.scalars()
+    assert sc["poisson_relres"] <= 1e-9
+    # rounding of r's terms: a few 1e-16 of |A| |phi|, far below 1e-9 |b|
+    assert rel <= 1.01e-9, rel
+
+
 @pytest.mark.parametrize("n,nr", [(64, 64), (120, 480)])
 def test_rz_self_consistent_steps_track_oracle(pd, xs, n, nr):
     """A few self-consistent steps: the two field solves agree to ~1e-9, so
