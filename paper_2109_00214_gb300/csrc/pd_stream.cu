@@ -1,9 +1,11 @@
 // pd_stream.cu -- the particle-streaming kernels of the step.
 //
-//   k_push4       Newton push (Sec. 2.1) with the field gathered by the CIC
-//                 weights of Eq. (10), r-z rotation or periodic wrap,
-//                 absorbing walls, fused with the fixed-point CIC deposit of
-//                 Eq. (9)-(10) and the bookkeeping of the cell sort.
+//   k_push4, k_push_rz
+//                 Newton push (Sec. 2.1) with the field gathered by the CIC
+//                 weights of Eq. (10), fused with the fixed-point CIC deposit
+//                 of Eq. (9)-(10) and the bookkeeping of the cell sort:
+//                 k_push4 with periodic walls (Cartesian), k_push_rz with the
+//                 r-z rotation and absorbing walls.
 //   k_bins        per heavy bin: new count, overflow check, closing of the
 //                 holes the push left (short bins; long ones are queued for
 //                 k_compact_big, a warp per bin).
@@ -39,7 +41,7 @@
 // order inside a bin is not canonical (ascending id is found where it
 // matters, in the collisions).
 //
-// The push moves four consecutive particles per thread with 128-bit loads
+// k_push4 moves four consecutive particles per thread with 128-bit loads
 // issued before use.  Sorted input means the four usually share a cell, so
 // counts and deposited charge are merged over runs of equal keys inside the
 // thread (no warp-wide collectives on the common path), and the push
@@ -119,8 +121,8 @@ __device__ __forceinline__ bool flagged(uint32_t k) { return k != DEAD && (k & K
 // whose particle is in the mover buffer M; out_cnt / in_cnt: particles
 // leaving / entering each bin.  Every electron is a mover (the electron bins
 // are rebuilt each step), and so is every particle of the tail.
-template <bool RZ, bool FIELD, bool MULTI>
-__global__ void __launch_bounds__(256, (RZ || FIELD) ? 3 : 4) k_push4(Particles A, const float2* __restrict__ E, long long* rho_e,
+template <bool FIELD, bool MULTI>
+__global__ void __launch_bounds__(256, FIELD ? 3 : 4) k_push4(Particles A, const float2* __restrict__ E, long long* rho_e,
                                                long long* rho_h, uint32_t* out_cnt, uint32_t* in_cnt,
                                                uint32_t* mv, uint32_t* mm, Particles M, DevState* st, KParams P) {
     __shared__ RunInfo s_runs[MULTI ? MAX_RUNS_SMEM : 1];
@@ -134,7 +136,7 @@ __global__ void __launch_bounds__(256, (RZ || FIELD) ? 3 : 4) k_push4(Particles 
     if (blockIdx.x == 0 && threadIdx.x == 0) st->e_from = n_sorted;
     const uint32_t nv = (n + 3u) >> 2;
     const uint32_t stride = gridDim.x * blockDim.x;
-    const int geom = RZ ? 0 : 1;
+    constexpr int geom = 1;
     uint4* key4 = reinterpret_cast<uint4*>(A.key);
     float4* pz4 = reinterpret_cast<float4*>(A.pz);
     float4* pr4 = reinterpret_cast<float4*>(A.pr);
@@ -148,7 +150,7 @@ __global__ void __launch_bounds__(256, (RZ || FIELD) ? 3 : 4) k_push4(Particles 
         const bool gv = g < nv;
         const uint4 K = Kn;
         Kn = g + stride < nv ? key4[g + stride] : dead4;
-        float4 Z = make_float4(0, 0, 0, 0), R4 = Z, VZ = Z, VR = Z, VT = Z;
+        float4 Z = make_float4(0, 0, 0, 0), R4 = Z, VZ = Z, VR = Z;
         // groups of four free slots (the bins' slack) read only their keys;
         // heavies move on heavy steps only, so on the other steps a group of
         // the heavy bins needs work only where the last collisions converted
@@ -162,9 +164,8 @@ __global__ void __launch_bounds__(256, (RZ || FIELD) ? 3 : 4) k_push4(Particles 
             R4 = pr4[g];
             VZ = vz4[g];
             VR = vr4[g];
-            if (RZ) VT = vt4[g];
         }
-        if constexpr (!RZ && !FIELD && !MULTI) {
+        if constexpr (!FIELD && !MULTI) {
             // Neutral copper staying in its cell.  On a heavy step, when every
             // live particle of the warp's groups is a neutral copper atom of
             // the heavy bins (its key carries no conversion) whose new
@@ -201,16 +202,16 @@ __global__ void __launch_bounds__(256, (RZ || FIELD) ? 3 : 4) k_push4(Particles 
             }
         }
         uint32_t key[4], newbin[4], oldbin[4];
-        float zo[4], ro[4], vzo[4], vro[4], vto[4];
-        int sp_[4], iz_[4], ir_[4], wall_[4], run_[4];
-        bool mover[4], inmv[4], dep[4], absd[4];
+        float zo[4], ro[4], vzo[4], vro[4];
+        int sp_[4], iz_[4], ir_[4], run_[4];
+        bool mover[4], inmv[4], dep[4];
         uint32_t flags = 0;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const uint32_t i = 4u * g + (uint32_t)q;
             const uint32_t key_in = (gv && i < n) ? lane_of(K, q) : DEAD;
             const float pz = lane_of(Z, q), pr = lane_of(R4, q);
-            float vz = lane_of(VZ, q), vr = lane_of(VR, q), vt = lane_of(VT, q);
+            float vz = lane_of(VZ, q), vr = lane_of(VR, q);
             const bool live = key_in != DEAD;
             const int sp = live ? (int)key_species(key_in) : 0;
             const uint32_t gcell_in = live ? key_cell(key_in) : 0u;
@@ -238,47 +239,21 @@ __global__ void __launch_bounds__(256, (RZ || FIELD) ? 3 : 4) k_push4(Particles 
             int niz = iz + (int)fz;
             float npz = z - fz;
             npz = npz >= 1.0f ? 0x1.fffffep-1f : npz;
-            int nir;
-            float npr;
-            bool out = false;
-            bool fin;        // the new position is finite (a fault upstream makes it NaN or infinite)
-            if (RZ) {
-                const float x = ((float)ir + pr) + vr * dtr;
-                const float y = vt * dtr;
-                const float rr = sqrtf(x * x + y * y);
-                fin = isfinite(z) && isfinite(rr);
-                const bool pos = rr > 0.0f;
-                const float c = pos ? x / rr : 1.0f, s = pos ? y / rr : 0.0f;
-                const float nvr = c * vr + s * vt;
-                const float nvt = c * vt - s * vr;
-                vr = nvr;
-                vt = nvt;
-                const float fr = floorf(rr);
-                nir = (int)fr;
-                npr = rr - fr;
-                npr = npr >= 1.0f ? 0x1.fffffep-1f : npr;
-                out = niz < 0 || niz >= RI.nz || nir >= RI.nr;
-                // cathode (z = 0) before anode (z = L) before the outer wall (r = R)
-                wall_[q] = niz < 0 ? 0 : (niz >= RI.nz ? 1 : 2);
-            } else {
-                wall_[q] = 0;
-                const float rr = pr + vr * dtr;
-                const float fr = floorf(rr);
-                nir = ir + (int)fr;
-                npr = rr - fr;
-                npr = npr >= 1.0f ? 0x1.fffffep-1f : npr;
-                // a particle crosses at most one period per step (|v dt| < one domain)
-                niz = wrap1(niz, RI.nz);
-                nir = wrap1(nir, RI.nr);
-                // a finite step stays within one period, so the indices are in range
-                fin = (unsigned)niz < (unsigned)RI.nz && (unsigned)nir < (unsigned)RI.nr;
-            }
+            const float rr = pr + vr * dtr;
+            const float fr = floorf(rr);
+            int nir = ir + (int)fr;
+            float npr = rr - fr;
+            npr = npr >= 1.0f ? 0x1.fffffep-1f : npr;
+            // a particle crosses at most one period per step (|v dt| < one domain)
+            niz = wrap1(niz, RI.nz);
+            nir = wrap1(nir, RI.nr);
+            // a finite step stays within one period, so the indices are in range
+            const bool fin = (unsigned)niz < (unsigned)RI.nz && (unsigned)nir < (unsigned)RI.nr;
             // a non-finite position (a fault upstream) would index outside the
             // grid: the particle is dropped and the error flagged
             const bool bad = move && !fin;
             if (bad) set_error(st, ERR_NONFINITE);
-            const bool absorbed = move && (out || bad);
-            const bool kp = live && !absorbed;
+            const bool kp = live && !bad;
             const uint32_t gcell =
                 move ? RI.cell_base + (uint32_t)niz * (uint32_t)RI.nr + (uint32_t)nir : gcell_in;
             const uint32_t k = kp ? make_key((uint32_t)sp, gcell) : DEAD;
@@ -290,58 +265,21 @@ __global__ void __launch_bounds__(256, (RZ || FIELD) ? 3 : 4) k_push4(Particles 
             newbin[q] = nb;
             mover[q] = mvq;
             inmv[q] = inq;
-            absd[q] = absorbed && !bad;                   // (ledgers and impacts of finite particles only)
             zo[q] = mk ? npz : pz;
-            ro[q] = (mk || absorbed) ? npr : pr;           // an absorbed particle keeps its impact r
+            ro[q] = mk ? npr : pr;
             vzo[q] = move ? vz : lane_of(VZ, q);
             vro[q] = move ? vr : lane_of(VR, q);
-            vto[q] = move ? vt : lane_of(VT, q);
             sp_[q] = sp;
             run_[q] = r;
             iz_[q] = mk ? niz : iz;
-            ir_[q] = (mk || absorbed) ? nir : ir;
+            ir_[q] = mk ? nir : ir;
             dep[q] = mk && charge_of(sp) != 0;
             // 16: the particle moved and keeps its slot (written back); a
-            // mover's slot is refilled by the sort, an absorbed one's too
-            flags |= (absorbed ? 1u : 0u) | (mvq ? 2u : 0u) | (inq ? 4u : 0u) | (dep[q] ? 8u : 0u) |
+            // mover's slot is refilled by the sort
+            flags |= (mvq ? 2u : 0u) | (inq ? 4u : 0u) | (dep[q] ? 8u : 0u) |
                      ((mk && !inq) ? 16u : 0u);
         }
         const uint32_t wflags = __reduce_or_sync(FULL_MASK, flags);
-        if (RZ && (wflags & 1u)) {  // absorbed at an electrode or the outer wall: ledgers
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                if (!absd[q]) continue;
-                const int sp = sp_[q];
-                const int electrode = wall_[q];
-                RunState& rs = P.rs[run_[q]];
-                const double v2 = (double)vzo[q] * vzo[q] + (double)vro[q] * vro[q] + (double)vto[q] * vto[q];
-                const double w = MULTI ? s_runs[run_[q]].weight : P.run0.weight;
-                const double ke = w * (0.5 * pick_sp(P.masses, sp) * v2);
-                atomicAdd(&rs.ctr[C_ABS + electrode * NSP + sp], 1ull);
-                atomicAdd(&rs.absorbed_energy[electrode], ke);
-                const double qw = (double)charge_of(sp) * 1.602176634e-19 * w;
-                if (electrode == 1) atomicAdd(&rs.anode_charge_step, qw);
-                if (electrode == 0) atomicAdd(&rs.charge_cathode, qw);
-                // an ion arriving at an electrode inside the outer radius sputters
-                // floor(Y(E) + R) atoms (emitted by k_sputter)
-                const RunInfo& RI = MULTI ? s_runs[run_[q]] : P.run0;
-                if (P.sputter && electrode < 2 && charge_of(sp) > 0 && ir_[q] < RI.nr) {
-                    const float E = (float)((0.5 * pick_sp(P.masses, sp) * v2) / 1.602176634e-19);
-                    const float Y = xs_lookup(P.xsE, P.ytab, E);
-                    const uint32_t id = A.id[4u * g + (uint32_t)q];
-                    Stream rs_(id, st->step, SID_SPUT, RI.seed, RI.run);
-                    const uint32_t nsp = (uint32_t)floorf(Y + rs_.u01());
-                    if (nsp) {
-                        const uint32_t x = atomicAdd(&st->n_sput, 1u);
-                        if (x < P.squeue_cap)
-                            P.squeue[x] = SputRec{id, ((uint32_t)run_[q] << 1) | (uint32_t)electrode, (uint32_t)ir_[q],
-                                                  ro[q], nsp};
-                        else
-                            set_error(st, ERR_CAPACITY);
-                    }
-                }
-            }
-        }
         if (wflags & 2u) {          // movers out of their sorted bin
             uint32_t nib = 0;
 #pragma unroll
@@ -370,7 +308,7 @@ __global__ void __launch_bounds__(256, (RZ || FIELD) ? 3 : 4) k_push4(Particles 
                 reinterpret_cast<float4*>(M.pr)[g] = make_float4(ro[0], ro[1], ro[2], ro[3]);
                 reinterpret_cast<float4*>(M.vz)[g] = make_float4(vzo[0], vzo[1], vzo[2], vzo[3]);
                 reinterpret_cast<float4*>(M.vr)[g] = make_float4(vro[0], vro[1], vro[2], vro[3]);
-                reinterpret_cast<float4*>(M.vt)[g] = RZ ? make_float4(vto[0], vto[1], vto[2], vto[3]) : vt4[g];
+                reinterpret_cast<float4*>(M.vt)[g] = vt4[g];
                 reinterpret_cast<uint4*>(M.id)[g] = reinterpret_cast<const uint4*>(A.id)[g];
                 atomicOr(&mm[g >> 3], nib << (4u * (g & 7u)));
             }
@@ -396,55 +334,21 @@ __global__ void __launch_bounds__(256, (RZ || FIELD) ? 3 : 4) k_push4(Particles 
                 if (link[q])
 #pragma unroll
                     for (int c = 0; c < 4; ++c) W[q - 1][c] += W[q][c];
-            // r-z plumes hold cells of thousands of particles: when all 128
-            // particles of the warp deposit into one cell, the warp sums the
-            // four corner weights and issues four atomics instead of 128
-            bool one_cell_warp = false;
-            if constexpr (RZ) {
-                const uint32_t k0 = __shfl_sync(FULL_MASK, key[0], 0);
-                const bool one_cell = dep[0] && dep[1] && dep[2] && dep[3] && key[0] == k0 && key[1] == k0 &&
-                                      key[2] == k0 && key[3] == k0;
-                one_cell_warp = __all_sync(FULL_MASK, one_cell);
-            }
-            if (one_cell_warp) {
-                unsigned long long Ws[4];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    Ws[c] = W[0][c];
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) Ws[c] += __shfl_down_sync(FULL_MASK, Ws[c], o);
-                }
-                if ((threadIdx.x & 31u) == 0) {
-                    const long long zq = charge_of(sp_[0]);
-                    long long* rho = sp_[0] == SP_E ? rho_e : rho_h;
-                    const RunInfo& RI = MULTI ? s_runs[run_[0]] : P.run0;
-                    const int iz = iz_[0], ir = ir_[0];
-                    atomicAdd((unsigned long long*)&rho[node_of(RI, geom, iz, ir)],
-                              (unsigned long long)(zq * (long long)Ws[0]));
-                    atomicAdd((unsigned long long*)&rho[node_of(RI, geom, iz + 1, ir)],
-                              (unsigned long long)(zq * (long long)Ws[1]));
-                    atomicAdd((unsigned long long*)&rho[node_of(RI, geom, iz, ir + 1)],
-                              (unsigned long long)(zq * (long long)Ws[2]));
-                    atomicAdd((unsigned long long*)&rho[node_of(RI, geom, iz + 1, ir + 1)],
-                              (unsigned long long)(zq * (long long)Ws[3]));
-                }
-            } else {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    if (!len[q]) continue;
-                    const long long zq = charge_of(sp_[q]);
-                    long long* rho = sp_[q] == SP_E ? rho_e : rho_h;
-                    const RunInfo& RI = MULTI ? s_runs[run_[q]] : P.run0;
-                    const int iz = iz_[q], ir = ir_[q];
-                    atomicAdd((unsigned long long*)&rho[node_of(RI, geom, iz, ir)],
-                              (unsigned long long)(zq * (long long)W[q][0]));
-                    atomicAdd((unsigned long long*)&rho[node_of(RI, geom, iz + 1, ir)],
-                              (unsigned long long)(zq * (long long)W[q][1]));
-                    atomicAdd((unsigned long long*)&rho[node_of(RI, geom, iz, ir + 1)],
-                              (unsigned long long)(zq * (long long)W[q][2]));
-                    atomicAdd((unsigned long long*)&rho[node_of(RI, geom, iz + 1, ir + 1)],
-                              (unsigned long long)(zq * (long long)W[q][3]));
-                }
+            for (int q = 0; q < 4; ++q) {
+                if (!len[q]) continue;
+                const long long zq = charge_of(sp_[q]);
+                long long* rho = sp_[q] == SP_E ? rho_e : rho_h;
+                const RunInfo& RI = MULTI ? s_runs[run_[q]] : P.run0;
+                const int iz = iz_[q], ir = ir_[q];
+                atomicAdd((unsigned long long*)&rho[node_of(RI, geom, iz, ir)],
+                          (unsigned long long)(zq * (long long)W[q][0]));
+                atomicAdd((unsigned long long*)&rho[node_of(RI, geom, iz + 1, ir)],
+                          (unsigned long long)(zq * (long long)W[q][1]));
+                atomicAdd((unsigned long long*)&rho[node_of(RI, geom, iz, ir + 1)],
+                          (unsigned long long)(zq * (long long)W[q][2]));
+                atomicAdd((unsigned long long*)&rho[node_of(RI, geom, iz + 1, ir + 1)],
+                          (unsigned long long)(zq * (long long)W[q][3]));
             }
         }
         // write back the particles that moved and keep their slot (keys do not
@@ -452,11 +356,10 @@ __global__ void __launch_bounds__(256, (RZ || FIELD) ? 3 : 4) k_push4(Particles 
         if (gv && (flags & 16u)) {
             pz4[g] = make_float4(zo[0], zo[1], zo[2], zo[3]);
             pr4[g] = make_float4(ro[0], ro[1], ro[2], ro[3]);
-            if (FIELD || RZ) {
+            if (FIELD) {
                 vz4[g] = make_float4(vzo[0], vzo[1], vzo[2], vzo[3]);
                 vr4[g] = make_float4(vro[0], vro[1], vro[2], vro[3]);
             }
-            if (RZ) vt4[g] = make_float4(vto[0], vto[1], vto[2], vto[3]);
         }
     }
 }
@@ -1141,21 +1044,301 @@ __global__ void k_relayout_done(const uint32_t* __restrict__ off, uint32_t nbins
     for (int k = 0; k < NSP; ++k) st->sp_cnt[k] = st->sp_act[k] = 0ull;
 }
 
+// ---------------------------------------------------------------------
+// the push in r-z
+// ---------------------------------------------------------------------
+// sum of the corner weights of `cnt` particles from the sums of w_z, w_r and
+// w_z w_r: corner 0 (2^16 - w_z)(2^16 - w_r), 1 w_z (2^16 - w_r), 2 (2^16 - w_z) w_r,
+// 3 w_z w_r
+__device__ __forceinline__ unsigned long long corner_sum(int c, uint32_t cnt, uint32_t swz, uint32_t swr,
+                                                         unsigned long long pw) {
+    const unsigned long long a = (unsigned long long)swz << 16, b = (unsigned long long)swr << 16;
+    return c == 0 ? ((unsigned long long)cnt << 32) - a - b + pw : c == 1 ? a - pw : c == 2 ? b - pw : pw;
+}
+
+// One row of 32 consecutive slots (a lane a slot, i = row * 32 + lane), loaded by
+// the caller; see k_push_rz.  EL: electrons after the heavy bins only (all of
+// them move, and all are movers).
+template <bool FIELD, bool MULTI, bool EL>
+__device__ __forceinline__ void push_row(uint32_t row, uint32_t n_sorted, uint32_t key_in, float pz, float pr, float vz,
+                                         float vr, float vt, const RunInfo* s_runs, const Particles& A,
+                                         const float2* __restrict__ E, long long* rho_e, long long* rho_h,
+                                         uint32_t* out_cnt, uint32_t* in_cnt, uint32_t* mv, uint32_t* mm,
+                                         const Particles& M, DevState* st, const KParams& P) {
+    const uint32_t lane = threadIdx.x & 31u, i = row * 32u + lane;
+    const bool live = key_in != DEAD;
+    // an electron's id is needed for its record: loaded ahead of the arithmetic
+    const uint32_t id_e = EL && live ? A.id[i] : 0u;
+    const int sp = EL ? SP_E : live ? (int)key_species(key_in) : 0;
+    const uint32_t gcell_in = live ? key_cell(key_in) : 0u;
+    const int r = live ? run_of(P, gcell_in) : 0;
+    const RunInfo& RI = MULTI ? s_runs[r] : P.run0;
+    const bool in_sorted = !EL && live && i < n_sorted;
+    const uint32_t oldbin = in_sorted ? key_sorted_species(key_in) * P.ncell + gcell_in : NOBIN;
+    const bool move = live && (EL || sp == SP_E || P.heavy_step);
+    const uint32_t lcell = move ? gcell_in - RI.cell_base : 0u;       // dead lanes read a valid node
+    int iz, ir;
+    decode_cell(lcell, RI.nr, RI.inv_nr, iz, ir);
+    const float qmdt = spc<MULTI>(RI.qmdt, sp), dtz = spc_eh<MULTI>(RI.dtz, sp), dtr = spc_eh<MULTI>(RI.dtr, sp);
+    const float vz0 = vz, vr0 = vr, vt0 = vt;
+    if (FIELD) {
+        const uint32_t k0 = node_of(RI, 0, iz, ir), k1 = k0 + (uint32_t)RI.nrn;
+        const float2 e00 = E[k0], e10 = E[k1], e01 = E[k0 + 1u], e11 = E[k1 + 1u];
+        const float gz = 1.0f - pz, gr = 1.0f - pr;
+        const float w00 = gz * gr, w10 = pz * gr, w01 = gz * pr, w11 = pz * pr;
+        const float ez = ((w00 * e00.x + w10 * e10.x) + w01 * e01.x) + w11 * e11.x;
+        const float er = ((w00 * e00.y + w10 * e10.y) + w01 * e01.y) + w11 * e11.y;
+        vz = vz + qmdt * ez;
+        vr = vr + qmdt * er;
+    }
+    const float z = pz + vz * dtz;
+    const float fz = floorf(z);
+    const int niz = iz + (int)fz;
+    float npz = z - fz;
+    npz = npz >= 1.0f ? 0x1.fffffep-1f : npz;
+    const float x = ((float)ir + pr) + vr * dtr;
+    const float y = vt * dtr;
+    const float rr = sqrtf(x * x + y * y);
+    const bool fin = isfinite(z) && isfinite(rr);    // (a fault upstream makes the new position NaN or infinite)
+    const bool pos = rr > 0.0f;
+    const float c = pos ? x / rr : 1.0f, s = pos ? y / rr : 0.0f;
+    const float nvr = c * vr + s * vt;
+    const float nvt = c * vt - s * vr;
+    vr = nvr;
+    vt = nvt;
+    const float fr = floorf(rr);
+    const int nir = (int)fr;
+    float npr = rr - fr;
+    npr = npr >= 1.0f ? 0x1.fffffep-1f : npr;
+    const bool out = niz < 0 || niz >= RI.nz || nir >= RI.nr;
+    // a non-finite position would index outside the grid: the particle is
+    // dropped and the error flagged
+    const bool bad = move && !fin;
+    if (bad) set_error(st, ERR_NONFINITE);
+    const bool absorbed = move && (out || bad);
+    const bool kp = live && !absorbed;
+    const uint32_t gcell = move ? RI.cell_base + (uint32_t)niz * (uint32_t)RI.nr + (uint32_t)nir : gcell_in;
+    const uint32_t key = kp ? make_key((uint32_t)sp, gcell) : DEAD;
+    const uint32_t newbin = kp ? (uint32_t)sp * P.ncell + gcell : NOBIN;
+    const bool mover = in_sorted && newbin != oldbin;
+    const bool inmv = kp && (!in_sorted || newbin != oldbin);
+    const bool mk = move && kp;
+    const int zq = charge_of(sp);
+    const bool dep = mk && zq != 0;
+    const float zo = mk ? npz : pz, ro = mk ? npr : pr;
+    if (!EL && !move) {
+        vz = vz0;
+        vr = vr0;
+        vt = vt0;
+    }
+    if (absorbed && !bad) {     // at an electrode or the outer wall: ledgers (finite particles only)
+        // cathode (z = 0) before anode (z = L) before the outer wall (r = R)
+        const int electrode = niz < 0 ? 0 : (niz >= RI.nz ? 1 : 2);
+        RunState& rs = P.rs[r];
+        const double v2 = (double)vz * vz + (double)vr * vr + (double)vt * vt;
+        const double w = RI.weight;
+        const double ke = w * (0.5 * pick_sp(P.masses, sp) * v2);
+        atomicAdd(&rs.ctr[C_ABS + electrode * NSP + sp], 1ull);
+        atomicAdd(&rs.absorbed_energy[electrode], ke);
+        const double qw = (double)zq * 1.602176634e-19 * w;
+        if (electrode == 1) atomicAdd(&rs.anode_charge_step, qw);
+        if (electrode == 0) atomicAdd(&rs.charge_cathode, qw);
+        // an ion arriving at an electrode inside the outer radius sputters
+        // floor(Y(E) + R) atoms (emitted by k_sputter)
+        if (P.sputter && electrode < 2 && zq > 0 && nir < RI.nr) {
+            const float Ei = (float)((0.5 * pick_sp(P.masses, sp) * v2) / 1.602176634e-19);
+            const float Y = xs_lookup(P.xsE, P.ytab, Ei);
+            const uint32_t id = A.id[i];
+            Stream rs_(id, st->step, SID_SPUT, RI.seed, RI.run);
+            const uint32_t nsp = (uint32_t)floorf(Y + rs_.u01());
+            if (nsp) {
+                const uint32_t q = atomicAdd(&st->n_sput, 1u);
+                if (q < P.squeue_cap)
+                    P.squeue[q] = SputRec{id, ((uint32_t)r << 1) | (uint32_t)electrode, (uint32_t)nir, npr, nsp};
+                else
+                    set_error(st, ERR_CAPACITY);
+            }
+        }
+    }
+    const uint32_t m_out = EL ? 0u : __ballot_sync(FULL_MASK, mover);
+    if (m_out) {                // movers out of their sorted bin
+        if (mover) atomicAdd(&out_cnt[oldbin], 1u);
+        if (lane == 0) atomicOr(&mv[row], m_out);
+    }
+    const uint32_t m_in = __ballot_sync(FULL_MASK, inmv);
+    if (m_in) {                 // into their new bin (all particles after a load)
+        if (inmv) {
+            M.key[i] = key;
+            M.pz[i] = zo;
+            M.pr[i] = ro;
+            M.vz[i] = vz;
+            M.vr[i] = vr;
+            M.vt[i] = vt;
+            M.id[i] = EL ? id_e : A.id[i];
+        }
+        if (lane == 0) atomicOr(&mm[row], m_in);
+    }
+    // write back the particles that moved and keep their slot (keys do not change there)
+    if (!EL && mk && !inmv) {
+        A.pz[i] = zo;
+        A.pr[i] = ro;
+        A.vz[i] = vz;
+        A.vr[i] = vr;
+        A.vt[i] = vt;
+    }
+    // movers-in counts and fixed-point CIC deposit.  The row's particles come
+    // from one or two bins (sorted slots) and most stay in their cell: those
+    // that end in the cell of the row's first or last particle are summed over
+    // the warp and added by a lane a node, the others each add their own.
+    const uint32_t on = EL ? m_in : __ballot_sync(FULL_MASK, dep || inmv);
+    if (!on) return;
+    const uint32_t wz = __float2uint_rn(zo * 65536.0f), wr = __float2uint_rn(ro * 65536.0f);
+    const unsigned long long pw = (unsigned long long)wz * wr;
+    const uint32_t home = live ? make_key((uint32_t)sp, gcell_in) : DEAD;
+    bool todo = dep || inmv;
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+        const uint32_t k0 = __shfl_sync(FULL_MASK, home, side ? 31 - __clz(on) : __ffs(on) - 1);
+        const bool mine = todo && key == k0;
+        const uint32_t m = __ballot_sync(FULL_MASK, mine);
+        if (__popc(m) < 4) continue;
+        todo = todo && !mine;
+        const uint32_t cin = EL ? __popc(m) : __popc(__ballot_sync(FULL_MASK, mine && inmv));
+        const int z0 = EL ? -1 : charge_of((int)key_species(k0));
+        const uint32_t c0 = key_cell(k0);
+        const int r0 = run_of(P, c0);
+        const RunInfo& R0 = MULTI ? s_runs[r0] : P.run0;
+        if (lane == 0 && cin) atomicAdd(&in_cnt[key_species(k0) * P.ncell + c0], cin);
+        const bool d = mine && dep;
+        const uint32_t md = EL ? m : __ballot_sync(FULL_MASK, d);
+        if (!md) continue;
+        const uint32_t swz = __reduce_add_sync(FULL_MASK, d ? wz : 0u), swr = __reduce_add_sync(FULL_MASK, d ? wr : 0u);
+        const uint32_t ph = __reduce_add_sync(FULL_MASK, d ? (uint32_t)(pw >> 16) : 0u);
+        const uint32_t pl = __reduce_add_sync(FULL_MASK, d ? (uint32_t)(pw & 0xFFFFu) : 0u);
+        if (lane < 4u) {
+            int jz, jr;
+            decode_cell(c0 - R0.cell_base, R0.nr, R0.inv_nr, jz, jr);
+            const unsigned long long w =
+                corner_sum((int)lane, __popc(md), swz, swr, ((unsigned long long)ph << 16) + pl);
+            long long* rho = EL || key_species(k0) == (uint32_t)SP_E ? rho_e : rho_h;
+            atomicAdd((unsigned long long*)&rho[node_of(R0, 0, jz + (int)(lane & 1u), jr + (int)(lane >> 1))],
+                      (unsigned long long)((long long)z0 * (long long)w));
+        }
+    }
+    if (todo) {
+        if (inmv) atomicAdd(&in_cnt[newbin], 1u);
+        if (dep) {
+            long long* rho = (sp == SP_E ? rho_e : rho_h) + node_of(RI, 0, niz, nir);
+            const long long q = zq;
+            atomicAdd((unsigned long long*)rho, (unsigned long long)(q * (long long)corner_sum(0, 1u, wz, wr, pw)));
+            atomicAdd((unsigned long long*)(rho + RI.nrn),
+                      (unsigned long long)(q * (long long)corner_sum(1, 1u, wz, wr, pw)));
+            atomicAdd((unsigned long long*)(rho + 1), (unsigned long long)(q * (long long)corner_sum(2, 1u, wz, wr, pw)));
+            atomicAdd((unsigned long long*)(rho + RI.nrn + 1),
+                      (unsigned long long)(q * (long long)corner_sum(3, 1u, wz, wr, pw)));
+        }
+    }
+}
+
+// The push of the r-z geometry: the same step as k_push4's, a lane a particle.
+// Gathering the field, absorbing and depositing take too many registers for
+// four particles a thread: that form spilled at 24 warps an SM, waited on memory
+// and issued 1.8 atomics an electron (512 x 512 cells, 1.1e7 electrons: 460 us, 18 %
+// of the DRAM rate).  Here a warp takes rows of 32 consecutive slots with the
+// next row's loads in flight, sums what the row's first and last bins receive
+// over the warp (0.8 atomics an electron), and has a form for the rows of
+// electrons alone: 215 us, bound by the issue of its 420 instructions a row (60 %
+// of the slots; 40 warps an SM spilled and took 263 us).  mv, mm, counts: see
+// k_push4.
+template <bool FIELD, bool MULTI>
+__global__ void __launch_bounds__(256, 4) k_push_rz(Particles A, const float2* __restrict__ E, long long* rho_e,
+                                                                long long* rho_h, uint32_t* out_cnt, uint32_t* in_cnt,
+                                                                uint32_t* mv, uint32_t* mm, Particles M, DevState* st,
+                                                                KParams P) {
+    __shared__ RunInfo s_runs[MULTI ? MAX_RUNS_SMEM : 1];
+    if (st->error) return;                           // a fault was flagged: the state is not stepped further
+    if (MULTI) {
+        for (int r = threadIdx.x; r < P.nruns; r += blockDim.x) s_runs[r] = P.runs[r];
+        __syncthreads();
+    }
+    const uint32_t n = (uint32_t)st->n_slots;
+    const uint32_t n_sorted = (uint32_t)st->e_base;      // slots of the heavy bins; the electron bins follow
+    if (blockIdx.x == 0 && threadIdx.x == 0) st->e_from = n_sorted;
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    const uint32_t nrow = (n + 31u) / 32u, erow = min(n_sorted / 32u, nrow);
+    // On heavy steps every row; on the others the electron bins and the tail,
+    // and of the heavy bins the rows where the last collisions converted a
+    // particle (it changes bin).
+    uint32_t row = (P.heavy_step ? 0u : erow) + w;
+    uint32_t key = DEAD;
+    float pz = 0, pr = 0, vz = 0, vr = 0, vt = 0;
+    auto load = [&](uint32_t q) {
+        const uint32_t i = q * 32u + lane;
+        const bool in = q < nrow && i < n;
+        key = in ? A.key[i] : DEAD;
+        pz = in ? A.pz[i] : 0.0f;
+        pr = in ? A.pr[i] : 0.0f;
+        vz = in ? A.vz[i] : 0.0f;
+        vr = in ? A.vr[i] : 0.0f;
+        vt = in ? A.vt[i] : 0.0f;
+    };
+    load(row);
+    for (; row < nrow; row += nw) {
+        const uint32_t k = key;
+        const float a = pz, b = pr, c = vz, d = vr, e = vt;
+        load(row + nw);
+        if (__any_sync(FULL_MASK, k != DEAD)) {
+            if (row * 32u >= n_sorted && __all_sync(FULL_MASK, k == DEAD || key_species(k) == (uint32_t)SP_E))
+                push_row<FIELD, MULTI, true>(row, n_sorted, k, a, b, c, d, e, s_runs, A, E, rho_e, rho_h, out_cnt,
+                                             in_cnt, mv, mm, M, st, P);
+            else
+                push_row<FIELD, MULTI, false>(row, n_sorted, k, a, b, c, d, e, s_runs, A, E, rho_e, rho_h, out_cnt,
+                                              in_cnt, mv, mm, M, st, P);
+        }
+    }
+    if (P.heavy_step) return;
+    // keys of four rows a load, four loads in flight
+    const uint4* key4 = reinterpret_cast<const uint4*>(A.key);
+    const uint32_t n4 = erow * 8u;                   // groups of four slots
+    const uint4 dead4 = make_uint4(DEAD, DEAD, DEAD, DEAD);
+    for (uint32_t u = w; u * 32u < n4; u += 4u * nw) {
+        uint4 K[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t g = (u + (uint32_t)q * nw) * 32u + lane;
+            K[q] = g < n4 ? key4[g] : dead4;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            uint32_t any = __ballot_sync(FULL_MASK, flagged(K[q].x) || flagged(K[q].y) || flagged(K[q].z) || flagged(K[q].w));
+            while (any) {
+                const uint32_t sub = (__ffs(any) - 1) >> 3;             // row of the four
+                any &= ~(0xFFu << (8u * sub));
+                const uint32_t rq = (u + (uint32_t)q * nw) * 4u + sub;
+                load(rq);
+                push_row<FIELD, MULTI, false>(rq, n_sorted, key, pz, pr, vz, vr, vt, s_runs, A, E, rho_e, rho_h,
+                                              out_cnt, in_cnt, mv, mm, M, st, P);
+            }
+        }
+    }
+}
+
 void launch_push(const Particles& A, const float2* E, long long* rho_e, long long* rho_h, uint32_t* out_cnt,
                  uint32_t* in_cnt, uint32_t* mv, uint32_t* mm, const Particles& M, DevState* st, const KParams& P,
                  int grid, cudaStream_t s) {
     const bool rz = P.geom == 0, field = P.field_on != 0;
 #define PD_PUSH_ARGS A, E, rho_e, rho_h, out_cnt, in_cnt, mv, mm, M, st, P
     if (P.nruns > 1) {
-        if (rz && field) k_push4<true, true, true><<<grid, 256, 0, s>>>(PD_PUSH_ARGS);
-        else if (rz) k_push4<true, false, true><<<grid, 256, 0, s>>>(PD_PUSH_ARGS);
-        else if (field) k_push4<false, true, true><<<grid, 256, 0, s>>>(PD_PUSH_ARGS);
-        else k_push4<false, false, true><<<grid, 256, 0, s>>>(PD_PUSH_ARGS);
+        if (rz && field) k_push_rz<true, true><<<grid, 256, 0, s>>>(PD_PUSH_ARGS);
+        else if (rz) k_push_rz<false, true><<<grid, 256, 0, s>>>(PD_PUSH_ARGS);
+        else if (field) k_push4<true, true><<<grid, 256, 0, s>>>(PD_PUSH_ARGS);
+        else k_push4<false, true><<<grid, 256, 0, s>>>(PD_PUSH_ARGS);
     } else {
-        if (rz && field) k_push4<true, true, false><<<grid, 256, 0, s>>>(PD_PUSH_ARGS);
-        else if (rz) k_push4<true, false, false><<<grid, 256, 0, s>>>(PD_PUSH_ARGS);
-        else if (field) k_push4<false, true, false><<<grid, 256, 0, s>>>(PD_PUSH_ARGS);
-        else k_push4<false, false, false><<<grid, 256, 0, s>>>(PD_PUSH_ARGS);
+        if (rz && field) k_push_rz<true, false><<<grid, 256, 0, s>>>(PD_PUSH_ARGS);
+        else if (rz) k_push_rz<false, false><<<grid, 256, 0, s>>>(PD_PUSH_ARGS);
+        else if (field) k_push4<true, false><<<grid, 256, 0, s>>>(PD_PUSH_ARGS);
+        else k_push4<false, false><<<grid, 256, 0, s>>>(PD_PUSH_ARGS);
     }
 #undef PD_PUSH_ARGS
 }
