@@ -746,8 +746,7 @@ pd_status issue_step(pd_sim* s, bool capturing) {
         Timed t(s, K_COLLIDE, capturing, 3);
         launch_collide(s->A, s->B, s->off, s->bcnt, s->nc, s->nc2, s->cand_off, s->active, s->mid, s->big, s->st,
                        s->rho_e, s->rho_h,
-                       s->xsE, s->xs, s->cw, P, s->cc, nbins, s->sms, grid_for(s, s->tune.collide_blocks_per_sm),
-                       s->stream);
+                       s->xsE, s->xs, P, s->cc, s->sms, grid_for(s, s->tune.collide_blocks_per_sm), s->stream);
     }
     if (P.coulomb) {
         Timed t(s, K_COULOMB, capturing, 1);

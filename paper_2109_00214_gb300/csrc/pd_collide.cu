@@ -10,11 +10,15 @@
 //   k_collide  one warp per active cell.  Candidate m draws from the stream
 //              (cell, step, k<<28 | m): the electron and target ranks (in
 //              ascending-id order inside the cell), the acceptance number and
-//              the channel number.  Lane 0 applies the kinematics.  Spawned electrons go to the slots
+//              the channel number.  The candidates that share no particle
+//              with an earlier one are applied side by side, a lane each,
+//              the others in order.  Spawned electrons go to the slots
 //              reserved for the cell at n_alive + 2 * (candidates of the
 //              cells before it); unused reserved slots are marked dead.
 //   k_finalize slot / id bookkeeping and the RC circuit update.
 // Compiled with -fmad=false (decision arithmetic is rounded op by op).
+#include <algorithm>
+
 #include "pd_internal.cuh"
 #include "pd_kernels.h"
 
@@ -27,7 +31,9 @@ struct V3 {
 };
 
 // isotropic unit vector, Marsaglia (1972)
-__device__ V3 iso_dir(Stream& st, uint32_t& fb) {
+template <typename S>
+__device__ __forceinline__ V3 iso_dir(S& st, uint32_t& fb) {
+#pragma unroll 1
     for (int a = 0; a < 64; ++a) {
         const float u1 = 2.0f * st.u01() - 1.0f;
         const float u2 = 2.0f * st.u01() - 1.0f;
@@ -42,7 +48,9 @@ __device__ V3 iso_dir(Stream& st, uint32_t& fb) {
 }
 
 // uniform azimuth (cos, sin) from a point of the unit disc
-__device__ void azimuth(Stream& st, float& c, float& s, uint32_t& fb) {
+template <typename S>
+__device__ __forceinline__ void azimuth(S& st, float& c, float& s, uint32_t& fb) {
+#pragma unroll 1
     for (int a = 0; a < 64; ++a) {
         const float u1 = 2.0f * st.u01() - 1.0f;
         const float u2 = 2.0f * st.u01() - 1.0f;
@@ -61,7 +69,8 @@ __device__ void azimuth(Stream& st, float& c, float& s, uint32_t& fb) {
 
 // Eq. (6): |u'|^2 = |u|^2 - 2 E_th / m_r (kth); Eq. (7) isotropic direction;
 // Eq. (5): v1 += (u' - u) m_r/m1, v2 -= (u' - u) m_r/m2.
-__device__ bool binary_scatter(Stream& st, V3& v1, V3& v2, float kth, float a1, float a2, uint32_t& fb) {
+template <typename S>
+__device__ __forceinline__ bool binary_scatter(S& st, V3& v1, V3& v2, float kth, float a1, float a2, uint32_t& fb) {
     const V3 u{v1.x - v2.x, v1.y - v2.y, v1.z - v2.z};
     const float g2 = (u.x * u.x + u.y * u.y) + u.z * u.z;
     const float up2 = g2 - kth;
@@ -80,7 +89,8 @@ __device__ bool binary_scatter(Stream& st, V3& v1, V3& v2, float kth, float a1, 
 
 // Eq. (15)-(20): v5 = cos(chi) |v| R^T(theta, phi) (sin chi cos psi,
 // sin chi sin psi, cos chi); v6 = v - v5; theta, phi from the components of v.
-__device__ void rectangle_split(Stream& st, const V3& v, V3& v5, V3& v6, int mode, uint32_t& fb) {
+template <typename S>
+__device__ __forceinline__ void rectangle_split(S& st, const V3& v, V3& v5, V3& v6, int mode, uint32_t& fb) {
     float cchi = st.u01();
     if (mode == 1) cchi = sqrtf(cchi);
     const float schi = sqrtf(1.0f - cchi * cchi);
@@ -108,7 +118,7 @@ __device__ void rectangle_split(Stream& st, const V3& v, V3& v5, V3& v6, int mod
 }
 
 // single-particle fixed-point CIC deposit of zq at (local cell, pz, pr) of run RI
-__device__ void deposit1(long long* rho, const RunInfo& RI, int geom, uint32_t lcell, float pz, float pr, int zq) {
+__device__ __noinline__ void deposit1(long long* rho, const RunInfo& RI, int geom, uint32_t lcell, float pz, float pr, int zq) {
     const int iz = (int)(lcell / (uint32_t)RI.nr);
     const int ir = (int)(lcell - (uint32_t)iz * (uint32_t)RI.nr);
     const uint32_t wz = __float2uint_rn(pz * 65536.0f);
@@ -126,23 +136,19 @@ __device__ void deposit1(long long* rho, const RunInfo& RI, int geom, uint32_t l
 // scatter's atomics, so each list the candidates use is mapped rank ->
 // position by one of:
 //   * ids already ascending with the position (rank = position);
-//   * up to 64 ids: a rank table by comparisons (the rank of an id is the
-//     number of smaller ids in the list);
-//   * up to 32 * RC ids with lookups that cost less than a table: a radix
-//     select over the ids held in registers, per lookup;
-//   * longer lists with at most SELECT_LOOKUPS lookups: a select per lookup
-//     over the list in global memory (select8);
-//   * otherwise a rank table, position of the r-th smallest id at table[r],
-//     from a stable LSD radix sort of (id, position) pairs by 8-bit digits:
-//     by the cell's warp in its shared memory for the register-cached lists
-//     (up to RANK_WARP_MAX = 32 * RC ids), by a block of k_rank_tables
-//     (before k_collide) for longer lists, in shared memory up to
-//     RANK_BLOCK_MAX ids and in the scratch buffers above that.
-// The table of the list at slots [b, b + n) is written to table[b, b + n).
+//   * a rank table, position of the r-th smallest id at table[r].  Up to 32
+//     ids (64 when their range needs two digits): by comparisons (the rank of
+//     an id is the number of smaller ids in the list); up to RANK_WARP_MAX =
+//     32 * RC: a stable LSD radix sort of (id, position) pairs by 8-bit digits
+//     of id - (smallest id), by the cell's warp in its shared memory; longer
+//     lists: the same sort by a block of k_rank_tables (before k_collide), in
+//     shared memory up to RANK_BLOCK_MAX ids and in the scratch buffers above
+//     that;
+//   * few lookups in a long list: a select per lookup over the list in global
+//     memory (select8).
+// A block's table of the list at slots [b, b + n) is written to table[b, b + n).
 
-// Register-cached id list of one cell and species: element lane + 32 k in
-// ids[k], for lists of up to 32 * RC ids (one coalesced load per cell).
-constexpr int RC = 8;
+constexpr int RC = 8;                           // rows of 32 ids a warp sorts itself
 constexpr uint32_t RANK_BLOCK_MAX = 12288;      // longest list the large kernel sorts in shared memory
 constexpr int RT_THREADS = 1024;                // threads of a large-kernel block
 constexpr int RT_MID_THREADS = 256;             // threads of a mid-size-kernel block
@@ -150,15 +156,11 @@ constexpr int RT_MID_BLOCKS_PER_SM = 5;
 constexpr uint32_t SENTINEL = 0xFFFFFFFFu;
 
 struct IdList {
-    uint32_t ids[RC];
     const uint32_t* table;           // rank -> position, or null
     const uint32_t* base;            // the ids in global memory (select8)
-    uint32_t* cnt;                   // the warp's 256 shared counters (select8)
+    int top;                         // highest set bit of any id (select8)
     uint32_t n;
-    int top;                         // highest set bit of any id (0 if none)
-    bool cached;
     bool sorted;                     // ids ascend with the position: rank = position
-    bool sel8;                       // a long list with few lookups: select8 per lookup
 };
 
 // lookups up to which a list longer than 32 * RC ids is searched per lookup
@@ -189,9 +191,10 @@ __device__ __forceinline__ unsigned digit_peers(uint32_t d, bool v) {
 // (windows aligned to bit 0 would leave the first pass one or two digits:
 // every id's atomic on the same counters); the last window holds the bits
 // that remain.  Each lane keeps eight loads in flight.
-__device__ uint32_t select8(const uint32_t* __restrict__ ids, uint32_t n, uint32_t rank, int top, uint32_t* cnt,
+__device__ __noinline__ uint32_t select8(const uint32_t* __restrict__ ids, uint32_t n, uint32_t rank, int top, uint32_t* cnt,
                             int lane) {
     uint32_t prefix = 0, want = rank;
+#pragma unroll 1
     for (int lo = top - 7;; lo -= 8) {
         const int sh = lo > 0 ? lo : 0;
         const int width = lo >= 0 ? 8 : 8 + lo;        // bits of this window
@@ -200,6 +203,7 @@ __device__ uint32_t select8(const uint32_t* __restrict__ ids, uint32_t n, uint32
 #pragma unroll
         for (int k = 0; k < 8; ++k) cnt[lane * 8 + k] = 0u;
         __syncwarp();
+#pragma unroll 1
         for (uint32_t q0 = 0; q0 < n; q0 += 256) {
             uint32_t x[8];
 #pragma unroll
@@ -247,6 +251,7 @@ __device__ uint32_t select8(const uint32_t* __restrict__ ids, uint32_t n, uint32
         if (sh == 0) break;
     }
     uint32_t pos = SENTINEL;
+#pragma unroll 1
     for (uint32_t q0 = 0; q0 < n; q0 += 256) {
         uint32_t x[8];
 #pragma unroll
@@ -289,6 +294,7 @@ __device__ void radix_pass(const uint32_t* sk, const uint32_t* sv, uint32_t* dk,
 #pragma unroll
     for (int k = 0; k < 8; ++k) c[lane * 8 + k] = 0u;
     __syncwarp();
+#pragma unroll 1
     for (uint32_t g = q0; g < q1; g += 32) {
         const uint32_t q = g + lane;
         const uint32_t d = q < q1 ? (sk[q] >> sh) & 255u : 256u;
@@ -341,6 +347,7 @@ __device__ void radix_pass(const uint32_t* sk, const uint32_t* sv, uint32_t* dk,
     }
     unsigned lt;
     asm("mov.u32 %0, %%lanemask_lt;" : "=r"(lt));
+#pragma unroll 1
     for (uint32_t g = q0; g < q1; g += 32) {
         const uint32_t q = g + lane;
         const bool in = q < q1;
@@ -369,6 +376,7 @@ __device__ void radix_table(uint32_t n, int top, uint32_t* xk, uint32_t* xv, uin
                             uint32_t* table, int nw, uint32_t* cnt, uint32_t* tot, uint32_t tid, int lane, int w) {
     const int passes = top / 8 + 1;
     const uint32_t *sk = xk, *sv = nullptr;
+#pragma unroll 1
     for (int p = 0; p < passes; ++p) {
         const bool last = p + 1 == passes;
         uint32_t* dk = last ? nullptr : ((p & 1) ? xk : yk);
@@ -437,129 +445,102 @@ __global__ void __launch_bounds__(NT) k_rank_tables(const uint32_t* __restrict__
     }
 }
 
-// ids of one cell and species at slots [slot0, slot0 + n); `lookups` rank
-// selections will follow.  sbuf: the warp's four arrays of RANK_WARP_MAX and
-// its 256 counters.
-__device__ __forceinline__ void load_ids(IdList& L, const uint32_t* __restrict__ ids, uint32_t slot0, uint32_t n,
-                                         uint32_t lookups, const RankScratch& S, uint32_t* sbuf, int lane,
-                                         int id_top, bool want_table = false) {
-    const uint32_t* base = ids + slot0;
-    L.n = n;
-    L.table = nullptr;
-    L.base = base;
-    L.cnt = sbuf + 4 * RANK_WARP_MAX;
-    L.cached = n <= 32u * RC;
-    L.sorted = false;
-    L.sel8 = false;
-    L.top = 0;
-    if (!want_table && !L.cached && lookups <= SELECT_LOOKUPS) {
-        L.sel8 = true;
-        L.top = id_top;
-        return;
-    }
-    if (!L.cached) {                 // table built by k_rank_tables
-        L.table = S.table + slot0;
-        return;
-    }
+// Ranks of the n <= RANK_WARP_MAX ids at base, `lookups` of which follow, by
+// one warp.  Returns 0 when the ids ascend, 1 when table[0, n) was written, 2 when
+// select8 costs less (never with want_table).  sbuf: four arrays of
+// RANK_WARP_MAX, then 256 counters.  Out of line: one copy serves every list.
+//
+// Costs in instructions: comparing 64 ids about 340 (32: 100), a radix pass 96 +
+// 64 per 32 ids, a select8 pass 130.  A cell's own heavies have neighbouring ids,
+// so that the digits of id - (smallest id), not of the id, decide the passes: a
+// cell of 80 atoms takes one or two instead of four.
+__device__ __noinline__ int rank_list(const uint32_t* __restrict__ base, uint32_t n, uint32_t lookups, uint32_t* table,
+                                      uint32_t* sbuf, int id_top, bool want_table) {
+    const uint32_t lane = threadIdx.x & 31u;
     uint32_t* xk = sbuf;
-    bool asc = true;
-    uint32_t orv = 0;
-    if (L.cached) {
+    uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+    const uint32_t n4 = (n + 127u) & ~127u;
+    __syncwarp();                                // the buffer's last readers are done
+#pragma unroll 1
+    for (uint32_t q0 = 0; q0 < n4; q0 += 128) {
+        uint32_t x[4];
 #pragma unroll
-        for (int k = 0; k < RC; ++k) {
-            const uint32_t q = (uint32_t)lane + 32u * k;
-            L.ids[k] = q < n ? base[q] : 0u;
-            orv |= L.ids[k];
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t q = q0 + 32u * k + lane;
+            x[k] = q < n ? base[q] : 0xFFFFFFFFu;
         }
 #pragma unroll
-        for (int k = 0; k < RC; ++k) {
-            // element q + 1 is lane + 1 of the same row, or lane 0 of the next
-            const uint32_t q = (uint32_t)lane + 32u * k;
-            const uint32_t right = __shfl_down_sync(FULL, L.ids[k], 1);
-            const uint32_t wrap = __shfl_sync(FULL, k + 1 < RC ? L.ids[k + 1 < RC ? k + 1 : k] : 0u, 0);
-            const uint32_t next = lane == 31 ? wrap : right;
-            if (q + 1 < n && !(L.ids[k] < next)) asc = false;
-        }
-        orv = __reduce_or_sync(FULL, orv);
-        L.top = orv ? 31 - __clz((int)orv) : 0;
-        L.sorted = __all_sync(FULL, asc);
-        if (L.sorted) return;
-        if (n <= 64u) {
-            // a short list's table by comparison: the rank of an id is the
-            // number of smaller ids (ids are unique), 32 exchanges per row
-            uint32_t r0 = 0, r1 = 0;
-            if (n <= 32u) {
-#pragma unroll 8
-                for (int j = 0; j < 32; ++j) {
-                    const uint32_t a = __shfl_sync(FULL, L.ids[0], j);
-                    r0 += ((uint32_t)j < n && a < L.ids[0]) ? 1u : 0u;
-                }
-            } else {
-#pragma unroll 8
-                for (int j = 0; j < 32; ++j) {
-                    const uint32_t a = __shfl_sync(FULL, L.ids[0], j), b = __shfl_sync(FULL, L.ids[1], j);
-                    const bool vb = 32u + (uint32_t)j < n;
-                    r0 += (a < L.ids[0] ? 1u : 0u) + (vb && b < L.ids[0] ? 1u : 0u);
-                    r1 += (a < L.ids[1] ? 1u : 0u) + (vb && b < L.ids[1] ? 1u : 0u);
-                }
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t q = q0 + 32u * k + lane;
+            xk[q] = x[k];                        // (ids are below 2^32 - 1: the rest sorts last)
+            if (q < n) {
+                lo = min(lo, x[k]);
+                hi = max(hi, x[k]);
             }
-            uint32_t* table = S.table + slot0;
-            if ((uint32_t)lane < n) table[r0] = (uint32_t)lane;
-            if (32u + (uint32_t)lane < n) table[r1] = 32u + (uint32_t)lane;
-            __syncwarp();
-            L.table = table;
-            L.cached = false;
-            return;
-        }
-        // a select sweeps the registers once per significant bit, per lookup
-        // (about 48 instructions a bit); the table takes a radix pass per
-        // 8-bit digit (about 96 plus 64 per 32 ids)
-        const uint32_t sel_cost = lookups * (uint32_t)(L.top + 1) * 48u;
-        const uint32_t tab_cost = (uint32_t)(L.top / 8 + 1) * (96u + ((n + 31u) / 32u) * 64u);
-        if (!want_table && sel_cost <= tab_cost) return;
-#pragma unroll
-        for (int k = 0; k < RC; ++k) {
-            const uint32_t q = (uint32_t)lane + 32u * k;
-            if (q < n) xk[q] = L.ids[k];
         }
     }
     __syncwarp();
-    uint32_t* table = S.table + slot0;
-    radix_table<false>(n, L.top, xk, sbuf + RANK_WARP_MAX, sbuf + 2 * RANK_WARP_MAX, sbuf + 3 * RANK_WARP_MAX, table,
-                       1, sbuf + 4 * RANK_WARP_MAX, nullptr, (uint32_t)lane, lane, 0);
-    L.table = table;                 // ordered for the warp by radix_pass's final __syncwarp
-    L.cached = false;
+    bool asc = true;
+#pragma unroll 1
+    for (uint32_t q = lane; q + 1 < n; q += 32)
+        if (!(xk[q] < xk[q + 1])) asc = false;
+    if (__all_sync(FULL, asc)) return 0;
+    lo = __reduce_min_sync(FULL, lo);
+    hi = __reduce_max_sync(FULL, hi);
+    const int top = hi > lo ? 31 - __clz((int)(hi - lo)) : 0;
+    const uint32_t passes = (uint32_t)(top / 8 + 1);
+    if (n <= 32u || (n <= 64u && passes > 1u)) {
+        const uint4* x4 = reinterpret_cast<const uint4*>(xk);
+        const uint32_t a = xk[lane], b = xk[32u + lane];
+        uint32_t r0 = 0, r1 = 0;
+#pragma unroll 1
+        for (uint32_t j = 0; 4u * j < n; ++j) {
+            const uint4 v = x4[j];
+            r0 += (v.x < a ? 1u : 0u) + (v.y < a ? 1u : 0u) + (v.z < a ? 1u : 0u) + (v.w < a ? 1u : 0u);
+            if (n > 32u)
+                r1 += (v.x < b ? 1u : 0u) + (v.y < b ? 1u : 0u) + (v.z < b ? 1u : 0u) + (v.w < b ? 1u : 0u);
+        }
+        if (lane < n) table[r0] = lane;
+        if (32u + lane < n) table[r1] = 32u + lane;
+        __syncwarp();
+        return 1;
+    }
+    const uint32_t tab_cost = passes * (96u + ((n + 31u) / 32u) * 64u);
+    if (!want_table && lookups * (uint32_t)(id_top / 8 + 2) * 130u < tab_cost) return 2;
+#pragma unroll 1
+    for (uint32_t q = lane; q < n; q += 32) xk[q] -= lo;
+    __syncwarp();
+    radix_table<false>(n, top, xk, sbuf + RANK_WARP_MAX, sbuf + 2 * RANK_WARP_MAX, sbuf + 3 * RANK_WARP_MAX, table, 1,
+                       sbuf + 4 * RANK_WARP_MAX, nullptr, lane, (int)lane, 0);
+    return 1;                                    // ordered for the warp by radix_pass's final __syncwarp
 }
 
-// position of the rank-th smallest id of the list
-__device__ __forceinline__ uint32_t select_rank_list(const IdList& L, uint32_t rank, int lane) {
-    if (L.sorted) return rank;
-    if (L.table) return L.table[rank];
-    if (L.sel8) return select8(L.base, L.n, rank, L.top, L.cnt, lane);
-    // register-cached list: bitwise radix select
-    uint32_t prefix = 0, want = rank;
-    for (int bit = L.top; bit >= 0; --bit) {
-        const uint32_t hm = bit == 31 ? 0u : (0xFFFFFFFFu << (bit + 1));
-        uint32_t cnt = 0;
-#pragma unroll
-        for (int k = 0; k < RC; ++k) {
-            const uint32_t q = (uint32_t)lane + 32u * k;
-            cnt += (q < L.n && (L.ids[k] & hm) == prefix && !((L.ids[k] >> bit) & 1u)) ? 1u : 0u;
-        }
-        cnt = __reduce_add_sync(FULL, cnt);
-        if (want >= cnt) {
-            want -= cnt;
-            prefix |= 1u << bit;
-        }
+// ids of one cell and species at slots [slot0, slot0 + n), `lookups` rank
+// selections to follow; stab: where a table of the warp's own goes
+__device__ __forceinline__ void load_ids(IdList& L, const uint32_t* __restrict__ ids, uint32_t slot0, uint32_t n,
+                                         uint32_t lookups, const RankScratch& S, uint32_t* sbuf, uint32_t* stab,
+                                         int id_top, bool want_table = false) {
+    L.n = n;
+    L.base = ids + slot0;
+    L.top = id_top;
+    L.table = nullptr;
+    L.sorted = false;
+    if (n > 32u * RC) {
+        // a table built by k_rank_tables, or few lookups
+        if (want_table || lookups > SELECT_LOOKUPS) L.table = S.table + slot0;
+        return;
     }
-    uint32_t pos = SENTINEL;
-#pragma unroll
-    for (int k = 0; k < RC; ++k) {
-        const uint32_t q = (uint32_t)lane + 32u * k;
-        if (q < L.n && L.ids[k] == prefix) pos = q;
-    }
-    return __reduce_min_sync(FULL, pos);
+    const int how = rank_list(L.base, n, lookups, stab, sbuf, id_top, want_table);
+    L.sorted = how == 0;
+    if (how == 1) L.table = stab;
 }
+
+// A cell of this many candidates is taken by a block of k_collide: one warp would
+// still be at it when all others are done (candidates go with the square of the
+// density: 1300 in one cell where the average has three; 920 us with a warp, 541
+// with a block; lines at 64, 128 and 256 within 3 % of each other).
+constexpr uint32_t BIG_CELL = 256;
+constexpr uint32_t BIG_FLAG = 0x80000000u;      // (cells are below 2^24)
 
 // Heavy cells (a list the warp must sort or many candidates) go to the
 // front of `active`, the others to its back, so that k_collide starts them
@@ -681,7 +662,7 @@ __global__ void __launch_bounds__(256) k_ncand(const uint32_t* __restrict__ cnt,
         if (ml && lane == __ffs(ml) - 1) bl = atomicAdd(&st->n_light, (uint32_t)__popc(ml));
         if (mh) bh = __shfl_sync(FULL, bh, __ffs(mh) - 1);
         if (ml) bl = __shfl_sync(FULL, bl, __ffs(ml) - 1);
-        if (heavy) active[bh + __popc(mh & lt)] = c;
+        if (heavy) active[bh + __popc(mh & lt)] = ntot >= BIG_CELL ? c | BIG_FLAG : c;
         else if (act) active[C - 1u - (bl + __popc(ml & lt))] = c;
         if (act || (c < C && ncoul > 0)) {
             // the lists k_collide or k_coulomb will rank that need a block's
@@ -698,38 +679,6 @@ __global__ void __launch_bounds__(256) k_ncand(const uint32_t* __restrict__ cnt,
     }
 }
 
-struct CellCtx {
-    uint32_t cell;                   // global cell
-    const RunInfo* RI;
-    int geom;
-    unsigned long long slot0;        // first reserved spawn slot
-    uint32_t nres;                   // reserved slots
-    uint32_t id0;                    // id of the first reserved slot
-    uint32_t s;                      // spawned so far
-    uint32_t ev[NCH], nulls, consumed, thr, viol, fb;
-    uint32_t coul_ee, coul_ei, coul_ii;   // Coulomb pair collisions applied
-};
-
-__device__ bool spawn_electron(Particles& A, CellCtx& cx, DevState* st, long long* rho_e, uint32_t gcell, float pz,
-                               float pr, const V3& v) {
-    if (cx.s >= cx.nres) {
-        set_error(st, ERR_BOUNDS);
-        return false;
-    }
-    const unsigned long long slot = cx.slot0 + cx.s;
-    A.key[slot] = make_key(SP_E, gcell);
-    A.pz[slot] = pz;
-    A.pr[slot] = pr;
-    A.vz[slot] = v.x;
-    A.vr[slot] = v.y;
-    A.vt[slot] = v.z;
-    A.id[slot] = cx.id0 + cx.s;
-    ++cx.s;
-    deposit1(rho_e, *cx.RI, cx.geom, gcell - cx.RI->cell_base, pz, pr, -1);
-    return true;
-}
-
-// lane-0 part of one candidate after the pair is chosen
 // cross sections of a pair: running sums cum[] of the class's channels at
 // the pair's relative energy, and sigma_T g
 struct PairEval {
@@ -765,88 +714,6 @@ __device__ __forceinline__ PairEval evaluate_pair(int k, const V3& ve, const V3&
     return e;
 }
 
-// (tkey, ve, vt: the target's key and both velocities as they are now; ev:
-// evaluate_pair of ve, vt)
-// (accepted: the candidate is known to pass the target and acceptance
-// tests, already counted by the caller)
-__device__ void process_candidate(Particles& A, CellCtx& cx, Stream& rs, int k, uint32_t ie, uint32_t it,
-                                  uint32_t tkey, V3 ve, V3 vt, const PairEval& ev, float Racc, float Rch,
-                                  const float* __restrict__ xsE, const float* __restrict__ xs,
-                                  const CollConsts& cc, DevState* st, long long* rho_e, long long* rho_h,
-                                  bool accepted) {
-    const int ts = class_target(k);
-    if (!accepted && ((tkey & KEY_FLAG) || (int)key_species(tkey) != ts)) {   // target already ionized this step
-        ++cx.consumed;
-        return;
-    }
-    const int ch0 = class_ch0(k);
-    const int nch = k == 0 ? 4 : 1;
-    const float* cum = ev.cum;
-    const float sT = cum[nch - 1];
-    const float sg = ev.sg;
-    if (!accepted) {
-        if (sg > cc.sgmax[k]) ++cx.viol;
-        if (!(Racc * cc.sgmax[k] < sg)) {
-            ++cx.nulls;
-            return;
-        }
-    }
-    const float r = Rch * sT;
-    int q = -1;
-    for (int a = 0; a < nch; ++a)
-        if (r < cum[a]) {
-            q = a;
-            break;
-        }
-    if (q < 0) {
-        q = nch - 1;
-        for (int a = nch - 1; a >= 0; --a)
-            if (cum[a] > (a ? cum[a - 1] : 0.0f)) {
-                q = a;
-                break;
-            }
-    }
-    const int ch = ch0 + q;
-    if (ch == CH_EL || ch == CH_EXC) {
-        if (!binary_scatter(rs, ve, vt, ch == CH_EL ? 0.0f : cc.kth[ch], cc.a_e, cc.a_t, cx.fb)) {
-            ++cx.thr;
-            return;
-        }
-        A.vz[ie] = ve.x; A.vr[ie] = ve.y; A.vt[ie] = ve.z;
-        A.vz[it] = vt.x; A.vr[it] = vt.y; A.vt[it] = vt.z;
-        ++cx.ev[ch];
-        return;
-    }
-    // Stage 1, Eq. (12): e + A -> e1 + A*, losing the threshold energy
-    if (!binary_scatter(rs, ve, vt, cc.kth[ch], cc.a_e, cc.a_t, cx.fb)) {
-        ++cx.thr;
-        return;
-    }
-    // Stage 2, Eq. (13): A* -> e2 + ion with the position and velocity of A*
-    V3 e2 = vt;
-    // Stage 3, Eq. (14): e1 + e2 elastic, equal masses
-    binary_scatter(rs, ve, e2, 0.0f, 0.5f, 0.5f, cx.fb);
-    const int new_sp = ch == CH_SI ? SP_CUP : ch == CH_SW ? SP_CU2_SW : ch == CH_DI ? SP_CU2_DI
-                     : ch == CH_S3 ? SP_CU3 : SP_CU4;
-    const int dq = charge_of(new_sp) - charge_of(ts);
-    V3 keep = ve, e6{0.0f, 0.0f, 0.0f};
-    if (ch == CH_DI) {
-        // Stage 4, Eq. (15): e3 -> e5 + e6 (velocity rectangle)
-        V3 e5;
-        rectangle_split(rs, ve, e5, e6, cc.di_split_mode, cx.fb);
-        keep = e5;
-    }
-    A.vz[ie] = keep.x; A.vr[ie] = keep.y; A.vt[ie] = keep.z;
-    A.vz[it] = vt.x; A.vr[it] = vt.y; A.vt[it] = vt.z;
-    const uint32_t tcell = key_cell(tkey);
-    A.key[it] = converted_key((uint32_t)new_sp, (uint32_t)ts, tcell);
-    const float tpz = A.pz[it], tpr = A.pr[it];
-    deposit1(rho_h, *cx.RI, cx.geom, tcell - cx.RI->cell_base, tpz, tpr, dq);
-    spawn_electron(A, cx, st, rho_e, tcell, tpz, tpr, e2);
-    if (ch == CH_DI) spawn_electron(A, cx, st, rho_e, key_cell(A.key[ie]), A.pz[ie], A.pr[ie], e6);
-    ++cx.ev[ch];
-}
-
 // a pair whose particles are no longer what its class draws: a target
 // ionized earlier this step or, for the heavy classes, a Cu that was
 __device__ __forceinline__ bool consumed_pair(int k, uint32_t akey, uint32_t tkey) {
@@ -856,35 +723,104 @@ __device__ __forceinline__ bool consumed_pair(int k, uint32_t akey, uint32_t tke
     return t_gone || (akey & KEY_FLAG) || (int)key_species(akey) != SP_CU;
 }
 
-// lane-0 part of one heavy-pair candidate (classes 5 and 6: one channel
-// each, nothing spawned), the counterpart of process_candidate.  Charge
-// exchange Cu + Cu+ -> Cu+ + Cu moves the electron, not the atoms: each slot
-// keeps its species and takes the other's velocity.  Cu + Cu is elastic and
-// isotropic in the centre of mass, equal masses.
-__device__ void process_heavy_pair(Particles& A, CellCtx& cx, Stream& rs, int k, uint32_t ia, uint32_t ib,
-                                   uint32_t akey, uint32_t bkey, V3 va, V3 vb, const PairEval& ev, float Racc,
-                                   const CollConsts& cc, bool accepted) {
-    if (!accepted) {
-        if (consumed_pair(k, akey, bkey)) {
-            ++cx.consumed;
-            return;
-        }
-        if (ev.sg > cc.sgmax[k]) ++cx.viol;
-        if (!(Racc * cc.sgmax[k] < ev.sg)) {
-            ++cx.nulls;
-            return;
-        }
+// What became of a candidate: a channel's event (its channel), or one of these
+// (indices of a warp's counters).
+enum { OUT_NULL = NCH, OUT_CONSUMED, OUT_THR, OUT_VIOL, OUT_FB, OUT_N };
+constexpr int COLL_WARPS = 4;                   // warps of a k_collide block
+constexpr int COLL_SORT_WORDS = 4 * RANK_WARP_MAX + 256;
+constexpr uint32_t CLAIMS = 4 * RANK_WARP_MAX;  // places of a block's claim tables (in the rank buffers of its warps 1 and 2)
+// a spawned electron (its position is a particle's of the pair)
+struct Spawn {
+    uint32_t cell;
+    float pz, pr;
+    V3 v;
+};
+
+// One candidate of class k on particles ie (electron, or Cu of a heavy pair) and
+// it, by its lane: target and acceptance tests, channel, kinematics, the
+// particles' new state and the target's charge.  Returns the outcome; `viol`: the
+// pair broke the majorant; the electrons it makes (nsp of them, in order) go to
+// sp[], to be placed by the caller in candidate order.
+template <bool EXT>
+__device__ __forceinline__ int collide_pair(Particles& A, int k, uint32_t ie, uint32_t it, uint32_t lc, uint32_t m,
+                                            float Racc, float Rch, const RunInfo* RI, int geom,
+                                            const float* __restrict__ xsE, const float* __restrict__ xs,
+                                            const CollConsts& cc, const DevState* st, long long* rho_h, bool& viol,
+                                            uint32_t& fb, int& nsp, Spawn (&sp)[2]) {
+    const uint32_t tkey = A.key[it];
+    const uint32_t akey = EXT && k >= NECLS ? A.key[ie] : 0u;
+    V3 ve{A.vz[ie], A.vr[ie], A.vt[ie]}, vt{A.vz[it], A.vr[it], A.vt[it]};
+    const PairEval ev = evaluate_pair(k, ve, vt, xsE, xs, cc);
+    if (consumed_pair(k, akey, tkey)) return OUT_CONSUMED;       // ionized (or charged) earlier this step
+    viol = ev.sg > cc.sgmax[k];
+    if (!(Racc * cc.sgmax[k] < ev.sg)) return OUT_NULL;
+    if (EXT && k == 5) {
+        // charge exchange Cu + Cu+ -> Cu+ + Cu moves the electron, not the
+        // atoms: each slot keeps its species and takes the other's velocity
+        A.vz[ie] = vt.x; A.vr[ie] = vt.y; A.vt[ie] = vt.z;
+        A.vz[it] = ve.x; A.vr[it] = ve.y; A.vt[it] = ve.z;
+        return CH_CX;
     }
-    if (k == 5) {
-        A.vz[ia] = vb.x; A.vr[ia] = vb.y; A.vt[ia] = vb.z;
-        A.vz[ib] = va.x; A.vr[ib] = va.y; A.vt[ib] = va.z;
-        ++cx.ev[CH_CX];
-        return;
+    // channel: the first whose running sum exceeds Rch sigma_T (else the last
+    // with a cross section)
+    const int nch = k == 0 ? 4 : 1;
+    const float r = Rch * ev.cum[3];
+    int q = -1, last = nch - 1;
+#pragma unroll
+    for (int a = 3; a >= 0; --a)
+        if (a < nch && r < ev.cum[a]) q = a;
+    if (q < 0) {
+        bool found = false;
+#pragma unroll
+        for (int a = 3; a >= 0; --a)
+            if (!found && a < nch && ev.cum[a] > (a ? ev.cum[a > 0 ? a - 1 : 0] : 0.0f)) {
+                last = a;
+                found = true;
+            }
+        q = last;
     }
-    binary_scatter(rs, va, vb, 0.0f, 0.5f, 0.5f, cx.fb);
-    A.vz[ia] = va.x; A.vr[ia] = va.y; A.vt[ia] = va.z;
-    A.vz[ib] = vb.x; A.vr[ib] = vb.y; A.vt[ib] = vb.z;
-    ++cx.ev[CH_NN];
+    const int ch = class_ch0(k) + q;
+    const bool ionizes = ch != CH_EL && ch != CH_EXC && ch != CH_NN;
+    // the candidate's stream after its four pair-choice draws
+    StreamOf<true> rs(lc, st->step, sid_cand(k, m), RI->seed, RI->run);
+    rs.ctr.w = 1u;
+    // Stage 1, Eq. (12): the pair scatters and loses the channel's energy (a Cu
+    // pair elastically, equal masses); stage 3, Eq. (14), of an ionization: e1 + e2
+    // elastic, e2 born with the velocity of A* (stage 2, Eq. (13))
+    V3 a = ve, b = vt;
+    float kth = ch == CH_EL || ch == CH_NN ? 0.0f : cc.kth[ch];
+    float a1 = ch == CH_NN ? 0.5f : cc.a_e, a2 = ch == CH_NN ? 0.5f : cc.a_t;
+#pragma unroll 1
+    for (int stage = 0;; ++stage) {
+        if (!binary_scatter(rs, a, b, kth, a1, a2, fb)) return OUT_THR;
+        if (stage == 0) vt = b;
+        if (stage == 1 || !ionizes) break;
+        kth = 0.0f;
+        a1 = a2 = 0.5f;
+    }
+    ve = a;
+    if (ionizes) {
+        const uint32_t tcell = key_cell(tkey);
+        const int ts = class_target(k);
+        const int new_sp = ch == CH_SI ? SP_CUP : ch == CH_SW ? SP_CU2_SW : ch == CH_DI ? SP_CU2_DI
+                         : ch == CH_S3 ? SP_CU3 : SP_CU4;
+        const float tpz = A.pz[it], tpr = A.pr[it];
+        sp[0] = Spawn{tcell, tpz, tpr, b};
+        nsp = 1;
+        if (ch == CH_DI) {
+            // Stage 4, Eq. (15): e3 -> e5 + e6 (velocity rectangle)
+            V3 e5, e6;
+            rectangle_split(rs, ve, e5, e6, cc.di_split_mode, fb);
+            sp[1] = Spawn{key_cell(A.key[ie]), A.pz[ie], A.pr[ie], e6};
+            nsp = 2;
+            ve = e5;
+        }
+        A.key[it] = converted_key((uint32_t)new_sp, (uint32_t)ts, tcell);
+        deposit1(rho_h, *RI, geom, tcell - RI->cell_base, tpz, tpr, charge_of(new_sp) - charge_of(ts));
+    }
+    A.vz[ie] = ve.x; A.vr[ie] = ve.y; A.vt[ie] = ve.z;
+    A.vz[it] = vt.x; A.vr[it] = vt.y; A.vt[it] = vt.z;
+    return ch;
 }
 
 // ---------------------------------------------------------------------
@@ -1123,7 +1059,7 @@ __global__ void __launch_bounds__(128, 6) k_coulomb(Particles A, RankScratch S, 
                                                    const uint32_t* __restrict__ cnt, DevState* st, KParams P,
                                                    CollConsts cc, const double* __restrict__ cw) {
     if (st->error) return;                           // a fault was flagged: the state is not stepped further
-    __shared__ uint32_t s_sort[COUL_WARPS][COUL_SBUF];   // per-warp rank-table sort, then velocity cache
+    __shared__ __align__(16) uint32_t s_sort[COUL_WARPS][COUL_SBUF];   // per-warp rank-table sort, then velocity cache
     __shared__ CoulWarp s_cw[COUL_WARPS];
     const int lane = threadIdx.x & 31;
     const int wib = (threadIdx.x >> 5) & (COUL_WARPS - 1);
@@ -1223,7 +1159,7 @@ __global__ void __launch_bounds__(128, 6) k_coulomb(Particles A, RankScratch S, 
             if (!u) continue;
             tot += n;
             IdList L;
-            load_ids(L, A.id, b, n, n, S, sbuf, lane, id_top, true);
+            load_ids(L, A.id, b, n, n, S, sbuf, S.table + b, id_top, true);
             if (L.sorted) sorted |= 1u << l;
         }
         if (lane == 0) W.sorted = sorted;
@@ -1358,73 +1294,141 @@ __global__ void __launch_bounds__(128, 6) k_coulomb(Particles A, RankScratch S, 
     }
 }
 
+// position of the rank-th smallest id for each lane's rank (lanes with has)
+__device__ __forceinline__ uint32_t lookup_ranks(const IdList& L, uint32_t rank, bool has, uint32_t nb, uint32_t* cnt,
+                                                 int lane) {
+    if (L.sorted) return rank;
+    if (L.table) return has ? L.table[rank] : 0u;
+    uint32_t pos = 0;
+#pragma unroll 1
+    for (uint32_t q = 0; q < nb; ++q) {
+        const uint32_t p = select8(L.base, L.n, __shfl_sync(FULL, rank, (int)q), L.top, cnt, lane);
+        if ((uint32_t)lane == q) pos = p;
+    }
+    return pos;
+}
+
+// One warp per active cell, or a block per cell of BIG_CELL candidates or more.
+// What bounds it is neither memory nor arithmetic but the instruction caches, the
+// latency of a cell's dependent loads and the largest cell.  Unrolled over the
+// classes, with the rank code and the kinematics inlined at every use and the
+// accepted candidates applied one by one on lane 0, the kernel was 132 KB long and
+// waited for instructions half of the time.  Now each part has one copy
+// (rank_list, select8 and the Philox rounds out of line, one loop over the classes,
+// one over the candidates to apply; no spills to speak of: at 96 registers and five
+// blocks an SM it is slower), and the candidates of a batch are applied in rounds.
+// 256 x 512 cells, 4e5 candidates in 1.2e5 cells, the largest with 1300: 2290 ->
+// 920 us with one copy of each part, 541 us with the large cells on blocks, then
+// evenly spread over the SMs (at 38 % of the issue slots, 16 warps an SM).  Plume
+// of 2e7 particles: 214 -> 145 us.
 template <bool EXT>
-__global__ void __launch_bounds__(128, 3) k_collide(Particles A, RankScratch S, const uint32_t* __restrict__ off,
-                                                 const uint32_t* __restrict__ cnt,
-                                                 const uint4* __restrict__ nc, const uint4* __restrict__ nc2,
-                                                 const uint32_t* __restrict__ cand_off,
-                                                 const uint32_t* __restrict__ active, DevState* st, long long* rho_e,
-                                                 long long* rho_h, const float* __restrict__ xsE,
-                                                 const float* __restrict__ xs, const double* __restrict__ cw,
-                                                 KParams P, CollConsts cc, uint32_t nbins) {
+__global__ void __launch_bounds__(32 * COLL_WARPS, 4) k_collide(
+    Particles A, RankScratch S, const uint32_t* __restrict__ off, const uint32_t* __restrict__ cnt,
+    const uint4* __restrict__ nc, const uint4* __restrict__ nc2, const uint32_t* __restrict__ cand_off,
+    const uint32_t* __restrict__ active, DevState* st, long long* rho_e, long long* rho_h,
+    const float* __restrict__ xsE, const float* __restrict__ xs, KParams P, CollConsts cc, uint32_t big_blocks) {
     if (st->error) return;                           // a fault was flagged: the state is not stepped further
-    __shared__ uint32_t s_sort[4][4 * RANK_WARP_MAX + 256];   // per-warp rank-table sort
-    const int lane = threadIdx.x & 31;
-    uint32_t* sbuf = s_sort[(threadIdx.x >> 5) & 3];
+    __shared__ __align__(16) uint32_t s_sort[COLL_WARPS][COLL_SORT_WORDS + 2 * RANK_WARP_MAX];
+    __shared__ uint32_t s_ctr[COLL_WARPS][OUT_N];
+    __shared__ uint32_t s_nsp[COLL_WARPS];           // electrons each warp of a block's batch made
+    __shared__ int s_how[2];                         // how the cell's lists are ranked (rank_list by warp 0)
+    const int lane = threadIdx.x & 31, wib = (threadIdx.x >> 5) & (COLL_WARPS - 1);
+    uint32_t* ctr = s_ctr[wib];
+    if (lane < OUT_N) ctr[lane] = 0u;
+    __syncwarp();
     const uint32_t C = P.ncell;
     const uint32_t n_heavy = st->n_heavy, n_light = st->n_light;
     const uint32_t n_alive = (uint32_t)st->tail_base;   // spawn slots follow the bins
-    // heavy cells first, taken one at a time from a shared cursor by the
-    // first min(n_heavy, warps) warps; then the light cells, warp-strided
+    // a counter's place in RunState::ctr
+    auto flush = [&](int r) {
+        __syncwarp();
+        if (lane < OUT_N && ctr[lane]) {
+            const int c = lane < NCH ? c_event(lane) : lane == OUT_NULL ? C_NULL : lane == OUT_CONSUMED ? C_CONSUMED
+                        : lane == OUT_THR ? C_THR : lane == OUT_VIOL ? C_VIOL : C_ISOFB;
+            atomicAdd(&P.rs[r].ctr[c], (unsigned long long)ctr[lane]);
+            ctr[lane] = 0u;
+        }
+        __syncwarp();
+    };
+    // The big cells first, a block each: the first blocks (those resident from
+    // the start) look for them among the heavy ones.  Then the other heavy cells,
+    // taken one at a time from a shared cursor by the first min(n_heavy, warps)
+    // warps, and the light cells, warp-strided.
     const uint32_t warp0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
     bool heavy_phase = warp0 < n_heavy;
-    uint32_t wl = warp0;
+    uint32_t wl = warp0, wb = blockIdx.x < big_blocks ? blockIdx.x : n_heavy;
+    uint32_t tag = 0;                                // rounds of the block so far
     for (;;) {
+        bool blk = false;                            // (the same in all warps of the block while there are big cells)
         uint32_t c = 0;
-        if (heavy_phase) {
+        while (wb < n_heavy && !blk) {
+            c = active[wb];
+            wb += big_blocks;
+            blk = (c & BIG_FLAG) != 0u;
+        }
+        c &= ~BIG_FLAG;
+        if (!blk && heavy_phase) {
             uint32_t w = 0;
             if (lane == 0) w = atomicAdd(&st->collide_next, 1u);
             w = __shfl_sync(FULL, w, 0);
-            if (w < n_heavy) c = active[w];
-            else heavy_phase = false;
+            if (w < n_heavy) {
+                c = active[w];
+                if (c & BIG_FLAG) continue;
+            } else {
+                heavy_phase = false;
+            }
         }
-        if (!heavy_phase) {
+        if (!blk && !heavy_phase) {
             if (wl >= n_light) break;
             c = active[C - 1u - wl];
             wl += nwarps;
         }
+        // the group that takes the cell: this warp, or the block (with warp 0's buffers)
+        const uint32_t GS = blk ? 32u * COLL_WARPS : 32u, me = blk ? threadIdx.x : (uint32_t)lane;
+        uint32_t* sbuf = s_sort[blk ? 0 : wib];          // rank_list's buffers and counters,
+        uint32_t* tab0 = sbuf + COLL_SORT_WORDS;         // then the tables of the pair's two lists
+        auto ranks = [&](IdList& L, int which, uint32_t slot0, uint32_t n, uint32_t lookups, int id_top) {
+            if (!blk) {
+                load_ids(L, A.id, slot0, n, lookups, S, sbuf, tab0 + which * RANK_WARP_MAX, id_top);
+                return;
+            }
+            __syncthreads();                             // the buffers' last readers are done
+            if (wib == 0) {
+                load_ids(L, A.id, slot0, n, lookups, S, sbuf, tab0 + which * RANK_WARP_MAX, id_top);
+                if (lane == 0) s_how[which] = L.sorted ? 0 : L.table ? 1 : 2;
+            }
+            __syncthreads();
+            const int how = s_how[which];
+            L.n = n;
+            L.base = A.id + slot0;
+            L.top = id_top;
+            L.sorted = how == 0;
+            L.table = how == 1 ? (n > 32u * RC ? S.table + slot0 : tab0 + which * RANK_WARP_MAX) : nullptr;
+        };
         const uint4 n = nc[c];         // candidates of the classes (e,Cu), (e,Cu+), (Cu,Cu+), (Cu,Cu)
         // and of (e,Cu2+ SW), (e,Cu2+ DI), (e,Cu3+)
         const uint4 n2 = EXT && P.charge_max >= 3 ? nc2[c] : make_uint4(0u, 0u, 0u, 0u);
+        const uint32_t e_base = off[c], Ne = cnt[c], co = cand_off[c];
         const int r = run_of(P, c);
         const RunInfo* RI = &P.runs[r];
         const uint32_t lc = c - RI->cell_base;
-        CellCtx cx;
-        cx.cell = c;
-        cx.RI = RI;
-        cx.geom = P.geom;
-        cx.nres = 2u * (n.x + n.y + n2.x + n2.y + n2.z);
-        cx.slot0 = (unsigned long long)n_alive + 2ull * cand_off[c];
-        // ids: the run's next id plus twice the candidates of the run's earlier cells
-        cx.id0 = P.rs[r].id_next + 2u * (cand_off[c] - cand_off[RI->cell_base]);
-        // every id in the cell's lists is below the run's next id
+        const uint32_t nres = 2u * (n.x + n.y + n2.x + n2.y + n2.z);     // reserved spawn slots
+        const unsigned long long slot0 = (unsigned long long)n_alive + 2ull * co;
+        // ids: the run's next id plus twice the candidates of the run's earlier
+        // cells; every id in the cell's lists is below the run's next id
         const uint32_t idn = P.rs[r].id_next;
+        const uint32_t id0 = idn + 2u * (co - cand_off[RI->cell_base]);
         const int id_top = idn > 1u ? 31 - __clz((int)(idn - 1u)) : 0;
-        cx.s = 0;
-        for (int q = 0; q < NCH; ++q) cx.ev[q] = 0;
-        cx.nulls = cx.consumed = cx.thr = cx.viol = cx.fb = 0;
-        cx.coul_ee = cx.coul_ei = cx.coul_ii = 0;
-        if (cx.slot0 + cx.nres > P.capacity) {
+        uint32_t nspawn = 0;
+        if (slot0 + nres > P.capacity) {
             // no room for this cell's spawns: report, and leave its reserved
             // slots (those that exist) dead
-            if (lane == 0) set_error(st, ERR_CAPACITY);
-            for (unsigned long long q = cx.slot0 + lane; q < P.capacity && q < cx.slot0 + cx.nres; q += 32)
-                A.key[q] = DEAD;
+            if (me == 0) set_error(st, ERR_CAPACITY);
+#pragma unroll 1
+            for (unsigned long long q = slot0 + me; q < P.capacity && q < slot0 + nres; q += GS) A.key[q] = DEAD;
             continue;
         }
-        const uint32_t e_base = off[c];
-        const uint32_t Ne = cnt[c];
         // lookups of each list over all classes (the rank-table decisions of
         // k_ncand use the same totals): the Coulomb pairs look up every
         // electron and every ion of a cell with electrons
@@ -1438,16 +1442,17 @@ __global__ void __launch_bounds__(128, 3) k_collide(Particles A, RankScratch S, 
         IdList el;
         uint32_t a_base = e_base, Na = Ne;
         bool cu_first = false;
-        if (look_e) load_ids(el, A.id, e_base, Ne, look_e, S, sbuf, lane, id_top);
+        if (look_e) ranks(el, 0, e_base, Ne, look_e, id_top);
+#pragma unroll 1
         for (int k = 0; k < (EXT ? NCLS : 2); ++k) {
             const uint32_t ncand = k == 0 ? n.x : k == 1 ? n.y : k == 2 ? n2.x : k == 3 ? n2.y : k == 4 ? n2.z
                                  : k == 5 ? n.z : n.w;
             if (ncand == 0) continue;
-            if (k >= NECLS && !cu_first) {
+            if (EXT && k >= NECLS && !cu_first) {
                 cu_first = true;
                 a_base = off[C + c];
                 Na = cnt[C + c];
-                load_ids(el, A.id, a_base, Na, look_cu, S, sbuf, lane, id_top);
+                ranks(el, 0, a_base, Na, look_cu, id_top);
             }
             const int ts = class_target(k);
             const uint32_t tb = (uint32_t)ts * C + c;
@@ -1456,137 +1461,133 @@ __global__ void __launch_bounds__(128, 3) k_collide(Particles A, RankScratch S, 
             // the target list's lookups over every class that draws from it
             const uint32_t t_look = ts == SP_CU ? look_cu : (ts == SP_CUP ? look_ci : ncand) + (coul ? Nt : 0u);
             IdList tl;
-            load_ids(tl, A.id, t_base, Nt, t_look, S, sbuf, lane, id_top);
-            // candidates in batches of 32: lane q draws candidate m0 + q's pair and
-            // prefetches its particles; lane 0 then applies them in order,
-            // re-reading a candidate whose particles an earlier candidate of
-            // the batch may have changed
-            for (uint32_t m0 = 0; m0 < ncand; m0 += 32) {
-                const uint32_t nb = min(32u, ncand - m0);
-                const bool has = (uint32_t)lane < nb;
+            ranks(tl, 1, t_base, Nt, t_look, id_top);
+            // candidates in batches: thread q of the group draws candidate m0 + q's pair
+#pragma unroll 1
+            for (uint32_t m0 = 0; m0 < ncand; m0 += GS) {
+                const uint32_t nb = min(GS, ncand - m0);
+                const bool has = me < nb;
                 uint32_t i = 0, j = 0;
                 float Racc = 0.0f, Rch = 0.0f;
                 if (has) {
-                    Stream rs(lc, st->step, sid_cand(k, m0 + lane), RI->seed, RI->run);
-                    i = rs.pick(Na);
-                    if (k == 6) {           // a second, different Cu
-                        j = rs.pick(Na - 1u);
+                    const uint4 d = philox_block(make_uint4(lc, st->step, sid_cand(k, m0 + me), 0u),
+                                                 make_uint2(RI->seed, RI->run));
+                    i = (uint32_t)(((unsigned long long)d.x * Na) >> 32);
+                    if (EXT && k == 6) {    // a second, different Cu
+                        j = (uint32_t)(((unsigned long long)d.y * (Na - 1u)) >> 32);
                         if (j >= i) ++j;
                     } else {
-                        j = rs.pick(Nt);
+                        j = (uint32_t)(((unsigned long long)d.y * Nt) >> 32);
                     }
-                    Racc = rs.u01();
-                    Rch = rs.u01();
+                    Racc = __fmul_rn((float)(d.z >> 8), 5.9604644775390625e-08f);
+                    Rch = __fmul_rn((float)(d.w >> 8), 5.9604644775390625e-08f);
                 }
-                uint32_t pe = 0, pt = 0;
-                if (el.sorted) {
-                    pe = i;
-                } else if (el.table) {
-                    if (has) pe = el.table[i];
-                } else {
-                    for (uint32_t q = 0; q < nb; ++q) {
-                        const uint32_t p = select_rank_list(el, __shfl_sync(FULL, i, (int)q), lane);
-                        if ((uint32_t)lane == q) pe = p;
-                    }
-                }
-                if (tl.sorted) {
-                    pt = j;
-                } else if (tl.table) {
-                    if (has) pt = tl.table[j];
-                } else {
-                    for (uint32_t q = 0; q < nb; ++q) {
-                        const uint32_t p = select_rank_list(tl, __shfl_sync(FULL, j, (int)q), lane);
-                        if ((uint32_t)lane == q) pt = p;
-                    }
-                }
+                // (a select works on its own warp's candidates and counters)
+                const uint32_t nw = blk ? (nb > 32u * wib ? min(32u, nb - 32u * wib) : 0u) : nb;
+                uint32_t* scnt = s_sort[wib] + 4 * RANK_WARP_MAX;
+                const uint32_t pe = lookup_ranks(el, i, has, nw, scnt, lane);
+                const uint32_t pt = lookup_ranks(tl, j, has, nw, scnt, lane);
                 const bool ok = has && pe < Na && pt < Nt;   // ids not unique: corrupt state, never index with it
                 if (has && !ok) set_error(st, ERR_BOUNDS);
                 const uint32_t ie = a_base + (ok ? pe : 0u), it = t_base + (ok ? pt : 0u);
-                uint32_t tkey = 0, akey = 0;
-                V3 ve{0.0f, 0.0f, 0.0f}, vt{0.0f, 0.0f, 0.0f};
-                if (ok) {
-                    tkey = A.key[it];
-                    if (k >= NECLS) akey = A.key[ie];
-                    ve = V3{A.vz[ie], A.vr[ie], A.vt[ie]};
-                    vt = V3{A.vz[it], A.vr[it], A.vt[it]};
+                // Applied in rounds: every candidate to apply yet whose earlier
+                // sharers of a particle are all through (no two of a round touch
+                // the same particle), so that each sees its particles as the
+                // sequence leaves them.  A warp compares all pairs of its batch
+                // once; a block lets its candidates claim their particles' places
+                // in two tables each round, the earliest first (two particles
+                // of one place only wait needlessly).  The two particles of a
+                // (Cu, Cu) pair come from one list.
+                uint32_t conf = 0;
+                const uint32_t he = ie & (CLAIMS - 1u), ht = it & (CLAIMS - 1u);
+                uint32_t* te = s_sort[1];
+                uint32_t* tt = EXT && k == 6 ? te : s_sort[2];
+                if (!blk) {
+#pragma unroll 1
+                    for (uint32_t q = 0; q + 1 < nb; ++q) {
+                        const uint32_t e2 = __shfl_sync(FULL, ie, (int)q), t2 = __shfl_sync(FULL, it, (int)q);
+                        if (q < (uint32_t)lane && (e2 == ie || t2 == it || (EXT && k == 6 && (e2 == it || t2 == ie))))
+                            conf |= 1u << q;
+                    }
+                } else if (tag == 0u) {
+                    for (uint32_t q = me; q < CLAIMS; q += GS) s_sort[1][q] = s_sort[2][q] = 0u;
+                    __syncthreads();
                 }
-                // cross sections of every lane's pair, in parallel (redone by
-                // lane 0 for a pair an earlier candidate may have changed)
-                const PairEval ev = evaluate_pair(k, ve, vt, xsE, xs, cc);
-                // dirty: shares a particle with an earlier candidate of the batch
-                // (the two particles of a (Cu, Cu) pair come from one list)
-                bool dirty = false;
-                for (uint32_t q = 0; q + 1 < nb; ++q) {
-                    const uint32_t e2 = __shfl_sync(FULL, ie, (int)q), t2 = __shfl_sync(FULL, it, (int)q);
-                    if (q < (uint32_t)lane && (e2 == ie || t2 == it || (k == 6 && (e2 == it || t2 == ie))))
-                        dirty = true;
-                }
-                // a candidate no earlier one of the batch touches sees the
-                // particles as prefetched: its lane takes the target and
-                // acceptance tests (the same float operations lane 0 would),
-                // and only accepted or touched candidates go through lane 0,
-                // in candidate order
-                const bool cons = consumed_pair(k, akey, tkey);
-                const bool acc = !cons && Racc * cc.sgmax[k] < ev.sg;
-                const bool clean = ok && !dirty;
-                const unsigned m_cons = __ballot_sync(FULL, clean && cons);
-                const unsigned m_viol = __ballot_sync(FULL, clean && !cons && ev.sg > cc.sgmax[k]);
-                const unsigned m_null = __ballot_sync(FULL, clean && !cons && !acc);
-                if (lane == 0) {
-                    cx.consumed += (uint32_t)__popc(m_cons);
-                    cx.viol += (uint32_t)__popc(m_viol);
-                    cx.nulls += (uint32_t)__popc(m_null);
-                }
-                const unsigned todo = __ballot_sync(FULL, ok && (dirty || acc));
-                for (unsigned mq = todo; mq; mq &= mq - 1u) {
-                    const uint32_t q = (uint32_t)(__ffs(mq) - 1);
-                    const bool dq = __shfl_sync(FULL, dirty, (int)q);
-                    const uint32_t ieq = __shfl_sync(FULL, ie, (int)q), itq = __shfl_sync(FULL, it, (int)q);
-                    uint32_t tkq = __shfl_sync(FULL, tkey, (int)q), akq = __shfl_sync(FULL, akey, (int)q);
-                    V3 veq{__shfl_sync(FULL, ve.x, (int)q), __shfl_sync(FULL, ve.y, (int)q),
-                           __shfl_sync(FULL, ve.z, (int)q)};
-                    V3 vtq{__shfl_sync(FULL, vt.x, (int)q), __shfl_sync(FULL, vt.y, (int)q),
-                           __shfl_sync(FULL, vt.z, (int)q)};
-                    const float Ra = __shfl_sync(FULL, Racc, (int)q), Rc = __shfl_sync(FULL, Rch, (int)q);
-                    PairEval evq;
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) evq.cum[e] = __shfl_sync(FULL, ev.cum[e], (int)q);
-                    evq.sg = __shfl_sync(FULL, ev.sg, (int)q);
-                    if (lane == 0) {
-                        if (dq) {
-                            tkq = A.key[itq];
-                            if (k >= NECLS) akq = A.key[ieq];
-                            veq = V3{A.vz[ieq], A.vr[ieq], A.vt[ieq]};
-                            vtq = V3{A.vz[itq], A.vr[itq], A.vt[itq]};
-                            evq = evaluate_pair(k, veq, vtq, xsE, xs, cc);
+                bool pend = ok;
+                int out = -1, nsp = 0;
+                bool viol = false;
+                uint32_t fb = 0;
+                Spawn sp[2];
+                for (;;) {
+                    bool ready;
+                    if (!blk) {
+                        const uint32_t b = __ballot_sync(FULL, pend);
+                        if (!b) break;
+                        ready = pend && !(conf & b);
+                    } else {
+                        // claims of later rounds are larger, of earlier candidates too
+                        ++tag;
+                        const uint32_t v = tag * (32u * COLL_WARPS) + (32u * COLL_WARPS - 1u - me);
+                        if (pend) {
+                            atomicMax(&te[he], v);
+                            atomicMax(&tt[ht], v);
                         }
-                        // the candidate's stream after its four pair-choice draws
-                        Stream rs(lc, st->step, sid_cand(k, m0 + q), RI->seed, RI->run);
-                        rs.ctr.w = 1u;
-                        rs.used = 4;
-                        if (k < NECLS)
-                            process_candidate(A, cx, rs, k, ieq, itq, tkq, veq, vtq, evq, Ra, Rc, xsE, xs, cc, st,
-                                              rho_e, rho_h, !dq);
-                        else
-                            process_heavy_pair(A, cx, rs, k, ieq, itq, akq, tkq, veq, vtq, evq, Ra, cc, !dq);
+                        if (!__syncthreads_or(pend)) break;
+                        ready = pend && te[he] == v && tt[ht] == v;
+                    }
+                    if (ready) {
+                        out = collide_pair<EXT>(A, k, ie, it, lc, m0 + me, Racc, Rch, RI, P.geom, xsE, xs, cc, st,
+                                                rho_h, viol, fb, nsp, sp);
+                        pend = false;
+                    }
+                    if (blk) __syncthreads();
+                    else __syncwarp();
+                }
+                if (out >= 0) atomicAdd(&ctr[out], 1u);
+                if (viol) atomicAdd(&ctr[OUT_VIOL], 1u);
+                if (fb) atomicAdd(&ctr[OUT_FB], fb);
+                // the electrons made, in candidate order
+                const uint32_t b1 = __ballot_sync(FULL, nsp > 0), b2 = __ballot_sync(FULL, nsp > 1);
+                uint32_t made = __popc(b1) + __popc(b2), s0 = nspawn;
+                if (blk) {
+                    if (lane == 0) s_nsp[wib] = made;
+                    __syncthreads();
+                    made = 0;
+#pragma unroll
+                    for (int w = 0; w < COLL_WARPS; ++w) {
+                        if (w < wib) s0 += s_nsp[w];
+                        made += s_nsp[w];
                     }
                 }
-                __syncwarp();
+                nspawn += made;
+                if (b1) {
+                    const uint32_t lt = (1u << lane) - 1u;
+                    s0 += __popc(b1 & lt) + __popc(b2 & lt);
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        if (q >= nsp) continue;
+                        if (s0 + q >= nres) {
+                            set_error(st, ERR_BOUNDS);
+                            continue;
+                        }
+                        const unsigned long long slot = slot0 + s0 + q;
+                        A.key[slot] = make_key(SP_E, sp[q].cell);
+                        A.pz[slot] = sp[q].pz;
+                        A.pr[slot] = sp[q].pr;
+                        A.vz[slot] = sp[q].v.x;
+                        A.vr[slot] = sp[q].v.y;
+                        A.vt[slot] = sp[q].v.z;
+                        A.id[slot] = id0 + s0 + q;
+                        deposit1(rho_e, *RI, P.geom, sp[q].cell - RI->cell_base, sp[q].pz, sp[q].pr, -1);
+                    }
+                }
             }
         }
-        const uint32_t s = __shfl_sync(FULL, cx.s, 0);
-        for (uint32_t q = s + lane; q < cx.nres; q += 32) A.key[cx.slot0 + q] = DEAD;
-        if (lane == 0) {
-            RunState& rsv = P.rs[r];
-            for (int q = 0; q < NCH; ++q)
-                if (cx.ev[q]) atomicAdd(&rsv.ctr[c_event(q)], (unsigned long long)cx.ev[q]);
-            if (cx.nulls) atomicAdd(&rsv.ctr[C_NULL], (unsigned long long)cx.nulls);
-            if (cx.consumed) atomicAdd(&rsv.ctr[C_CONSUMED], (unsigned long long)cx.consumed);
-            if (cx.thr) atomicAdd(&rsv.ctr[C_THR], (unsigned long long)cx.thr);
-            if (cx.viol) atomicAdd(&rsv.ctr[C_VIOL], (unsigned long long)cx.viol);
-            if (cx.fb) atomicAdd(&rsv.ctr[C_ISOFB], (unsigned long long)cx.fb);
-        }
+#pragma unroll 1
+        for (uint32_t q = nspawn + me; q < nres; q += GS) A.key[slot0 + q] = DEAD;
+        if (P.nruns > 1) flush(r);
     }
+    if (P.nruns == 1) flush(0);
 }
 
 // slot / id bookkeeping of the step and the RC circuit of each run
@@ -1895,20 +1896,20 @@ void launch_collide(const Particles& A, const Particles& B, const uint32_t* off,
                     const uint4* nc2,
                     const uint32_t* cand_off, const uint32_t* active, const uint32_t* mid, const uint32_t* big,
                     DevState* st, long long* rho_e, long long* rho_h, const float* xsE, const float* xs,
-                    const double* cw, const KParams& P, const CollConsts& cc, uint32_t nbins, int sms, int grid,
-                    cudaStream_t s) {
+                    const KParams& P, const CollConsts& cc, int sms, int grid, cudaStream_t s) {
     const RankScratch S{B.key, reinterpret_cast<uint32_t*>(B.pz), reinterpret_cast<uint32_t*>(B.pr),
                         reinterpret_cast<uint32_t*>(B.vz), B.id};
     k_rank_tables<RT_MID_THREADS, RANK_MID_MAX><<<sms * RT_MID_BLOCKS_PER_SM, RT_MID_THREADS, RT_MID_SMEM, s>>>(
         A.id, S, off, cnt, mid, &st->n_mid, rank_queue_max(P.capacity, RANK_WARP_MAX), P.ncell, st);
     k_rank_tables<RT_THREADS, RANK_BLOCK_MAX><<<sms, RT_THREADS, RT_SMEM, s>>>(
         A.id, S, off, cnt, big, &st->n_big, rank_queue_max(P.capacity, RANK_MID_MAX), P.ncell, st);
+    const uint32_t nbig = (uint32_t)std::min(grid, 4 * sms);      // blocks resident from the start
     if (P.charge_max >= 3 || P.heavy_coll || P.coulomb)
-        k_collide<true><<<grid, 128, 0, s>>>(A, S, off, cnt, nc, nc2, cand_off, active, st, rho_e, rho_h, xsE, xs, cw, P,
-                                             cc, nbins);
+        k_collide<true><<<grid, 32 * COLL_WARPS, 0, s>>>(A, S, off, cnt, nc, nc2, cand_off, active, st, rho_e, rho_h,
+                                                         xsE, xs, P, cc, nbig);
     else
-        k_collide<false><<<grid, 128, 0, s>>>(A, S, off, cnt, nc, nc2, cand_off, active, st, rho_e, rho_h, xsE, xs, cw, P,
-                                              cc, nbins);
+        k_collide<false><<<grid, 32 * COLL_WARPS, 0, s>>>(A, S, off, cnt, nc, nc2, cand_off, active, st, rho_e, rho_h,
+                                                          xsE, xs, P, cc, nbig);
 }
 void launch_coulomb(const Particles& A, const Particles& B, const uint32_t* off, const uint32_t* cnt, DevState* st,
                     const KParams& P, const CollConsts& cc, const double* cw, int sms, cudaStream_t s) {

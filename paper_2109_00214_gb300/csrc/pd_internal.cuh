@@ -182,17 +182,22 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
     return c;
 }
 
+// the same out of line: a kernel with many draw sites keeps one copy of the
+// rounds (its instructions then fit the instruction caches)
+static __device__ __noinline__ uint4 philox_block(uint4 c, uint2 k) { return philox4x32_10(c, k); }
+
 // Draw stream keyed by (subject, step, stream id); block counter in word 3.
-struct Stream {
+template <bool CALL>
+struct StreamOf {
     uint4 ctr;
     uint2 key;
     uint4 buf;
     int used;
-    __device__ __forceinline__ Stream(uint32_t subject, uint32_t step, uint32_t sid, uint32_t seed, uint32_t run)
+    __device__ __forceinline__ StreamOf(uint32_t subject, uint32_t step, uint32_t sid, uint32_t seed, uint32_t run)
         : ctr(make_uint4(subject, step, sid, 0u)), key(make_uint2(seed, run)), buf(make_uint4(0, 0, 0, 0)), used(4) {}
     __device__ __forceinline__ uint32_t next() {
         if (used == 4) {
-            buf = philox4x32_10(ctr, key);
+            buf = CALL ? philox_block(ctr, key) : philox4x32_10(ctr, key);
             ctr.w += 1u;
             used = 0;
         }
@@ -205,6 +210,7 @@ struct Stream {
     // uniform integer in [0, n)
     __device__ __forceinline__ uint32_t pick(uint32_t n) { return (uint32_t)(((unsigned long long)next() * n) >> 32); }
 };
+using Stream = StreamOf<false>;
 
 __host__ __device__ constexpr uint32_t sid_cand(int k, uint32_t m) { return ((uint32_t)k << 28) | m; }
 constexpr uint32_t SID_NCAND = 0xE0000000u;

@@ -104,10 +104,8 @@ void launch_ncand(const uint32_t* cnt, const float* ck, uint4* nc, uint4* nc2, u
 void launch_collide(const Particles& A, const Particles& B, const uint32_t* off, const uint32_t* cnt, const uint4* nc,
                     const uint4* nc2,
                     const uint32_t* cand_off, const uint32_t* active, const uint32_t* mid, const uint32_t* big,
-// cw: W dt_coll / V_cell per row (Coulomb pairs)
                     DevState* st, long long* rho_e, long long* rho_h, const float* xsE, const float* xs,
-                    const double* cw, const KParams& P, const CollConsts& cc, uint32_t nbins, int sms, int grid,
-                    cudaStream_t s);
+                    const KParams& P, const CollConsts& cc, int sms, int grid, cudaStream_t s);
 // Coulomb pairs (after launch_collide; one launch)
 void launch_coulomb(const Particles& A, const Particles& B, const uint32_t* off, const uint32_t* cnt, DevState* st,
                     const KParams& P, const CollConsts& cc, const double* cw, int sms, cudaStream_t s);
