@@ -379,6 +379,33 @@ double node_volume(const pd_config& c, int i, int j) {
 
 double mr_class() { return ME * M_CU / (ME + M_CU); }
 
+// channels of the pair classes: the first and their number
+constexpr int CLS_CH0[NCLS] = {CH_EL, CH_SW, CH_S3, CH_S3, CH_S4, CH_CX, CH_NN}, CLS_NCH[NCLS] = {4, 1, 1, 1, 1, 1, 1};
+
+// the NTC majorant (sigma g)_max of class k from the channels' tables
+void update_majorant(pd_sim* s, int k) {
+    CollConsts& cc = s->cc;
+    const double kd = (double)(k < NECLS ? cc.kmr : cc.kmr_h);
+    double best = 0.0;
+    float prev = 0.0f;
+    for (int q = 0; q < XS_N; ++q) {
+        float sT = 0.0f;
+        for (int c = 0; c < CLS_NCH[k]; ++c) sT = sT + s->h_xs[CLS_CH0[k] + c][q];
+        const float smax = sT > prev ? sT : prev;
+        // (an empty stretch of the table cannot raise it)
+        if (q > 0 && smax > 0.0f) {
+            const double g = std::sqrt((double)s->h_xsE[q] / kd);
+            const double cand = (double)smax * g;
+            if (cand > best) best = cand;
+        }
+        prev = sT;
+    }
+    best *= 1.0 + 1e-6;
+    float f = (float)best;
+    if ((double)f < best) f = std::nextafter(f, INFINITY);
+    cc.sgmax[k] = f;
+}
+
 // NTC majorants from the float tables (see pd_set_cross_section)
 void update_collision_consts(pd_sim* s) {
     const double mr = mr_class();
@@ -404,27 +431,7 @@ void update_collision_consts(pd_sim* s) {
         for (int a = 0; a < 5; ++a)
             for (int b = a; b < 5; ++b) cc.kc[cls++] = kc(ZQ[SP_CUP + a], ZQ[SP_CUP + b], 0.5 * M_CU);
     }
-    const int ch0[NCLS] = {CH_EL, CH_SW, CH_S3, CH_S3, CH_S4, CH_CX, CH_NN}, nch[NCLS] = {4, 1, 1, 1, 1, 1, 1};
-    for (int k = 0; k < NCLS; ++k) {
-        const double kd = (double)(k < NECLS ? cc.kmr : cc.kmr_h);
-        double best = 0.0;
-        float prev = 0.0f;
-        for (int q = 0; q < XS_N; ++q) {
-            float sT = 0.0f;
-            for (int c = 0; c < nch[k]; ++c) sT = sT + s->h_xs[ch0[k] + c][q];
-            if (q > 0) {
-                const float smax = sT > prev ? sT : prev;
-                const double g = std::sqrt((double)s->h_xsE[q] / kd);
-                const double cand = (double)smax * g;
-                if (cand > best) best = cand;
-            }
-            prev = sT;
-        }
-        best *= 1.0 + 1e-6;
-        float f = (float)best;
-        if ((double)f < best) f = std::nextafter(f, INFINITY);
-        cc.sgmax[k] = f;
-    }
+    for (int k = 0; k < NCLS; ++k) update_majorant(s, k);
 }
 
 // per-row factors c_k(j) = W (sigma g)_max dt_coll / V_cell(j) of every run
@@ -1357,13 +1364,13 @@ pd_status pd_set_cross_section(pd_sim* s, int ch, const double* E, const double*
     if (ch < 0 || ch >= NCH || n < 2 || !E || !sig) return fail(s, PD_ERR_ARG, "bad cross-section arguments");
     for (int a = 0; a + 1 < n; ++a)
         if (!(E[a + 1] > E[a])) return fail(s, PD_ERR_ARG, "cross-section energies must ascend");
-    for (int k = 0; k < XS_N; ++k) {
+    // both energy grids ascend: one pass over the points
+    for (int k = 0, a = 0; k < XS_N; ++k) {
         const double e = (double)s->h_xsE[k];
         double v;
         if (e <= E[0]) v = sig[0];
         else if (e >= E[n - 1]) v = sig[n - 1];
         else {
-            int a = 0;
             while (E[a + 1] <= e) ++a;
             const double t = (e - E[a]) / (E[a + 1] - E[a]);
             v = sig[a] + t * (sig[a + 1] - sig[a]);
@@ -1373,7 +1380,9 @@ pd_status pd_set_cross_section(pd_sim* s, int ch, const double* E, const double*
         s->h_xs[ch][k] = (float)v;
     }
     s->eth[ch] = threshold;
-    update_collision_consts(s);
+    s->cc.kth[ch] = (float)(2.0 * threshold * QE / mr_class());
+    for (int k = 0; k < NCLS; ++k)
+        if (ch >= CLS_CH0[k] && ch < CLS_CH0[k] + CLS_NCH[k]) update_majorant(s, k);
     drop_graph(s);
     CK(cudaMemcpyAsync(s->xs + (size_t)ch * XS_N, s->h_xs[ch], XS_N * 4, cudaMemcpyHostToDevice, s->stream));
     return upload_ck(s);
@@ -1384,13 +1393,12 @@ pd_status pd_set_sputter_yield(pd_sim* s, const double* E, const double* Y, int 
     if (n < 2 || !E || !Y) return fail(s, PD_ERR_ARG, "bad sputtering-yield arguments");
     for (int a = 0; a + 1 < n; ++a)
         if (!(E[a + 1] > E[a])) return fail(s, PD_ERR_ARG, "yield energies must ascend");
-    for (int k = 0; k < XS_N; ++k) {
+    for (int k = 0, a = 0; k < XS_N; ++k) {
         const double e = (double)s->h_xsE[k];
         double v;
         if (e <= E[0]) v = Y[0];
         else if (e >= E[n - 1]) v = Y[n - 1];
         else {
-            int a = 0;
             while (E[a + 1] <= e) ++a;
             const double t = (e - E[a]) / (E[a + 1] - E[a]);
             v = Y[a] + t * (Y[a + 1] - Y[a]);

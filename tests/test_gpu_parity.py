@@ -88,6 +88,21 @@ def test_dense_cells_bit_exact(pd, xs, n_e, n_t, ncells, scale, Te):
     assert_same_particles(sim.particles(), o.particles())
 
 
+@pytest.mark.parametrize("n", [2, 31, 33, 64, 65, 129, 256, 257])
+@pytest.mark.parametrize("cand", [100, 400])
+def test_few_particles_many_candidates_bit_exact(pd, xs, n, cand):
+    """One cell of n particles a species and about `cand` candidates a class and
+    step (a warp's batches of 32; a block's from 256 on): most candidates share
+    a particle with earlier ones of their batch, and the lists end on and
+    beside the sizes at which their ranks are found another way."""
+    cfg, parts = synthetic.heavy_cells(n_e=n, n_cu=n, n_cup=n, ncells=1, coll_scale=7.5e4 * cand / n ** 2)
+    sim, o = run_pair(pd, cfg, parts, xs, 3)
+    gc, oc = sim.counters(), o.counters()
+    assert_same_counters(gc, oc)
+    assert gc["cand_total"] > cand
+    assert_same_particles(sim.particles(), o.particles())
+
+
 @pytest.mark.parametrize("nz,nr,total,scale,steps", [
     (64, 64, 2e5, 3000.0, 4),      # stress: about one candidate per cell
     (37, 53, 6e4, 20000.0, 3),     # ragged grid, dense collisions, many spawns
