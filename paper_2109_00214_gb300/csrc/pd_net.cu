@@ -6,8 +6,9 @@
 // layers, forward and back-propagation alike, are implicit GEMMs on the
 // tensor cores (mma.sync m16n8k16, bfloat16 operands, float accumulators):
 //   forward / input gradient: M = 16 nodes of a tile row, N = 32 output
-//     channels, K = 9 taps x 32 input channels; a block stages an 8 x 16 node
-//     tile with its halo and the layer's weights in shared memory.  The input
+//     channels, K = 9 taps x 32 input channels; a block stages the layer's
+//     weights once and 8 x 32 node tiles with their halo in shared memory.  The
+//     input
 //     gradient is the same convolution over the output gradient with the
 //     weights mirrored in the tap and transposed in the channels.
 //   weight gradient: per tap, M = 32 output channels, N = 32 input channels,
@@ -42,10 +43,11 @@ constexpr int NP = PD_NET_NPARAMS;
 __host__ __device__ constexpr int off_w(int l) { return l == 0 ? 0 : (l < 5 ? 320 + (l - 1) * 9248 : 37312); }
 __host__ __device__ constexpr int off_b(int l) { return l == 0 ? 288 : off_w(l) + (l < 5 ? 9216 : 288); }
 static_assert(off_b(5) + 1 == PD_NET_NPARAMS, "parameter layout");
-constexpr int TY = 8, TX = 16;       // node tile of the tensor-core kernels
+constexpr int TY = 8, TX = 16;       // node tile of the weight gradients
+constexpr int CX = 32;               // columns of a convolution's tile (of TY rows)
+constexpr int CONV_THREADS = 128;    // a 32 -> 32 layer's block: two column groups by two channel halves
 constexpr int HP = 40;               // channel stride of a staged node (bf16): 80 bytes, conflict-free fragments
-constexpr int GP = 24;               // node stride of the transposed tiles of the weight gradient
-constexpr int MAX_PART_BLOCKS = 512;
+constexpr int MAX_PART_BLOCKS = 384;  // (k_reduce holds a value's partials in 48 KB of shared memory, 32 values a block)
 constexpr int PART_STRIDE = 9 * CH * CH + CH;
 constexpr int LOSS_BLOCKS = 256;
 
@@ -61,10 +63,6 @@ __device__ __forceinline__ void mma_bf16(float* c, uint32_t a0, uint32_t a1, uin
         "{%0,%1,%2,%3};\n"
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
-__device__ __forceinline__ uint32_t pack2(bf16 lo, bf16 hi) {
-    return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
 }
 
 __device__ __forceinline__ size_t node_index(const uint32_t* base, int b, int H, int W, int i, int j) {
@@ -92,150 +90,294 @@ __global__ void k_prep_weights(const float* __restrict__ master, bf16* wk, bf16*
 }
 
 // ---------------------------------------------------------------------------
-// layer 1 (1 -> 32): one thread per node
-__global__ void __launch_bounds__(256) k_conv1(const float* __restrict__ x, bf16* __restrict__ h,
-                                               const float* __restrict__ w1, const float* __restrict__ b1,
-                                               const uint32_t* __restrict__ base, int B, int H, int W) {
-    __shared__ float ws[9 * CH], bs[CH];
-    for (int q = threadIdx.x; q < 9 * CH; q += blockDim.x) ws[q] = w1[q];
-    if (threadIdx.x < CH) bs[threadIdx.x] = b1[threadIdx.x];
-    __syncthreads();
-    const long long n = (long long)H * W, total = n * B;
-    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < total;
-         p += (long long)gridDim.x * blockDim.x) {
-        const int b = (int)(p / n);
-        const int k = (int)(p - (long long)b * n);
-        const int i = k / W, j = k - i * W;
-        float xv[9];
+// a block's next tile of TY x CX nodes: sample and first node
+struct Tile {
+    int b, i0, j0;
+};
+__device__ __forceinline__ Tile tile_at(long long q, int tj, int ti) {
+    const int b = (int)(q / ((long long)tj * ti)), r = (int)(q - (long long)b * tj * ti);
+    return Tile{b, (r / tj) * TY, (r % tj) * CX};
+}
+
+// a tile of float nodes with its halo (zero outside the grid) in shared memory
+__device__ __forceinline__ void stage_nodes(float* xs, const float* __restrict__ x, const uint32_t* base, const Tile& t,
+                                            int H, int W) {
+    for (int q = threadIdx.x; q < (TY + 2) * (CX + 2); q += blockDim.x) {
+        const int hi = q / (CX + 2), hj = q - hi * (CX + 2);
+        const int gi = t.i0 + hi - 1, gj = t.j0 + hj - 1;
+        xs[q] = (gi >= 0 && gi < H && gj >= 0 && gj < W) ? x[node_index(base, t.b, H, W, gi, gj)] : 0.0f;
+    }
+}
+
+// layer 1 (1 -> 32): a warp a tile row, a lane an output channel with its nine
+// weights in registers, the row's 3 x 3 windows passing by in shared memory (three
+// broadcast reads and nine operations a node and lane; a node's 64 bytes are one
+// store of the warp).  513^2 nodes: 21 -> 10.5 us (a thread a node read 288 weights
+// from shared memory and stored 64 bytes a lane).
+__global__ void __launch_bounds__(32 * TY) k_conv1(const float* __restrict__ x, bf16* __restrict__ h,
+                                                   const float* __restrict__ w1, const float* __restrict__ b1,
+                                                   const uint32_t* __restrict__ base, int B, int H, int W) {
+    __shared__ float xs[(TY + 2) * (CX + 2)];
+    const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+    float w[9];
 #pragma unroll
-        for (int tap = 0; tap < 9; ++tap) {
-            const int ii = i + tap_dy(tap), jj = j + tap_dx(tap);
-            xv[tap] = (ii >= 0 && ii < H && jj >= 0 && jj < W) ? x[node_index(base, b, H, W, ii, jj)] : 0.0f;
+    for (int tap = 0; tap < 9; ++tap) w[tap] = w1[tap * CH + lane];
+    const float bias = b1[lane];
+    const int tj = (W + CX - 1) / CX, ti = (H + TY - 1) / TY;
+    const long long ntiles = (long long)B * tj * ti;
+    for (long long q = blockIdx.x; q < ntiles; q += gridDim.x) {
+        const Tile t = tile_at(q, tj, ti);
+        __syncthreads();
+        stage_nodes(xs, x, base, t, H, W);
+        __syncthreads();
+        const int i = t.i0 + row, nj = min(CX, W - t.j0);
+        if (i >= H) continue;
+        bf16* dst = h + node_index(base, t.b, H, W, i, t.j0) * CH + lane;
+        const float* xr = xs + row * (CX + 2);
+        float v[3][3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            v[d][1] = xr[d * (CX + 2)];
+            v[d][2] = xr[d * (CX + 2) + 1];
         }
-        uint32_t o[CH / 2];
+#pragma unroll 4
+        for (int j = 0; j < nj; ++j) {
 #pragma unroll
-        for (int c = 0; c < CH; c += 2) {
-            float a0 = bs[c], a1 = bs[c + 1];
-#pragma unroll
-            for (int tap = 0; tap < 9; ++tap) {
-                a0 += ws[tap * CH + c] * xv[tap];
-                a1 += ws[tap * CH + c + 1] * xv[tap];
+            for (int d = 0; d < 3; ++d) {
+                v[d][0] = v[d][1];
+                v[d][1] = v[d][2];
+                v[d][2] = xr[d * (CX + 2) + j + 2];
             }
-            o[c / 2] = pack2(__float2bfloat16_rn(fmaxf(a0, 0.0f)), __float2bfloat16_rn(fmaxf(a1, 0.0f)));
-        }
-        uint4* dst = (uint4*)(h + node_index(base, b, H, W, i, j) * CH);
+            float a = bias;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) dst[q] = make_uint4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+            for (int tap = 0; tap < 9; ++tap) a += w[tap] * v[tap / 3][tap % 3];
+            dst[(size_t)j * CH] = __float2bfloat16_rn(fmaxf(a, 0.0f));
+        }
     }
 }
 
 // ---------------------------------------------------------------------------
+// four 8 x 8 matrices of bfloat16 from shared memory, a row address a lane
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const bf16* p) {
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(a));
+}
+
+// 16 bytes from global to shared memory without a register, zeros unless `in`
+__device__ __forceinline__ void copy16(void* dst, const void* src, bool in) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(in ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+// all but the latest N groups of copies have landed (this thread's)
+template <int N>
+__device__ __forceinline__ void copy_wait() {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+}
+
+// a tile of rows x cols 32-channel nodes from node (i0, j0) on (zero outside the
+// grid) into shared memory, asynchronously
+__device__ __forceinline__ void stage_channels(bf16* xs, const bf16* __restrict__ in, size_t node0, int i0, int j0,
+                                               int rows, int cols, int H, int W) {
+    for (int q = threadIdx.x; q < rows * cols * 4; q += blockDim.x) {
+        const int nd = q >> 2, part = q & 3;
+        const int hi = nd / cols, hj = nd - hi * cols;
+        const int gi = i0 + hi, gj = j0 + hj;
+        const bool ok = gi >= 0 && gi < H && gj >= 0 && gj < W;
+        copy16(&xs[nd * HP + part * 8], in + (ok ? (node0 + (size_t)gi * W + gj) * CH + part * 8 : 0), ok);
+    }
+    copy_commit();
+}
+__device__ __forceinline__ void stage_halo(bf16* xs, const bf16* __restrict__ in, const uint32_t* base, const Tile& t,
+                                           int H, int W) {
+    stage_channels(xs, in, node_index(base, t.b, H, W, 0, 0), t.i0 - 1, t.j0 - 1, TY + 2, CX + 2, H, W);
+}
+constexpr int TILE_ELEMS = (TY + 2) * (CX + 2) * HP;
+constexpr int CONV_SMEM = 2 * TILE_ELEMS * 2;      // two tiles
+
 // 32 -> 32 convolution on the tensor cores.  MODE 0: out = relu(conv + bias);
 // MODE 1: out = conv where mask > 0, else 0 (input gradient through a ReLU).
-// Block: 8 warps, an 8 x 16 node tile (warp w: tile row w), grid (tiles
-// along j, tiles along i, samples).
+// A warp takes 16 columns of the tile and 16 output channels, their weights in
+// registers throughout (72), and marches down the staged rows: an ldmatrix of an
+// input row's 16 nodes feeds six mma, the row above's, its own and the row
+// below's by two channel octets, so that three rows of accumulators are open and a
+// row is written when its last input row has passed.  The block's next tile is on
+// its way while one is computed.  Shared-memory reads (twelve for four mma) and
+// the latency of staging bounded the form before: 513^2 nodes 27 -> 20.5 us a layer
+// (device time under ncu; the mma pipe 48 % busy).  Each output accumulates
+// in the same order (taps, then channel halves).
 template <int MODE>
-__global__ void __launch_bounds__(256) k_conv32(const bf16* __restrict__ in, bf16* __restrict__ out,
-                                                const bf16* __restrict__ w, const float* __restrict__ bias,
-                                                const bf16* __restrict__ mask, const uint32_t* __restrict__ base,
-                                                int H, int W) {
-    __shared__ __align__(16) bf16 xs[(TY + 2) * (TX + 2) * HP];
-    __shared__ __align__(16) bf16 ws[9 * CH * HP];
-    const int b = blockIdx.z;
-    const int i0 = blockIdx.y * TY, j0 = blockIdx.x * TX;
-    for (int q = threadIdx.x; q < 9 * CH * 4; q += blockDim.x) {
-        const int row = q >> 2, part = q & 3;
-        *(uint4*)&ws[row * HP + part * 8] = ((const uint4*)w)[q];
-    }
-    for (int q = threadIdx.x; q < (TY + 2) * (TX + 2) * 4; q += blockDim.x) {
-        const int nd = q >> 2, part = q & 3;
-        const int hi = nd / (TX + 2), hj = nd - hi * (TX + 2);
-        const int gi = i0 + hi - 1, gj = j0 + hj - 1;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (gi >= 0 && gi < H && gj >= 0 && gj < W) v = ((const uint4*)(in + node_index(base, b, H, W, gi, gj) * CH))[part];
-        *(uint4*)&xs[nd * HP + part * 8] = v;
-    }
-    __syncthreads();
+__global__ void __launch_bounds__(CONV_THREADS, 4) k_conv32(const bf16* __restrict__ in, bf16* __restrict__ out,
+                                                         const bf16* __restrict__ w, const float* __restrict__ bias,
+                                                         const bf16* __restrict__ mask,
+                                                         const uint32_t* __restrict__ base, int B, int H, int W) {
+    extern __shared__ __align__(16) bf16 smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    float acc[4][4];
+    const int cg = (warp >> 1) * 16, c0 = (warp & 1) * 16;     // first column and output channel
+    uint32_t wb[9][2][2][2];
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
+    for (int tap = 0; tap < 9; ++tap)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) acc[nt][e] = 0.0f;
-#pragma unroll 1
-    for (int tap = 0; tap < 9; ++tap) {
-        const bf16* xr = xs + ((warp + tap_dy(tap) + 1) * (TX + 2) + tap_dx(tap) + 1) * HP;
+        for (int kh = 0; kh < 2; ++kh)
 #pragma unroll
-        for (int kh = 0; kh < 2; ++kh) {
-            const int c0 = kh * 16 + 2 * t;
-            const uint32_t a0 = *(const uint32_t*)(xr + g * HP + c0);
-            const uint32_t a1 = *(const uint32_t*)(xr + (g + 8) * HP + c0);
-            const uint32_t a2 = *(const uint32_t*)(xr + g * HP + c0 + 8);
-            const uint32_t a3 = *(const uint32_t*)(xr + (g + 8) * HP + c0 + 8);
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt) {
-                const bf16* wr = ws + (tap * CH + nt * 8 + g) * HP + c0;
-                mma_bf16(acc[nt], a0, a1, a2, a3, *(const uint32_t*)wr, *(const uint32_t*)(wr + 8));
+            for (int nt = 0; nt < 2; ++nt) {
+                const uint32_t* p =
+                    (const uint32_t*)(w + (size_t)(tap * CH + c0 + nt * 8 + g) * CH + kh * 16 + 2 * t);
+                wb[tap][kh][nt][0] = __ldg(p);
+                wb[tap][kh][nt][1] = __ldg(p + 4);
             }
+    float bv[2][2] = {};
+    if (MODE == 0)
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) {
+            bv[nt][0] = bias[c0 + nt * 8 + 2 * t];
+            bv[nt][1] = bias[c0 + nt * 8 + 2 * t + 1];
         }
-    }
-    const int oi = i0 + warp;
-    if (oi >= H) return;
+    // row addresses of the lane's matrices: nodes 0-7, 8-15 by channels 0-7, then 8-15
+    const int xo = (cg + (lane & 15)) * HP + (lane >> 4) * 8;
+    const int tj = (W + CX - 1) / CX, ti = (H + TY - 1) / TY;
+    const long long ntiles = (long long)B * tj * ti;
+    long long q = blockIdx.x;
+    if (q < ntiles) stage_halo(smem, in, base, tile_at(q, tj, ti), H, W);
+    for (int buf = 0; q < ntiles; q += gridDim.x, buf ^= 1) {
+        const Tile tl = tile_at(q, tj, ti);
+        if (q + gridDim.x < ntiles) {
+            stage_halo(smem + (buf ^ 1) * TILE_ELEMS, in, base, tile_at(q + gridDim.x, tj, ti), H, W);
+            copy_wait<1>();
+        } else {
+            copy_wait<0>();
+        }
+        __syncthreads();
+        const bf16* xl = smem + buf * TILE_ELEMS + xo;
+        const bool on = tl.j0 + cg < W;                   // (the warp's columns)
+        float acc[3][2][4];
+        // MODE 1: the mask of the next row to write, loaded a row ahead
+        __nv_bfloat162 mk[2][2], mn[2][2];
+        auto load_mask = [&](int r) {
 #pragma unroll
-    for (int half = 0; half < 2; ++half) {
-        const int oj = j0 + g + 8 * half;
-        if (oj >= W) continue;
-        const size_t nd = node_index(base, b, H, W, oi, oj);
+            for (int half = 0; half < 2; ++half)
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            const int c = nt * 8 + 2 * t;
-            float v0 = acc[nt][2 * half], v1 = acc[nt][2 * half + 1];
-            if (MODE == 0) {
-                v0 = fmaxf(v0 + bias[c], 0.0f);
-                v1 = fmaxf(v1 + bias[c + 1], 0.0f);
-            } else {
-                const __nv_bfloat162 m = *(const __nv_bfloat162*)(mask + nd * CH + c);
-                if (!(__bfloat162float(m.x) > 0.0f)) v0 = 0.0f;
-                if (!(__bfloat162float(m.y) > 0.0f)) v1 = 0.0f;
+                for (int nt = 0; nt < 2; ++nt) {
+                    const int oi = tl.i0 + r, oj = tl.j0 + cg + g + 8 * half;
+                    mn[half][nt] = __floats2bfloat162_rn(0.0f, 0.0f);
+                    if (oi < H && oj < W)
+                        mn[half][nt] = *(const __nv_bfloat162*)(mask + node_index(base, tl.b, H, W, oi, oj) * CH + c0 +
+                                                                nt * 8 + 2 * t);
+                }
+        };
+        if (MODE == 1) load_mask(0);
+        if (on) {
+#pragma unroll
+        for (int hi = 0; hi < TY + 2; ++hi) {              // staged input row
+            if (hi < TY)
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) acc[hi % 3][nt][e] = 0.0f;
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+                for (int kh = 0; kh < 2; ++kh) {
+                    uint32_t a[4];
+                    ldsm4(a, xl + (hi * (CX + 2) + dx) * HP + kh * 16);
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {          // tap row: output row hi - d
+                        if (hi - d < 0 || hi - d >= TY) continue;
+#pragma unroll
+                        for (int nt = 0; nt < 2; ++nt)
+                            mma_bf16(acc[(hi - d + 3) % 3][nt], a[0], a[1], a[2], a[3], wb[3 * d + dx][kh][nt][0],
+                                     wb[3 * d + dx][kh][nt][1]);
+                    }
+                }
+            if (hi < 2) continue;
+            const int r = hi - 2, oi = tl.i0 + r;
+            if (MODE == 1) {
+#pragma unroll
+                for (int half = 0; half < 2; ++half)
+#pragma unroll
+                    for (int nt = 0; nt < 2; ++nt) mk[half][nt] = mn[half][nt];
+                if (r + 1 < TY) load_mask(r + 1);
             }
-            *(__nv_bfloat162*)(out + nd * CH + c) = __floats2bfloat162_rn(v0, v1);
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
-// layer 6 (32 -> 1): one thread per node
-__global__ void __launch_bounds__(256) k_conv6(const bf16* __restrict__ h, float* __restrict__ y,
-                                               const float* __restrict__ w6, const float* __restrict__ b6,
-                                               const uint32_t* __restrict__ base, int B, int H, int W) {
-    __shared__ float ws[9 * CH];
-    for (int q = threadIdx.x; q < 9 * CH; q += blockDim.x) ws[q] = w6[q];
-    __syncthreads();
-    const float bias = b6[0];
-    const long long n = (long long)H * W, total = n * B;
-    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < total;
-         p += (long long)gridDim.x * blockDim.x) {
-        const int b = (int)(p / n);
-        const int k = (int)(p - (long long)b * n);
-        const int i = k / W, j = k - i * W;
-        float acc = bias;
-        for (int tap = 0; tap < 9; ++tap) {
-            const int ii = i + tap_dy(tap), jj = j + tap_dx(tap);
-            if (ii < 0 || ii >= H || jj < 0 || jj >= W) continue;
-            const uint4* src = (const uint4*)(h + node_index(base, b, H, W, ii, jj) * CH);
+            if (oi >= H) continue;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const uint4 v = src[q];
-                const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+            for (int half = 0; half < 2; ++half) {
+                const int oj = tl.j0 + cg + g + 8 * half;
+                if (oj >= W) continue;
+                const size_t nd = node_index(base, tl.b, H, W, oi, oj);
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int c = q * 8 + e * 2;
-                    acc += ws[tap * CH + c] * __uint_as_float(u[e] << 16);
-                    acc += ws[tap * CH + c + 1] * __uint_as_float(u[e] & 0xFFFF0000u);
+                for (int nt = 0; nt < 2; ++nt) {
+                    const int c = c0 + nt * 8 + 2 * t;
+                    float v0 = acc[r % 3][nt][2 * half], v1 = acc[r % 3][nt][2 * half + 1];
+                    if (MODE == 0) {
+                        v0 = fmaxf(v0 + bv[nt][0], 0.0f);
+                        v1 = fmaxf(v1 + bv[nt][1], 0.0f);
+                    } else {
+                        const __nv_bfloat162 m = mk[half][nt];
+                        if (!(__bfloat162float(m.x) > 0.0f)) v0 = 0.0f;
+                        if (!(__bfloat162float(m.y) > 0.0f)) v1 = 0.0f;
+                    }
+                    *(__nv_bfloat162*)(out + nd * CH + c) = __floats2bfloat162_rn(v0, v1);
                 }
             }
         }
-        y[node_index(base, b, H, W, i, j)] = acc;
+        }
+        __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------------------
+// layer 6 (32 -> 1): a thread two nodes (rows r and r + 4) of a tile staged in
+// shared memory, sharing the weights' reads (read from global memory, the 36
+// 16-byte pieces of a node's window are on as many lines a lane: 513^2 nodes 35 ->
+// 17 us)
+__global__ void __launch_bounds__(16 * TY) k_conv6(const bf16* __restrict__ h, float* __restrict__ y,
+                                                   const float* __restrict__ w6, const float* __restrict__ b6,
+                                                   const uint32_t* __restrict__ base, int B, int H, int W) {
+    __shared__ __align__(16) bf16 xs[(TY + 2) * (CX + 2) * HP];
+    __shared__ __align__(16) float ws[9 * CH];
+    for (int q = threadIdx.x; q < 9 * CH; q += blockDim.x) ws[q] = w6[q];
+    const float bias = b6[0];
+    const int row = threadIdx.x / CX, col = threadIdx.x % CX;
+    const int tj = (W + CX - 1) / CX, ti = (H + TY - 1) / TY;
+    const long long ntiles = (long long)B * tj * ti;
+    for (long long q = blockIdx.x; q < ntiles; q += gridDim.x) {
+        const Tile t = tile_at(q, tj, ti);
+        __syncthreads();
+        stage_halo(xs, h, base, t, H, W);
+        copy_wait<0>();
+        __syncthreads();
+        const int j = t.j0 + col;
+        float acc[2] = {bias, bias};
+#pragma unroll
+        for (int tap = 0; tap < 9; ++tap) {
+            const int i0 = t.i0 + row + tap_dy(tap), jj = j + tap_dx(tap);
+            if (jj < 0 || jj >= W) continue;
+            const uint4* src = (const uint4*)(xs + ((row + tap / 3) * (CX + 2) + col + tap % 3) * HP);
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+                const float4 wa = *(const float4*)&ws[tap * CH + p * 8], wc = *(const float4*)&ws[tap * CH + p * 8 + 4];
+                const float wv[8] = {wa.x, wa.y, wa.z, wa.w, wc.x, wc.y, wc.z, wc.w};
+#pragma unroll
+                for (int n = 0; n < 2; ++n) {
+                    if (i0 + n * (TY / 2) < 0 || i0 + n * (TY / 2) >= H) continue;
+                    const uint4 v = src[(size_t)n * (TY / 2) * (CX + 2) * HP / 8 + p];
+                    const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        acc[n] += wv[2 * e] * __uint_as_float(u[e] << 16);
+                        acc[n] += wv[2 * e + 1] * __uint_as_float(u[e] & 0xFFFF0000u);
+                    }
+                }
+            }
+        }
+        if (j >= W) continue;
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+            const int i = t.i0 + row + n * (TY / 2);
+            if (i < H) y[node_index(base, t.b, H, W, i, j)] = acc[n];
+        }
     }
 }
 
@@ -322,54 +464,48 @@ __global__ void __launch_bounds__(256) k_rz_resid_grad(const float* __restrict__
     }
 }
 
-__global__ void k_loss_sum(const double* part, int n, double inv_count, double* out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0;
-        for (int q = 0; q < n; ++q) s += part[q];
-        *out = s * inv_count;
-    }
+// the sum of a loss's n <= LOSS_BLOCKS partials in their order, by one block (a
+// chain of double additions, 8 us: it runs beside k_wgrad6's blocks)
+__device__ __forceinline__ void loss_sum(const double* __restrict__ part, int n, double inv_count, double* out,
+                                         double* p) {
+    if ((int)threadIdx.x < n) p[threadIdx.x] = part[threadIdx.x];
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    double s = 0.0;
+#pragma unroll 8
+    for (int q = 0; q < n; ++q) s += p[q];
+    *out = s * inv_count;
 }
 
-// gradient with respect to a_5: (sum_tap w6[tap][c] g6[p - tap]) where h5 > 0
-__global__ void __launch_bounds__(256) k_conv6_bwd(const float* __restrict__ g6, const bf16* __restrict__ h5,
-                                                   bf16* __restrict__ g5, const float* __restrict__ w6, int B, int H,
-                                                   int W) {
-    __shared__ float ws[9 * CH];
-    for (int q = threadIdx.x; q < 9 * CH; q += blockDim.x) ws[q] = w6[q];
-    __syncthreads();
-    const long long n = (long long)H * W, total = n * B;
-    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < total;
-         p += (long long)gridDim.x * blockDim.x) {
-        const int b = (int)(p / n);
-        const int k = (int)(p - (long long)b * n);
-        const int i = k / W, j = k - i * W;
-        float gv[9];
+// gradient with respect to a_5: (sum_tap w6[tap][c] g6[p - tap]) where h5 > 0, a
+// lane a channel as in k_conv1 (129^2 nodes, eight samples: 13.8 -> 11.4 us)
+__global__ void __launch_bounds__(32 * TY) k_conv6_bwd(const float* __restrict__ g6, const bf16* __restrict__ h5,
+                                                       bf16* __restrict__ g5, const float* __restrict__ w6, int B,
+                                                       int H, int W) {
+    __shared__ float xs[(TY + 2) * (CX + 2)];
+    const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+    float w[9];
 #pragma unroll
-        for (int tap = 0; tap < 9; ++tap) {
-            const int ii = i - tap_dy(tap), jj = j - tap_dx(tap);
-            gv[tap] = (ii >= 0 && ii < H && jj >= 0 && jj < W) ? g6[(size_t)b * n + (size_t)ii * W + jj] : 0.0f;
-        }
-        const uint4* hm = (const uint4*)(h5 + (size_t)p * CH);
-        uint4* dst = (uint4*)(g5 + (size_t)p * CH);
+    for (int tap = 0; tap < 9; ++tap) w[tap] = w6[tap * CH + lane];
+    const int tj = (W + CX - 1) / CX, ti = (H + TY - 1) / TY;
+    const long long ntiles = (long long)B * tj * ti;
+    for (long long q = blockIdx.x; q < ntiles; q += gridDim.x) {
+        const Tile t = tile_at(q, tj, ti);
+        __syncthreads();
+        stage_nodes(xs, g6, nullptr, t, H, W);
+        __syncthreads();
+        const int i = t.i0 + row, nj = min(CX, W - t.j0);
+        if (i >= H) continue;
+        const size_t p0 = node_index(nullptr, t.b, H, W, i, t.j0) * CH + lane;
+        const float* xr = xs + row * (CX + 2);
+#pragma unroll 4
+        for (int j = 0; j < nj; ++j) {
+            const bf16 m = h5[p0 + (size_t)j * CH];
+            float a = 0.0f;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint4 mv = hm[q];
-            const uint32_t mu[4] = {mv.x, mv.y, mv.z, mv.w};
-            uint32_t o[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int c = q * 8 + e * 2;
-                float a0 = 0.0f, a1 = 0.0f;
-#pragma unroll
-                for (int tap = 0; tap < 9; ++tap) {
-                    a0 += ws[tap * CH + c] * gv[tap];
-                    a1 += ws[tap * CH + c + 1] * gv[tap];
-                }
-                if (!(__uint_as_float(mu[e] << 16) > 0.0f)) a0 = 0.0f;
-                if (!(__uint_as_float(mu[e] & 0xFFFF0000u) > 0.0f)) a1 = 0.0f;
-                o[e] = pack2(__float2bfloat16_rn(a0), __float2bfloat16_rn(a1));
-            }
-            dst[q] = make_uint4(o[0], o[1], o[2], o[3]);
+            for (int tap = 0; tap < 9; ++tap) a += w[tap] * xr[(2 - tap / 3) * (CX + 2) + j + 2 - tap % 3];
+            if (!(__bfloat162float(m) > 0.0f)) a = 0.0f;
+            g5[p0 + (size_t)j * CH] = __float2bfloat16_rn(a);
         }
     }
 }
@@ -394,10 +530,17 @@ __global__ void __launch_bounds__(320) k_wgrad1(const float* __restrict__ x, con
         const int r = (int)(tile - (long long)b * tj * ti);
         const int i0 = (r / tj) * TY, j0 = (r % tj) * TX;
         __syncthreads();
-        for (int q = tid; q < TY * TX * CH; q += blockDim.x) {
-            const int nd = q / CH, c = q % CH;
+        for (int q = tid; q < TY * TX * 4; q += blockDim.x) {     // eight channels a load
+            const int nd = q >> 2, part4 = q & 3;
             const int gi = i0 + nd / TX, gj = j0 + nd % TX;
-            gsm[nd][c] = (gi < H && gj < W) ? __bfloat162float(g1[((size_t)b * n + (size_t)gi * W + gj) * CH + c]) : 0.0f;
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            if (gi < H && gj < W) v = ((const uint4*)(g1 + ((size_t)b * n + (size_t)gi * W + gj) * CH))[part4];
+            const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                gsm[nd][part4 * 8 + 2 * e] = __uint_as_float(u[e] << 16);
+                gsm[nd][part4 * 8 + 2 * e + 1] = __uint_as_float(u[e] & 0xFFFF0000u);
+            }
         }
         for (int q = tid; q < (TY + 2) * (TX + 2); q += blockDim.x) {
             const int gi = i0 + q / (TX + 2) - 1, gj = j0 + q % (TX + 2) - 1;
@@ -405,26 +548,34 @@ __global__ void __launch_bounds__(320) k_wgrad1(const float* __restrict__ x, con
         }
         __syncthreads();
         if (tid < 9 * CH) {
+#pragma unroll 32
             for (int nd = 0; nd < TY * TX; ++nd)
                 acc += gsm[nd][co] * xsm[(nd / TX + dy + 1) * (TX + 2) + nd % TX + dx + 1];
         } else {
+#pragma unroll 32
             for (int nd = 0; nd < TY * TX; ++nd) acc += gsm[nd][tid - 9 * CH];
         }
     }
     part[(size_t)blockIdx.x * (9 * CH + CH) + tid] = acc;
 }
 
+// (a last block, beyond the gridDim.x - 1 that take tiles, sums the loss)
 __global__ void __launch_bounds__(320) k_wgrad6(const float* __restrict__ g6, const bf16* __restrict__ h5,
-                                                float* part, int B, int H, int W) {
+                                                float* part, int B, int H, int W, const double* __restrict__ lpart,
+                                                int lb, double inv_count, double* lsum) {
     __shared__ float gsm[TY * TX];
-    __shared__ float hsm[(TY + 2) * (TX + 2)][CH + 1];
-    const int tid = threadIdx.x;
+    __shared__ __align__(16) float hsm[(TY + 2) * (TX + 2)][CH + 1];
+    const int tid = threadIdx.x, nblk = (int)gridDim.x - 1;
+    if ((int)blockIdx.x == nblk) {
+        loss_sum(lpart, lb, inv_count, lsum, reinterpret_cast<double*>(&hsm[0][0]));
+        return;
+    }
     const int tap = tid / CH, ci = tid % CH;
     const int dy = tap < 9 ? tap_dy(tap) : 0, dx = tap < 9 ? tap_dx(tap) : 0;
     const int tj = (W + TX - 1) / TX, ti = (H + TY - 1) / TY;
     const long long ntiles = (long long)B * tj * ti, n = (long long)H * W;
     float acc = 0.0f;
-    for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    for (long long tile = blockIdx.x; tile < ntiles; tile += nblk) {
         const int b = (int)(tile / ((long long)tj * ti));
         const int r = (int)(tile - (long long)b * tj * ti);
         const int i0 = (r / tj) * TY, j0 = (r % tj) * TX;
@@ -433,33 +584,56 @@ __global__ void __launch_bounds__(320) k_wgrad6(const float* __restrict__ g6, co
             const int gi = i0 + q / TX, gj = j0 + q % TX;
             gsm[q] = (gi < H && gj < W) ? g6[(size_t)b * n + (size_t)gi * W + gj] : 0.0f;
         }
-        for (int q = tid; q < (TY + 2) * (TX + 2) * CH; q += blockDim.x) {
-            const int nd = q / CH, c = q % CH;
+        for (int q = tid; q < (TY + 2) * (TX + 2) * 4; q += blockDim.x) {     // eight channels a load
+            const int nd = q >> 2, part4 = q & 3;
             const int gi = i0 + nd / (TX + 2) - 1, gj = j0 + nd % (TX + 2) - 1;
-            hsm[nd][c] = (gi >= 0 && gi < H && gj >= 0 && gj < W)
-                             ? __bfloat162float(h5[((size_t)b * n + (size_t)gi * W + gj) * CH + c])
-                             : 0.0f;
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            if (gi >= 0 && gi < H && gj >= 0 && gj < W)
+                v = ((const uint4*)(h5 + ((size_t)b * n + (size_t)gi * W + gj) * CH))[part4];
+            const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                hsm[nd][part4 * 8 + 2 * e] = __uint_as_float(u[e] << 16);
+                hsm[nd][part4 * 8 + 2 * e + 1] = __uint_as_float(u[e] & 0xFFFF0000u);
+            }
         }
         __syncthreads();
         if (tid < 9 * CH) {
+#pragma unroll 32
             for (int nd = 0; nd < TY * TX; ++nd)
                 acc += gsm[nd] * hsm[(nd / TX + dy + 1) * (TX + 2) + nd % TX + dx + 1][ci];
         } else if (tid == 9 * CH) {
+#pragma unroll 32
             for (int nd = 0; nd < TY * TX; ++nd) acc += gsm[nd];
         }
     }
     if (tid <= 9 * CH) part[(size_t)blockIdx.x * (9 * CH + 1) + tid] = acc;
 }
 
-// weight gradient of a 32 -> 32 layer on the tensor cores: warp = tap.
-// Tiles are staged transposed (channel-major rows of 16 nodes) so that the
-// node index is the contiguous GEMM k dimension of both operands.
+// the same, each 8 x 8 matrix transposed
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], const bf16* p) {
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(a));
+}
+
+// weight gradient of a 32 -> 32 layer on the tensor cores: warp = tap.  Both
+// operands have the nodes as the GEMM's k: the tiles are staged as they lie
+// (node-major) and read through transposing ldmatrix, four for eight mma, where a
+// tap's shift is an offset of nodes.  (Staged channel-major by 2-byte stores with
+// bank conflicts and read by 2-byte loads: 129^2 nodes, eight samples, 27 -> 18.5 us.)
 __global__ void __launch_bounds__(288) k_wgrad32(const bf16* __restrict__ h, const bf16* __restrict__ g,
                                                  float* part, int B, int H, int W) {
-    __shared__ __align__(16) bf16 gs[TY * CH * GP];          // [row][co][col]
-    __shared__ __align__(16) bf16 hs[(TY + 2) * CH * GP];    // [halo row][ci][halo col]
+    __shared__ __align__(16) bf16 gs[TY * TX * HP];
+    __shared__ __align__(16) bf16 hs[(TY + 2) * (TX + 2) * HP];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gq = lane >> 2, t = lane & 3;
     const int dy = tap_dy(warp), dx = tap_dx(warp);
+    // row addresses of the lane's matrices.  A (output channels by nodes): nodes
+    // 0-7 by channels 0-7, 8-15, then nodes 8-15; B (nodes by input channels):
+    // channels 0-7 by nodes 0-7, 8-15, then channels 8-15
+    const bf16* ga = gs + ((lane & 7) + (lane >> 4) * 8) * HP + ((lane >> 3) & 1) * 8;
+    const bf16* hb = hs + ((dy + 1) * (TX + 2) + dx + 1 + (lane & 7) + ((lane >> 3) & 1) * 8) * HP + (lane >> 4) * 8;
     float acc[2][4][4];
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt)
@@ -476,51 +650,27 @@ __global__ void __launch_bounds__(288) k_wgrad32(const bf16* __restrict__ h, con
         const int r = (int)(tile - (long long)b * tj * ti);
         const int i0 = (r / tj) * TY, j0 = (r % tj) * TX;
         __syncthreads();
-        for (int q = threadIdx.x; q < TY * TX * 4; q += blockDim.x) {
-            const int nd = q >> 2, part4 = q & 3;
-            const int ri = nd / TX, rj = nd - ri * TX;
-            const int gi = i0 + ri, gj = j0 + rj;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (gi < H && gj < W) v = ((const uint4*)(g + ((size_t)b * n + (size_t)gi * W + gj) * CH))[part4];
-            const bf16* e = (const bf16*)&v;
-#pragma unroll
-            for (int k = 0; k < 8; ++k) gs[(ri * CH + part4 * 8 + k) * GP + rj] = e[k];
-        }
-        for (int q = threadIdx.x; q < (TY + 2) * (TX + 2) * 4; q += blockDim.x) {
-            const int nd = q >> 2, part4 = q & 3;
-            const int hi = nd / (TX + 2), hj = nd - hi * (TX + 2);
-            const int gi = i0 + hi - 1, gj = j0 + hj - 1;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (gi >= 0 && gi < H && gj >= 0 && gj < W)
-                v = ((const uint4*)(h + ((size_t)b * n + (size_t)gi * W + gj) * CH))[part4];
-            const bf16* e = (const bf16*)&v;
-#pragma unroll
-            for (int k = 0; k < 8; ++k) hs[(hi * CH + part4 * 8 + k) * GP + hj] = e[k];
-        }
+        stage_channels(gs, g, (size_t)b * n, i0, j0, TY, TX, H, W);
+        stage_channels(hs, h, (size_t)b * n, i0 - 1, j0 - 1, TY + 2, TX + 2, H, W);
+        copy_wait<0>();
         __syncthreads();
-#pragma unroll 1
+#pragma unroll
         for (int ri = 0; ri < TY; ++ri) {
-            uint32_t a[2][4];
+            uint32_t a[2][4], bb[2][4];
+            ldsm4t(a[0], ga + ri * TX * HP);
+            ldsm4t(a[1], ga + ri * TX * HP + 16);
+            ldsm4t(bb[0], hb + ri * (TX + 2) * HP);
+            ldsm4t(bb[1], hb + ri * (TX + 2) * HP + 16);
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt) {
-                const bf16* gr = gs + (ri * CH + mt * 16 + gq) * GP + 2 * t;
-                a[mt][0] = *(const uint32_t*)gr;
-                a[mt][1] = *(const uint32_t*)(gr + 8 * GP);
-                a[mt][2] = *(const uint32_t*)(gr + 8);
-                a[mt][3] = *(const uint32_t*)(gr + 8 * GP + 8);
-            }
+            for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
-            for (int nt = 0; nt < 4; ++nt) {
-                const bf16* hr = hs + ((ri + dy + 1) * CH + nt * 8 + gq) * GP + dx + 1;
-                const uint32_t b0 = pack2(hr[2 * t], hr[2 * t + 1]);
-                const uint32_t b1 = pack2(hr[2 * t + 8], hr[2 * t + 9]);
-#pragma unroll
-                for (int mt = 0; mt < 2; ++mt) mma_bf16(acc[mt][nt], a[mt][0], a[mt][1], a[mt][2], a[mt][3], b0, b1);
-            }
+                for (int mt = 0; mt < 2; ++mt)
+                    mma_bf16(acc[mt][nt], a[mt][0], a[mt][1], a[mt][2], a[mt][3], bb[nt >> 1][2 * (nt & 1)],
+                             bb[nt >> 1][2 * (nt & 1) + 1]);
         }
         if (threadIdx.x < CH)
-            for (int ri = 0; ri < TY; ++ri)
-                for (int rj = 0; rj < TX; ++rj) bacc += __bfloat162float(gs[(ri * CH + threadIdx.x) * GP + rj]);
+#pragma unroll 32
+            for (int nd = 0; nd < TY * TX; ++nd) bacc += __bfloat162float(gs[nd * HP + threadIdx.x]);
     }
     float* P = part + (size_t)blockIdx.x * PART_STRIDE;
 #pragma unroll
@@ -536,13 +686,25 @@ __global__ void __launch_bounds__(288) k_wgrad32(const bf16* __restrict__ h, con
     if (threadIdx.x < CH) P[9 * CH * CH + threadIdx.x] = bacc;
 }
 
-// out[k] = sum over blocks c (in order) of part[c * stride + k], k < count
-__global__ void k_reduce(const float* __restrict__ part, int nblocks, int stride, int count, float* out) {
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < count; k += gridDim.x * blockDim.x) {
-        float s = 0.0f;
-        for (int c = 0; c < nblocks; ++c) s += part[(size_t)c * stride + k];
-        out[k] = s;
-    }
+// out[k] = sum over blocks c (in order) of part[c * stride + k], k < count: a block
+// brings 32 values' partials into shared memory with all its loads in flight, a
+// warp adds them in order (the chain of additions waited for a load each: 304
+// partials of 9248 values 31 -> 10 us)
+constexpr int RED_COLS = 32;
+__global__ void __launch_bounds__(256) k_reduce(const float* __restrict__ part, int nblocks, int stride, int count,
+                                                float* out) {
+    extern __shared__ float ps[];
+    const int k0 = blockIdx.x * RED_COLS, lane = threadIdx.x & 31;
+    const bool in = k0 + lane < count;
+#pragma unroll 8
+    for (int c = threadIdx.x >> 5; c < nblocks; c += 8)
+        ps[c * RED_COLS + lane] = in ? part[(size_t)c * stride + k0 + lane] : 0.0f;
+    __syncthreads();
+    if (threadIdx.x >= RED_COLS || !in) return;
+    float s = 0.0f;
+#pragma unroll 16
+    for (int c = 0; c < nblocks; ++c) s += ps[c * RED_COLS + lane];
+    out[k0 + lane] = s;
 }
 
 __global__ void k_adam(float* w, float* m, float* v, const float* __restrict__ g, float lr, float b1, float b2,
@@ -627,16 +789,21 @@ bool shape_ok(const pd_net* net, int B, int H, int W) {
     return B >= 1 && H >= 1 && W >= 1 && (int64_t)B * H * W <= net->max_nodes;
 }
 
+// blocks of a kernel over the tiles of TY x CX nodes, `per_sm` to an SM
+int tile_blocks(const pd_net* net, int B, int H, int W, int per_sm) {
+    const long long n = (long long)B * ((W + CX - 1) / CX) * ((H + TY - 1) / TY);
+    return (int)std::min(n, (long long)net->sms * per_sm);
+}
+
 void forward_layers(pd_net* net, const float* x, float* y, int B, int H, int W, const uint32_t* base,
                     cudaStream_t s) {
-    const long long total = (long long)B * H * W;
     const float* P = net->master;
-    k_conv1<<<elem_blocks(net, total), 256, 0, s>>>(x, net->h[0], net->w1r, P + off_b(0), base, B, H, W);
-    const dim3 grid((W + TX - 1) / TX, (H + TY - 1) / TY, B);
+    const int gc = tile_blocks(net, B, H, W, 4), ge = tile_blocks(net, B, H, W, 8);
+    k_conv1<<<ge, 32 * TY, 0, s>>>(x, net->h[0], net->w1r, P + off_b(0), base, B, H, W);
     for (int l = 1; l <= 4; ++l)
-        k_conv32<0><<<grid, 256, 0, s>>>(net->h[l - 1], net->h[l], net->wk + (size_t)(l - 1) * 9 * CH * CH,
-                                         P + off_b(l), nullptr, base, H, W);
-    k_conv6<<<elem_blocks(net, total), 256, 0, s>>>(net->h[4], y, net->w6r, P + off_b(5), base, B, H, W);
+        k_conv32<0><<<gc, CONV_THREADS, CONV_SMEM, s>>>(net->h[l - 1], net->h[l], net->wk + (size_t)(l - 1) * 9 * CH * CH,
+                                                   P + off_b(l), nullptr, base, B, H, W);
+    k_conv6<<<ge, 16 * TY, 0, s>>>(net->h[4], y, net->w6r, P + off_b(5), base, B, H, W);
 }
 
 pd_status upload_weights(pd_net* net) {
@@ -676,7 +843,9 @@ pd_status pd_net_create(int64_t max_nodes, void* ws, size_t bytes, void* stream,
     if (!net) return PD_ERR_ARG;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&net->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaDeviceGetAttribute(&net->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaFuncSetAttribute(k_conv32<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, CONV_SMEM) != cudaSuccess ||
+        cudaFuncSetAttribute(k_conv32<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, CONV_SMEM) != cudaSuccess) {
         delete net;
         return PD_ERR_CUDA;
     }
@@ -750,30 +919,34 @@ pd_status pd_net_forward(pd_net* net, const float* x, int B, int H, int W, float
 
 namespace {
 
+// sum of `blocks` partials of n values each
+void reduce(const float* part, int blocks, int n, float* out, cudaStream_t s) {
+    k_reduce<<<(n + RED_COLS - 1) / RED_COLS, 256, (size_t)blocks * RED_COLS * 4, s>>>(part, blocks, n, n, out);
+}
+
 // back-propagation of the output gradient g6 (B H W floats) to the
-// parameter gradient, and the loss and gradient out to the host if asked
-pd_status backprop(pd_net* net, const float* x, const float* g6, int B, int H, int W, double* loss, float* grads) {
+// parameter gradient, and the loss (of lb partials) and gradient out to the host
+// if asked
+pd_status backprop(pd_net* net, const float* x, const float* g6, int B, int H, int W, int lb, double inv_count,
+                   double* loss, float* grads) {
     cudaStream_t s = net->stream;
-    const long long total = (long long)B * H * W;
     const int pb = part_blocks(net);
-    const int eb = elem_blocks(net, total);
+    const int gc = tile_blocks(net, B, H, W, 4), ge = tile_blocks(net, B, H, W, 8);
     // layer 6
-    k_wgrad6<<<pb, 320, 0, s>>>(g6, net->h[4], net->part, B, H, W);
-    k_reduce<<<2, 160, 0, s>>>(net->part, pb, 9 * CH + 1, 9 * CH + 1, net->grad + off_w(5));
-    k_conv6_bwd<<<eb, 256, 0, s>>>(g6, net->h[4], net->g[4], net->w6r, B, H, W);
+    k_wgrad6<<<pb + 1, 320, 0, s>>>(g6, net->h[4], net->part, B, H, W, net->lpart, lb, inv_count, net->lsum);
+    reduce(net->part, pb, 9 * CH + 1, net->grad + off_w(5), s);
+    k_conv6_bwd<<<ge, 32 * TY, 0, s>>>(g6, net->h[4], net->g[4], net->w6r, B, H, W);
     // layers 5 .. 2
-    const dim3 grid((W + TX - 1) / TX, (H + TY - 1) / TY, B);
     for (int l = 4; l >= 1; --l) {
         k_wgrad32<<<pb, 288, 0, s>>>(net->h[l - 1], net->g[l], net->part, B, H, W);
         // weights then biases: both contiguous in the parameter vector
-        k_reduce<<<(PART_STRIDE + 255) / 256, 256, 0, s>>>(net->part, pb, PART_STRIDE, PART_STRIDE,
-                                                          net->grad + off_w(l));
-        k_conv32<1><<<grid, 256, 0, s>>>(net->g[l], net->g[l - 1], net->wt + (size_t)(l - 1) * 9 * CH * CH,
-                                         nullptr, net->h[l - 1], nullptr, H, W);
+        reduce(net->part, pb, PART_STRIDE, net->grad + off_w(l), s);
+        k_conv32<1><<<gc, CONV_THREADS, CONV_SMEM, s>>>(net->g[l], net->g[l - 1], net->wt + (size_t)(l - 1) * 9 * CH * CH,
+                                                   nullptr, net->h[l - 1], nullptr, B, H, W);
     }
     // layer 1
     k_wgrad1<<<pb, 320, 0, s>>>(x, net->g[0], net->part, B, H, W);
-    k_reduce<<<2, 160, 0, s>>>(net->part, pb, 9 * CH + CH, 9 * CH + CH, net->grad + off_w(0));
+    reduce(net->part, pb, 9 * CH + CH, net->grad + off_w(0), s);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return net_fail(net, PD_ERR_CUDA, cudaGetErrorString(e));
     net->have_grad = true;
@@ -796,8 +969,7 @@ pd_status pd_net_loss_grad(pd_net* net, const float* x, const float* t, int B, i
     forward_layers(net, x, net->ybuf, B, H, W, nullptr, s);
     const int lb = (int)std::min<long long>(LOSS_BLOCKS, (total + 255) / 256);
     k_loss<<<lb, 256, 0, s>>>(net->ybuf, t, net->g6, net->lpart, total);
-    k_loss_sum<<<1, 32, 0, s>>>(net->lpart, lb, 1.0 / (double)total, net->lsum);
-    return backprop(net, x, net->g6, B, H, W, loss, grads);
+    return backprop(net, x, net->g6, B, H, W, lb, 1.0 / (double)total, loss, grads);
 }
 
 pd_status pd_net_loss_grad_rz(pd_net* net, const float* x, int B, int H, int W, double* loss, float* grads) {
@@ -810,10 +982,9 @@ pd_status pd_net_loss_grad_rz(pd_net* net, const float* x, int B, int H, int W, 
     const int lb = (int)std::min<long long>(LOSS_BLOCKS, (total + 255) / 256);
     // r into g6, then dL/dy = -(2 / N) S r into ybuf (y is not needed after r)
     k_rz_resid<<<lb, 256, 0, s>>>(x, net->ybuf, net->g6, net->lpart, B, H, W);
-    k_loss_sum<<<1, 32, 0, s>>>(net->lpart, lb, 1.0 / (double)n_int, net->lsum);
     k_rz_resid_grad<<<elem_blocks(net, total), 256, 0, s>>>(net->g6, net->ybuf, (float)(-2.0 / (double)n_int), B, H,
                                                            W);
-    return backprop(net, x, net->ybuf, B, H, W, loss, grads);
+    return backprop(net, x, net->ybuf, B, H, W, lb, 1.0 / (double)n_int, loss, grads);
 }
 
 pd_status pd_net_adam(pd_net* net, float lr, float b1, float b2, float eps) {
