@@ -72,6 +72,25 @@ def test_forward_loss_and_gradients_match_the_oracle(pd, torch, B, H, W):
     net.close()
 
 
+@pytest.mark.parametrize("B,H,W", [(1, 8, 32), (2, 9, 33), (1, 7, 31), (3, 17, 65), (1, 1, 1)])
+def test_tile_edges_match_the_oracle(pd, torch, B, H, W):
+    """Grids that end on and beside the 8 x 32 node tiles, forward and gradients
+    (the tolerances of the comparison above: bfloat16 activations)."""
+    rng = np.random.default_rng(H * W)
+    p = _params(4)
+    x = rng.standard_normal((B, H, W)).astype(np.float32)
+    t = (0.1 * rng.standard_normal((B, H, W))).astype(np.float32)
+    net = pd.Net(B * H * W, params=p)
+    xd, td = torch.from_numpy(x).cuda(), torch.from_numpy(t).cuda()
+    yo, _ = cnn.forward(p.astype(np.float64), x, bf16=True)
+    assert _rel(net.forward(xd).cpu().numpy(), yo) <= 2e-3
+    loss, g = net.loss_grad(xd, td, want_grads=True)
+    lo, go = cnn.loss_and_grad(p.astype(np.float64), x, t, bf16=True)
+    assert loss == pytest.approx(lo, rel=2e-3)
+    assert _rel(g, go) <= 1e-2
+    net.close()
+
+
 def test_gradient_check_fails_for_a_wrong_gradient(pd, torch):
     """The comparison above has teeth: the GPU gradient is far from the
     oracle's gradient of a perturbed problem (targets shifted)."""
