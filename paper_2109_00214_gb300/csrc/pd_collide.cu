@@ -136,9 +136,9 @@ __device__ __noinline__ void deposit1(long long* rho, const RunInfo& RI, int geo
 // scatter's atomics, so each list the candidates use is mapped rank ->
 // position by one of:
 //   * ids already ascending with the position (rank = position);
-//   * a rank table, position of the r-th smallest id at table[r].  Up to 32
-//     ids (64 when their range needs two digits): by comparisons (the rank of
-//     an id is the number of smaller ids in the list); up to RANK_WARP_MAX =
+//   * a rank table, position of the r-th smallest id at table[r].  Up to
+//     COMPARE_MAX ids: by comparisons (the rank of an id is the number of
+//     smaller ids in the list); up to RANK_WARP_MAX =
 //     32 * RC: a stable LSD radix sort of (id, position) pairs by 8-bit digits
 //     of id - (smallest id), by the cell's warp in its shared memory; longer
 //     lists: the same sort by a block of k_rank_tables (before k_collide), in
@@ -149,6 +149,7 @@ __device__ __noinline__ void deposit1(long long* rho, const RunInfo& RI, int geo
 // A block's table of the list at slots [b, b + n) is written to table[b, b + n).
 
 constexpr int RC = 8;                           // rows of 32 ids a warp sorts itself
+constexpr uint32_t COMPARE_MAX = 64;            // ids whose ranks come from comparisons
 constexpr uint32_t RANK_BLOCK_MAX = 12288;      // longest list the large kernel sorts in shared memory
 constexpr int RT_THREADS = 1024;                // threads of a large-kernel block
 constexpr int RT_MID_THREADS = 256;             // threads of a mid-size-kernel block
@@ -450,10 +451,12 @@ __global__ void __launch_bounds__(NT) k_rank_tables(const uint32_t* __restrict__
 // select8 costs less (never with want_table).  sbuf: four arrays of
 // RANK_WARP_MAX, then 256 counters.  Out of line: one copy serves every list.
 //
-// Costs in instructions: comparing 64 ids about 340 (32: 100), a radix pass 96 +
-// 64 per 32 ids, a select8 pass 130.  A cell's own heavies have neighbouring ids,
-// so that the digits of id - (smallest id), not of the id, decide the passes: a
-// cell of 80 atoms takes one or two instead of four.
+// Costs in instructions: comparing n ids 13 n / 4 per 32 of them, a radix pass 96 +
+// 64 per 32 ids, a select8 pass 130; but the comparisons are one short loop where
+// the sort's code is fetched anew for nearly every list (stress case, 685 -> 520
+// us with 64 ids by comparison; 128 the same, 256 slower).  A cell's own heavies
+// have neighbouring ids, so that the digits of id - (smallest id), not of the id,
+// decide the passes: a cell of 80 atoms takes one or two instead of four.
 __device__ __noinline__ int rank_list(const uint32_t* __restrict__ base, uint32_t n, uint32_t lookups, uint32_t* table,
                                       uint32_t* sbuf, int id_top, bool want_table) {
     const uint32_t lane = threadIdx.x & 31u;
@@ -489,19 +492,19 @@ __device__ __noinline__ int rank_list(const uint32_t* __restrict__ base, uint32_
     hi = __reduce_max_sync(FULL, hi);
     const int top = hi > lo ? 31 - __clz((int)(hi - lo)) : 0;
     const uint32_t passes = (uint32_t)(top / 8 + 1);
-    if (n <= 32u || (n <= 64u && passes > 1u)) {
+    if (n <= COMPARE_MAX) {
         const uint4* x4 = reinterpret_cast<const uint4*>(xk);
-        const uint32_t a = xk[lane], b = xk[32u + lane];
-        uint32_t r0 = 0, r1 = 0;
 #pragma unroll 1
-        for (uint32_t j = 0; 4u * j < n; ++j) {
-            const uint4 v = x4[j];
-            r0 += (v.x < a ? 1u : 0u) + (v.y < a ? 1u : 0u) + (v.z < a ? 1u : 0u) + (v.w < a ? 1u : 0u);
-            if (n > 32u)
-                r1 += (v.x < b ? 1u : 0u) + (v.y < b ? 1u : 0u) + (v.z < b ? 1u : 0u) + (v.w < b ? 1u : 0u);
+        for (uint32_t q = lane; q < ((n + 31u) & ~31u); q += 32) {
+            const uint32_t a = xk[q];
+            uint32_t r = 0;
+#pragma unroll 1
+            for (uint32_t j = 0; 4u * j < n; ++j) {
+                const uint4 v = x4[j];
+                r += (v.x < a ? 1u : 0u) + (v.y < a ? 1u : 0u) + (v.z < a ? 1u : 0u) + (v.w < a ? 1u : 0u);
+            }
+            if (q < n) table[r] = q;
         }
-        if (lane < n) table[r0] = lane;
-        if (32u + lane < n) table[r1] = 32u + lane;
         __syncwarp();
         return 1;
     }
