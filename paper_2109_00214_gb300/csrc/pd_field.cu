@@ -46,7 +46,8 @@ namespace {
 constexpr double QE_ = 1.602176634e-19;
 constexpr double EPS0_ = 8.8541878128e-12;
 constexpr double PI_ = 3.14159265358979323846;
-constexpr int RED_ROWS = 8;            // a warp's part of the residual: 32 radial nodes x 8 rows
+constexpr int RED_ROWS = 4;            // a warp's part of the residual: 32 radial nodes x 4 rows
+constexpr int RED_WARPS = 4;           // of a block
 constexpr int TILE_WARPS = 4;          // tiles of a block of the smoothing kernels
 // A smoothing tile is a window of 64 radial nodes x K rows, two columns to a
 // lane and the rows in registers; each half-sweep spoils a ring of the window,
@@ -84,19 +85,12 @@ int tail_level(const int* a, const int* b, int n) {
     return n - 1;
 }
 
-// k_mg_tail's shared memory for one run: e, f, r per node and ap, am, b,
-// dinv per radial node of each tail level
-size_t tail_floats(const int* a, const int* b, int n) {
-    size_t t = 0;
-    for (int l = tail_level(a, b, n); l < n; ++l) t += 3 * (size_t)(a[l] + 1) * (b[l] + 1) + 4 * (size_t)(b[l] + 1);
-    return t;
-}
-
 int tiles_of(int nz, int nr, int K, int halo) {
     const int ti = K - 2 * halo, tj = WIN_C - 2 * halo;
     return ((nz + ti - 1) / ti) * ((nr + tj) / tj);
 }
 int red_units(int nz, int nr) { return ((nz - 1 + RED_ROWS - 1) / RED_ROWS) * ((nr + 32) / 32); }
+int red_blocks(int nz, int nr) { return (red_units(nz, nr) + RED_WARPS - 1) / RED_WARPS; }
 
 // work-list entries of one run (all levels that smooth)
 size_t run_tasks(int nz, int nr) {
@@ -105,7 +99,7 @@ size_t run_tasks(int nz, int nr) {
     size_t t = 0;
     for (int l = 0; l + 1 < n; ++l)
         t += tiles_of(a[l], b[l], K_SMALL, PRE_H) + tiles_of(a[l], b[l], K_SMALL, POST_H);
-    return t + (red_units(nz, nr) + 7) / 8;
+    return t + red_blocks(nz, nr);
 }
 
 // device bytes of one run, in the order field_init takes them
@@ -120,7 +114,7 @@ size_t run_bytes(int nz, int nr) {
     }
     for (int l = tail_level(a, b, n); l < n; ++l) t += al(4 * ((size_t)b[l] + 1) * 4);   // k_mg_tail's coefficients
     const size_t m = (size_t)coarse_unknowns(a, b, n);
-    if (m <= (size_t)MG_DIRECT_MAX) t += al(m * m * 4);
+    if (m <= (size_t)MG_DIRECT_MAX) t += al(m * m * 4 + 16);            // (read in units of 16 bytes)
     return t;
 }
 }  // namespace
@@ -138,7 +132,7 @@ size_t field_workspace_bytes(const std::vector<int>& nz, const std::vector<int>&
     for (size_t r = 0; r < R; ++r) {
         t += run_bytes(nz[r], nr[r]);
         tasks += run_tasks(nz[r], nr[r]);
-        red += (red_units(nz[r], nr[r]) + 7) / 8;
+        red += red_blocks(nz[r], nr[r]);
     }
     t += al(R * MG_MAX_LEVELS * sizeof(MGLevel)) + al(R * sizeof(MGTop)) + al(R * 4) * 3 +
          al(red * 2 * 8) + al(R * 8) * 2 + al(R * sizeof(TailRun)) + al(tasks * sizeof(int2) + 8);
@@ -152,13 +146,13 @@ size_t field_workspace_bytes(const std::vector<int>& nz, const std::vector<int>&
 // first of a solve, that of b), and the right-hand side of the next correction:
 // level 0's f = r (float).  A warp takes 32 radial nodes and marches over
 // RED_ROWS rows, so that each node of phi is read once a row, not three times;
-// double arithmetic (seven operations a node) bounds it on a large grid.  Work
-// list of (run, first unit), eight units a block; the block that finishes a
+// double arithmetic (seven operations a node) bounds it, and small units spread it
+// over the SMs: 120 x 480 cells 11.8 us with 8 rows a warp and 8 warps a block, 8.8.  Work list of (run, first unit), four units a block; the block that finishes a
 // run's last units sums the blocks' parts in their order and judges the run:
 // relres = |r| / |b|, converged flag, bookkeeping.
 // 512 x 512 cells, device time of a launch under ncu: 14.7 us with the norm (13.8
 // + 8.9 us as a launch of rows and one of norms).
-__global__ void __launch_bounds__(256) k_residual_norms(const MGTop* top, const MGLevel* lev, const int2* tasks,
+__global__ void __launch_bounds__(32 * RED_WARPS) k_residual_norms(const MGTop* top, const MGLevel* lev, const int2* tasks,
                                                         const int* red_base, double* red, unsigned int* ticket,
                                                         double* bnorm, int* done, const double* tol, RunState* rs,
                                                         int cycle) {
@@ -213,23 +207,23 @@ __global__ void __launch_bounds__(256) k_residual_norms(const MGTop* top, const 
         acc += __shfl_down_sync(0xFFFFFFFFu, acc, o);
         accb += __shfl_down_sync(0xFFFFFFFFu, accb, o);
     }
-    __shared__ double sa[8], sb[8];
+    __shared__ double sa[RED_WARPS], sb[RED_WARPS];
     __shared__ bool s_last;
     if (lane == 0) {
         sa[w] = acc;
         sb[w] = accb;
     }
     __syncthreads();
-    const int blocks = (cols * rows + 7) / 8;
+    const int blocks = (cols * rows + RED_WARPS - 1) / RED_WARPS;
     double* rd = red + 2 * (size_t)red_base[run];
     if (threadIdx.x == 0) {
         double t = 0, tb = 0;
-        for (int q = 0; q < 8; ++q) {
+        for (int q = 0; q < RED_WARPS; ++q) {
             t += sa[q];
             tb += sb[q];
         }
-        __stcg(&rd[2 * (tk.y / 8)], t);
-        __stcg(&rd[2 * (tk.y / 8) + 1], tb);
+        __stcg(&rd[2 * (tk.y / RED_WARPS)], t);
+        __stcg(&rd[2 * (tk.y / RED_WARPS) + 1], tb);
         __threadfence();
         s_last = atomicAdd(&ticket[run], 1u) == (unsigned int)(blocks - 1);
     }
@@ -237,7 +231,7 @@ __global__ void __launch_bounds__(256) k_residual_norms(const MGTop* top, const 
     if (!s_last) return;
     __threadfence();
     acc = accb = 0.0;
-    for (int q = threadIdx.x; q < blocks; q += 256) {
+    for (int q = threadIdx.x; q < blocks; q += 32 * RED_WARPS) {
         acc += __ldcg(&rd[2 * q]);
         accb += __ldcg(&rd[2 * q + 1]);
     }
@@ -252,7 +246,7 @@ __global__ void __launch_bounds__(256) k_residual_norms(const MGTop* top, const 
     __syncthreads();
     if (threadIdx.x != 0) return;
     double a = 0, b = 0;
-    for (int q = 0; q < 8; ++q) {
+    for (int q = 0; q < RED_WARPS; ++q) {
         a += sa[q];
         b += sb[q];
     }
@@ -506,10 +500,15 @@ __global__ void __launch_bounds__(TILE_WARPS * 32, K == K_LARGE ? 2 : 3) k_up(co
 // its nodes (one of each color, two on a few narrow grids), their right-hand
 // sides and coefficients in registers through a level's sweeps, and a phase is
 // four shared-memory reads, five operations and a write; the run's table and
-// its coefficients come in one copy each.  Three levels from 32 x 32 cells: 26.5
-// -> 16.9 us; with 14 x 61 coarsest unknowns by 200 sweeps (the paper's domain):
-// 156 -> 39 us.
+// its coefficients come in one copy each.  An inverse of up to INV_SMEM unknowns is
+// copied into shared memory by cp.async meanwhile (21 KB at 8 x 8 cells; from L2,
+// when it is needed, it cost 1.2 us more).  Three levels from 28 x 12 cells: 9.3
+// -> 8.0 us by that; with 14 x 61 coarsest unknowns by 200 sweeps (the paper's
+// domain): 156 us with the nodes in shared memory, now 25 us.
 static_assert(sizeof(TailRun) / 4 <= TAIL_THREADS, "a thread a word");
+constexpr int INV_SMEM = 100;          // unknowns up to which the inverse is copied into shared memory (40 KB)
+constexpr int GS_DIM = 64;             // rows and radial nodes up to which the sweeps run in registers
+static_assert(GS_DIM / 4 * 32 <= TAIL_THREADS && GS_DIM == 2 * 32, "four rows a warp, two columns a lane");
 
 struct TailLevel {
     float *e, *f, *r, *ap, *am, *b, *d;
@@ -568,8 +567,79 @@ __device__ __forceinline__ void tail_half_sweep(const TailLevel& L, const TailNo
     __syncthreads();
 }
 
+// `sweeps` Gauss-Seidel sweeps (color 0, then 1) from zero on a grid of at most
+// GS_DIM rows (the cathode's included) and radial nodes, the operations of
+// tail_half_sweep.  The sweeps are a serial chain, so the nodes stay in registers:
+// four rows a warp, two columns a lane; a half-sweep exchanges columns by
+// shuffles and each warp's outer rows through shared memory, one barrier of the
+// sweeping warps.  15 x 60 cells, 200 sweeps, whole kernel: 51 us with a node a
+// thread in shared memory, 35-41 us by a single warp (no barrier; its FMAs
+// bound it), 25 us.
+__device__ __forceinline__ void tail_sweeps_rows(const TailLevel& L, int sweeps, int warps) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x / 32, W = L.nr + 1;
+    __shared__ float first[GS_DIM / 4 + 2][2][32], last[GS_DIM / 4 + 2][2][32];    // rows of warp w at w + 1, by column
+    float x[2][6], f[2][6], d[2][6], ap[2], am[2], b[2];        // [1 + k]: row 4 w + k
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const int j = 2 * lane + c;
+        const bool in = j < W;
+        const float dj = in ? L.d[j] : 0.0f;
+        ap[c] = j < L.nr ? L.ap[j] : 0.0f;
+        am[c] = in && j > 0 ? L.am[j] : 0.0f;
+        b[c] = in ? L.b[j] : 0.0f;
+        x[c][0] = x[c][5] = 0.0f;
+#pragma unroll
+        for (int k = 1; k < 5; ++k) {
+            const int i = 4 * w + k - 1;
+            const bool inner = in && i >= 1 && i < L.nz;        // others stay zero
+            x[c][k] = 0.0f;
+            f[c][k] = inner ? L.f[i * W + j] : 0.0f;
+            d[c][k] = inner ? dj : 0.0f;
+        }
+        if (w == 0) last[0][c][lane] = 0.0f;
+        if (w == warps - 1) first[warps + 1][c][lane] = 0.0f;
+    }
+    // rows of parity o of the lane's column c
+    auto half = [&](int c, int o) {
+#pragma unroll
+        for (int k = o ? 2 : 1; k < 5; k += 2) {
+            const float same = x[1 - c][k];
+            const float other = c ? __shfl_down_sync(0xFFFFFFFFu, same, 1) : __shfl_up_sync(0xFFFFFFFFu, same, 1);
+            float v = fmaf(ap[c], c ? other : same, f[c][k]);
+            v = fmaf(am[c], c ? same : other, v);
+            v = fmaf(b[c], x[c][k + 1], v);
+            v = fmaf(b[c], x[c][k - 1], v);
+            x[c][k] = v * d[c][k];
+        }
+        if (o == 0) first[w + 1][c][lane] = x[c][1];
+        else last[w + 1][c][lane] = x[c][4];
+    };
+    // the neighbours' rows, after even rows of column c and odd ones of the other
+    auto meet = [&](int c) {
+        asm volatile("bar.sync 1, %0;" ::"r"(32 * warps) : "memory");
+        x[c][5] = first[w + 2][c][lane];
+        x[1 - c][0] = last[w][1 - c][lane];
+    };
+#pragma unroll 1
+    for (int it = 0; it < sweeps; ++it) {
+        half(0, 0);
+        half(1, 1);
+        meet(0);
+        half(1, 0);
+        half(0, 1);
+        meet(1);
+    }
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int k = 1; k < 5; ++k) {
+            const int i = 4 * w + k - 1, j = 2 * lane + c;
+            if (i >= 1 && i < L.nz && j < W) L.e[i * W + j] = x[c][k];
+        }
+}
+
 __global__ void __launch_bounds__(TAIL_THREADS) k_mg_tail(const TailRun* runs, const int* done, int sweeps) {
-    extern __shared__ float sm[];
+    extern __shared__ __align__(16) float sm[];
     __shared__ TailRun R;
     __shared__ TailLevel tl[MG_MAX_LEVELS];
     const int run = blockIdx.x;
@@ -593,7 +663,12 @@ __global__ void __launch_bounds__(TAIL_THREADS) k_mg_tail(const TailRun* runs, c
         t.d = t.b + W;
     }
     // inputs: the coefficients (packed as they lie in shared memory), zero
-    // corrections, f of the first level
+    // corrections, f of the first level; a small inverse on its way meanwhile
+    if (R.inv_off >= 0)
+        for (int k = threadIdx.x; k < R.inv_len / 4; k += TAIL_THREADS) {
+            const uint32_t dst = (uint32_t)__cvta_generic_to_shared(sm + R.inv_off + 4 * k);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(R.inv + 4 * k) : "memory");
+        }
     for (int k = threadIdx.x; k < R.ncoef; k += TAIL_THREADS) sm[k] = __ldg(&R.coef[k]);
     {
         const int nodes0 = (R.nz[0] + 1) * (R.nr[0] + 1);
@@ -648,7 +723,11 @@ __global__ void __launch_bounds__(TAIL_THREADS) k_mg_tail(const TailRun* runs, c
         const TailLevel L = tl[n - 1];
         const int W = L.nr + 1;
         const int m = (L.nz - 1) * W;
-        const float* Ai = R.inv;
+        const float* Ai = R.inv_off >= 0 ? sm + R.inv_off : R.inv;
+        if (R.inv_off >= 0) {
+            asm volatile("cp.async.wait_all;\n" ::: "memory");
+            __syncthreads();
+        }
         if (Ai) {
             // e = A^-1 f: P threads per unknown, each summing every P-th
             // term (their loads in flight together), then a shuffle sum
@@ -664,6 +743,10 @@ __global__ void __launch_bounds__(TAIL_THREADS) k_mg_tail(const TailRun* runs, c
                 for (int o = P >> 1; o > 0; o >>= 1) acc += __shfl_down_sync(0xFFFFFFFFu, acc, o, P);
                 if (part == 0 && u < m) L.e[W + u] = acc;
             }
+            __syncthreads();
+        } else if (L.nz <= GS_DIM && W <= GS_DIM) {
+            const int warps = (L.nz + 3) / 4;
+            if ((int)threadIdx.x < 32 * warps) tail_sweeps_rows(L, sweeps, warps);
             __syncthreads();
         } else {
             tail_nodes(L, nd);
@@ -849,7 +932,7 @@ int field_init(FieldSolver& fs, const std::vector<pd_config>& cfgs, const std::v
     fs.max_nodes0 = 0;
     fs.max_cycles = cfgs[0].poisson_max_cycles > 0 ? cfgs[0].poisson_max_cycles : 60;
     std::vector<double> tol(R);
-    std::vector<TailRun> tails(R);
+    std::vector<TailRun> tails(R, TailRun{});
     for (int r = 0; r < R; ++r) {
         const pd_config& c = cfgs[r];
         int a[MG_MAX_LEVELS], b[MG_MAX_LEVELS], n;
@@ -858,7 +941,6 @@ int field_init(FieldSolver& fs, const std::vector<pd_config>& cfgs, const std::v
         fs.max_levels = std::max(fs.max_levels, n);
         fs.tail_lev[r] = tail_level(a, b, n);
         fs.max_tail = std::max(fs.max_tail, fs.tail_lev[r]);
-        fs.tail_smem = std::max(fs.tail_smem, tail_floats(a, b, n) * sizeof(float));
         fs.max_nodes0 = std::max(fs.max_nodes0, (c.nz + 1) * (c.nr + 1));
         tol[r] = c.poisson_tol;
         // level 0 in double
@@ -929,10 +1011,11 @@ int field_init(FieldSolver& fs, const std::vector<pd_config>& cfgs, const std::v
                 const int m = coarse_unknowns(a, b, n);
                 std::vector<double> Ai;
                 if (!invert_coarse(L.nz, L.nr, lap, lam, lbb, Ai)) return 1;
-                float* inv = (float*)take((size_t)m * m * 4);
+                float* inv = (float*)take((size_t)m * m * 4 + 16);
                 fai = to_float(Ai);
                 upload(inv, fai, s);
                 tails[r].inv = inv;
+                if (m <= INV_SMEM) tails[r].inv_len = (m * m + 3) / 4 * 4;
             }
             cudaStreamSynchronize(s);      // the host vectors above go out of scope
             if (l >= fs.tail_lev[r])
@@ -952,6 +1035,12 @@ int field_init(FieldSolver& fs, const std::vector<pd_config>& cfgs, const std::v
             o_coef += 4 * (b[l] + 1);
             o_node += 3 * (a[l] + 1) * (b[l] + 1);
         }
+        tr.inv_off = -1;
+        if (tr.inv_len) {
+            tr.inv_off = (o_node + 3) / 4 * 4;
+            o_node = tr.inv_off + tr.inv_len;
+        }
+        fs.tail_smem = std::max(fs.tail_smem, (size_t)o_node * sizeof(float));
         float* dcoef = (float*)take(coef.size() * 4);
         upload(dcoef, coef, s);
         cudaStreamSynchronize(s);
@@ -969,7 +1058,7 @@ int field_init(FieldSolver& fs, const std::vector<pd_config>& cfgs, const std::v
     int nred = 0;
     for (int r = 0; r < R; ++r) {
         red_base[r] = nred;
-        nred += (red_units(cfgs[r].nz, cfgs[r].nr) + 7) / 8;
+        nred += red_blocks(cfgs[r].nz, cfgs[r].nr);
     }
     fs.red = (double*)take((size_t)nred * 2 * 8);
     fs.bnorm = (double*)take((size_t)R * 8);
@@ -1000,9 +1089,12 @@ int field_init(FieldSolver& fs, const std::vector<pd_config>& cfgs, const std::v
     }
     fs.red_off = (int)tasks.size();
     for (int r = 0; r < R; ++r)
-        for (int u = 0; u < red_units(cfgs[r].nz, cfgs[r].nr); u += 8) tasks.push_back(make_int2(r, u));
+        for (int u = 0; u < red_units(cfgs[r].nz, cfgs[r].nr); u += RED_WARPS) tasks.push_back(make_int2(r, u));
     fs.red_len = (int)tasks.size() - fs.red_off;
-    if (fs.tail_smem > 48 * 1024) return 1;          // cannot happen: tail levels hold at most 34 x 34 nodes
+    // tail levels hold at most 34 x 34 nodes, the inverse 40 KB (10 KB are static)
+    if (fs.tail_smem > 36 * 1024 && cudaFuncSetAttribute(k_mg_tail, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                         (int)fs.tail_smem) != cudaSuccess)
+        return 1;
     fs.tasks = (int2*)take(tasks.size() * sizeof(int2) + 8);
     if (o > bytes) return 1;
     upload(fs.tasks, tasks, s);
@@ -1053,7 +1145,7 @@ static int vcycle(FieldSolver& fs, cudaStream_t s) {
 }
 
 static void norms(FieldSolver& fs, RunState* rs, int cycle, cudaStream_t s) {
-    k_residual_norms<<<fs.red_len, 256, 0, s>>>(fs.top, fs.lev, fs.tasks + fs.red_off, fs.red_base, fs.red, fs.ticket,
+    k_residual_norms<<<fs.red_len, 32 * RED_WARPS, 0, s>>>(fs.top, fs.lev, fs.tasks + fs.red_off, fs.red_base, fs.red, fs.ticket,
                                                 fs.bnorm, fs.done, fs.tol, rs, cycle);
 }
 

@@ -42,6 +42,7 @@ struct TailRun {
     float* e;                            // its correction, or
     double* phi;                         // the run's potential when it is level 0
     const float* inv;                    // inverse of the coarsest operator (transposed), or null
+    int inv_off, inv_len;                // its place in shared memory (-1: read where it is) and floats to copy
 };
 
 struct FieldSolver {

@@ -422,6 +422,10 @@ def test_rz_poisson_matches_oracle(pd, xs, n, nr):
     (96, 112),     # 12 rows x 56 of the post-smoothing, one over
     (88, 56),      # ragged both ways
     (28, 448),     # many column tiles, coarsest level by Gauss-Seidel sweeps
+    (120, 480),    # sweeps with the nodes in registers: 15 x 60 cells
+    (240, 60),     # 60 x 15
+    (15, 63),      # ... at most 64 radial nodes
+    (13, 64),      # ... one more
     (1024, 1024),  # long windows (from 608 tiles a level)
 ])
 def test_rz_poisson_residual_on_tile_edges(pd, xs, nz, nr):
@@ -458,6 +462,49 @@ def test_rz_poisson_residual_on_tile_edges(pd, xs, nz, nr):
     assert sc["poisson_relres"] <= 1e-9
     # rounding of r's terms: a few 1e-16 of |A| |phi|, far below 1e-9 |b|
     assert rel <= 1.01e-9, rel
+
+
+@pytest.mark.parametrize("nz,nr", [(64, 13), (65, 13), (6, 60)])
+def test_rz_poisson_sweeps_on_the_coarsest_grid(pd, xs, nz, nr):
+    """Grids that are their own coarsest level, up to 64 rows (swept in
+    registers) and above: the solve is `cycles` times 200 Gauss-Seidel sweeps
+    from zero, here in float64.  It need not converge on 64 rows."""
+    cfg, parts = synthetic.rz_plume(n=nz, total=5e3, seed=4)
+    keep = parts["ir"] < nr
+    parts = {k: v[keep] for k, v in parts.items()}
+    cfg.update(nr=nr, field_on=1, inject_on=0, poisson_tol=1e-9)
+    sim = pd.Simulation(cfg, xs)
+    sim.load(parts)
+    sim.step(0)
+    phi, (qe, qh) = sim.phi(), sim.rho()
+    d, j = cfg["dz"], np.arange(nr + 1)
+    ap, am = 2 * np.pi * (j + 0.5) * d, 2 * np.pi * (j - 0.5) * d
+    ap[-1] = am[0] = 0.0
+    area = 2 * np.pi * j * d * d
+    area[0], area[-1] = np.pi * d * d / 4, np.pi * d * d * (nr - 0.25)
+    verb = 2 * np.pi * d ** 3 * j
+    verb[0], verb[-1] = np.pi * d ** 3 / 3, 2 * np.pi * d ** 3 * (nr / 2 - 1 / 6)
+    b = 1.602176634e-19 * cfg["weight"] / 2.0 ** 32 * (qe + qh) * (area * d / (verb * 8.8541878128e-12))
+    b[-2] += area / d * phi[-1]
+    diag = ap + am + 2 * area / d
+    color = (np.arange(nz + 1)[:, None] + j) % 2
+
+    def off(p):
+        r = np.zeros_like(p)
+        r[1:-1] = area / d * (p[2:] + p[:-2])
+        r[1:-1, :-1] += ap[:-1] * p[1:-1, 1:]
+        r[1:-1, 1:] += am[1:] * p[1:-1, :-1]
+        return r
+
+    p = np.zeros_like(phi)
+    for _ in range(200 * int(sim.scalars()["poisson_cycles"])):
+        for c in (0, 1):
+            at = color == c
+            at[0] = at[-1] = False
+            p[at] = ((b + off(p)) / diag)[at]
+    # float sweeps: an update rounds off a few 2^-24 of the largest value, a sweep
+    # keeps up to 1 - 1.2e-3 of that (64 rows), a cycle of 200 sweeps 0.79
+    assert np.abs(phi - p)[1:-1].max() <= 1e-3 * np.abs(p).max()
 
 
 @pytest.mark.parametrize("n,nr", [(64, 64), (120, 480)])
