@@ -1009,31 +1009,31 @@ __device__ __forceinline__ bool coulomb_turn(V3& va, V3& vb, float Kn, float fa,
 // species i.
 constexpr int COUL_NCLS = 21;
 constexpr int COUL_NLIST = 6;
-// charged particles of a cell whose velocities its warp holds in shared
-// memory (in the words of its rank-table sort buffer, free once the tables
-// are built)
-constexpr int COUL_CACHE = 384;
-constexpr int COUL_WARPS = 4;           // warps of a k_coulomb block
-// words of a warp's buffer: the rank-table sort of a register-cached list,
-// then the velocity cache (three floats and a flag byte per particle)
-constexpr int COUL_SORT_WORDS = 4 * RANK_WARP_MAX + 256, COUL_CACHE_WORDS = (COUL_CACHE * 13 + 3) / 4;
+// A warp's batch of cells: at most 32 classes and 32 lists, and, unless it is one
+// cell, COUL_CACHE charged particles, whose velocities the warp holds in shared
+// memory (in the words of its rank-table sort buffer, free once the tables are
+// built; then COUL_MASKS words of the conflict table)
+constexpr int COUL_CACHE = 336, COUL_MASKS = 256;
+constexpr int COUL_CELLS = 10;          // most cells of a warp: with electrons and Cu+ their 30 classes fill a batch
+constexpr int COUL_BLOCKS = 22;         // blocks (of a warp) an SM
+constexpr int COUL_SORT_WORDS = 4 * RANK_WARP_MAX + 256, COUL_CACHE_WORDS = 3 * COUL_CACHE + COUL_MASKS;
 constexpr int COUL_SBUF = COUL_SORT_WORDS > COUL_CACHE_WORDS ? COUL_SORT_WORDS : COUL_CACHE_WORDS;
 
 struct CoulClass {
     uint4 k1, k2;          // permutation keys: of the one species; or of the more and the fewer
     float Kn, fa, fb;
-    uint32_t start;        // first pair in the cell's flattened order
-    uint32_t npairs;
     uint32_t P;            // one species: regular pairs; two: the fewer's count (a round)
     uint32_t N;            // one species: its count; two: the more numerous's
-    uint8_t la, lb;        // the lists of the pair's first and second particle
-    uint8_t cls, a_many;   // a_many: list la is the more numerous (la on a tie)
+    uint32_t lc;           // the cell's index in its run
+    uint32_t ba, na, ca;   // the list of a pair's first particle: first slot, count, place in the velocity cache
+    uint32_t bb, nb, cb;   // of its second
+    uint8_t cls, spa, spb;
+    uint8_t flags;         // 1: list a is the more numerous (a on a tie); 2, 4: the ids of list a, b ascend
 };
 struct CoulWarp {
-    CoulClass cl[COUL_NCLS];
-    uint32_t base[COUL_NLIST], n[COUL_NLIST];
-    uint32_t coff[COUL_NLIST], cn[COUL_NLIST];   // a list's place and count in the velocity cache
-    uint32_t sorted;       // bit l: list l's ids ascend (rank = position)
+    CoulClass cl[32];
+    uint32_t start[32];                 // a class's first pair in the batch's order
+    uint32_t lbase[32], lcoff[32];      // the lists: first slot, place in the cache
 };
 
 __device__ __forceinline__ void class_lists(int t, int& la, int& lb) {
@@ -1055,40 +1055,58 @@ __device__ __forceinline__ void class_lists(int t, int& la, int& lb) {
 __device__ __forceinline__ int list_species(int l) { return l == 0 ? SP_E : SP_CUP + l - 1; }
 
 // The Coulomb pairs (after all cells' DSMC classes: cells are independent,
-// so this is the order of cell-by-cell processing): one warp per cell with
-// charged particles, grid-stride over the cells, on the lists of the step's
+// so this is the order of cell-by-cell processing), on the lists of the step's
 // start; a particle whose species changed this step is left out.
-__global__ void __launch_bounds__(128, 6) k_coulomb(Particles A, RankScratch S, const uint32_t* __restrict__ off,
+//
+// Instructions bound it, and a cell has few pairs (ten to twenty with five
+// electrons and five ions).  A warp therefore collects cells (grid-stride) until
+// their classes or particles fill its tables and takes all their pairs together, a
+// lane a pair: their permutations, draws and lookups side by side, then their turns
+// in rounds.  A pair's turn waits for the earlier pairs of the chunk that share a
+// particle with it, no others: a pair of lane q sets bit q in the word of each of
+// its particles, and the lower bits in its two words are those it waits for (in a
+// cell beyond the cache particles share words, and the pairs named are compared).
+// Blocks of one warp and up to ten cells keep the SMs evenly loaded (cells differ).
+//
+// 256 x 512 cells of about eight electrons and eight Cu+ (lognormal), all pairs:
+// 826 us and 4060 instructions a cell with a warp a cell, its pairs in the
+// classes' waves of disjoint pairs (12.5 threads an instruction); 500 us and 2290
+// with batches and rounds; 450-475 us with blocks of one warp, at 22 an SM (20:
+// 490 us, 16: 530).  Of it the turns take 120 us, the rank tables 80, the
+// permutations 180 (their walks differ in length; tables of the permutations of
+// up to 16 places took as long to make).
+__global__ void __launch_bounds__(32, COUL_BLOCKS) k_coulomb(Particles A, RankScratch S, const uint32_t* __restrict__ off,
                                                    const uint32_t* __restrict__ cnt, DevState* st, KParams P,
-                                                   CollConsts cc, const double* __restrict__ cw) {
+                                                   CollConsts cc, const double* __restrict__ cw, uint32_t cells) {
     if (st->error) return;                           // a fault was flagged: the state is not stepped further
-    __shared__ __align__(16) uint32_t s_sort[COUL_WARPS][COUL_SBUF];   // per-warp rank-table sort, then velocity cache
-    __shared__ CoulWarp s_cw[COUL_WARPS];
-    const int lane = threadIdx.x & 31;
-    const int wib = (threadIdx.x >> 5) & (COUL_WARPS - 1);
-    uint32_t* sbuf = s_sort[wib];
-    CoulWarp& W = s_cw[wib];
-    const uint32_t C = P.ncell;
-    const uint32_t warp0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+    __shared__ __align__(16) uint32_t sbuf[COUL_SBUF];      // rank-table sort, then velocity cache and conflict table
+    __shared__ __align__(16) CoulWarp W;
+    const int lane = (int)threadIdx.x;
+    float* const cvz = reinterpret_cast<float*>(sbuf);
+    float* const cvr = cvz + COUL_CACHE;
+    float* const cvt = cvr + COUL_CACHE;
+    uint32_t* const mask = sbuf + 3 * COUL_CACHE;
+    const uint32_t C = P.ncell, step = st->step;
+    const uint32_t cell0 = blockIdx.x * cells, cell1 = min(cell0 + cells, C);
     unsigned lt;
     asm("mov.u32 %0, %%lanemask_lt;" : "=r"(lt));
-    for (uint32_t c = warp0; c < C; c += nwarps) {
+    int la = 0, lb = 0;                               // lane t < COUL_NCLS: the lists of class t
+    if (lane < COUL_NCLS) class_lists(lane, la, lb);
+    const int lsp = lane < COUL_NLIST ? list_species(lane) : NSP;
+    // the batch: run, classes, lists, particles, pairs
+    int run = 0, ncl = 0, nlist = 0;
+    uint32_t tot = 0, T = 0;
+    uint32_t n_ee = 0, n_ei = 0, n_ii = 0, n_fb = 0;
+    for (uint32_t c = cell0;; ++c) {
+        const bool end = c >= cell1;
         // the cell's charged lists (lane l reads list l)
         uint32_t nl = 0, bl = 0;
-        if (lane < COUL_NLIST) {
-            const int sp = list_species(lane);
-            if (sp < P.nsp) {
-                const uint32_t b = (uint32_t)sp * C + c;
-                nl = cnt[b];
-                bl = off[b];
-            }
+        if (!end && lsp < P.nsp) {
+            const uint32_t b = (uint32_t)lsp * C + c;
+            nl = cnt[b];
+            bl = off[b];
         }
-        const uint32_t Ne = __shfl_sync(FULL, nl, 0);
-        if (Ne == 0u && !P.heavy_step) continue;
-        // the class table: lane t takes class t
-        int la = 0, lb = 0;
-        if (lane < COUL_NCLS) class_lists(lane, la, lb);
+        // lane t: class t's pairs
         const uint32_t Na = __shfl_sync(FULL, nl, la), Nb = __shfl_sync(FULL, nl, lb);
         bool on = false;
         uint32_t np = 0, Pk = 0, Nk = 0;
@@ -1108,192 +1126,226 @@ __global__ void __launch_bounds__(128, 6) k_coulomb(Particles A, RankScratch S, 
             }
         }
         const unsigned mact = __ballot_sync(FULL, on);
-        if (mact == 0u) continue;
-        const int r = run_of(P, c);
-        const RunInfo* RI = &P.runs[r];
-        const uint32_t lc = c - RI->cell_base;
-        if (!on) np = 0;
-        uint32_t incl = np;
+        if (mact == 0u && !end) continue;
+        const unsigned used = __reduce_or_sync(FULL, on ? (1u << la) | (1u << lb) : 0u);
+        // the used lists' places in the cache, the classes' first pairs
+        uint32_t ncum = (used >> lane) & 1u ? nl : 0u, pcum = on ? np : 0u;
+        const uint32_t nown = ncum, pown = pcum;
+#pragma unroll
+        for (int d = 1; d < 8; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(FULL, ncum, d);
+            if (lane >= d) ncum += y;
+        }
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
-            const uint32_t y = __shfl_up_sync(FULL, incl, d);
-            if (lane >= d) incl += y;
+            const uint32_t y = __shfl_up_sync(FULL, pcum, d);
+            if (lane >= d) pcum += y;
         }
-        const uint32_t T = __shfl_sync(FULL, incl, 31);
-        const int nact = __popc(mact);
-        if (on) {
-            const uint32_t row = RI->row_base + lc % (uint32_t)RI->nr;
-            const double w = lane < 6 ? cw[row] : cw[P.cw_heavy + row];
-            const uint32_t Nf = la == lb ? Na : min(Na, Nb);
-            CoulClass K;
-            Stream ps(lc, st->step, SID_COUL_PERM | (uint32_t)lane, RI->seed, RI->run);
-            K.k1 = make_uint4(ps.next(), ps.next(), ps.next(), ps.next());
-            K.k2 = make_uint4(0u, 0u, 0u, 0u);
-            if (la != lb) K.k2 = make_uint4(ps.next(), ps.next(), ps.next(), ps.next());
-            K.Kn = (float)(cc.kc[lane] * (double)Nf * w);
-            K.fa = lane >= 1 && lane < 6 ? cc.a_e : 0.5f;
-            K.fb = lane >= 1 && lane < 6 ? cc.a_t : 0.5f;
-            K.start = incl - np;
-            K.npairs = np;
-            K.P = Pk;
-            K.N = Nk;
-            K.la = (uint8_t)la;
-            K.lb = (uint8_t)lb;
-            K.cls = (uint8_t)lane;
-            K.a_many = a_many ? 1 : 0;
-            W.cl[__popc(mact & lt)] = K;
+        const uint32_t ctot = __shfl_sync(FULL, ncum, COUL_NLIST - 1), cT = __shfl_sync(FULL, pcum, 31);
+        const int r = end ? run : run_of(P, c);
+        if (ncl > 0 && (end || r != run || ncl + __popc(mact) > 32 || nlist + __popc(used) > 32 ||
+                        tot + ctot > (uint32_t)COUL_CACHE)) {
+            const RunInfo* RI = &P.runs[run];
+            __syncwarp();
+            // the classes' keys
+            uint32_t cs = 0xFFFFFFFFu;
+            if (lane < ncl) {
+                CoulClass& K = W.cl[lane];
+                Stream ps(K.lc, step, SID_COUL_PERM | (uint32_t)K.cls, RI->seed, RI->run);
+                K.k1 = make_uint4(ps.next(), ps.next(), ps.next(), ps.next());
+                if (K.spa != K.spb) K.k2 = make_uint4(ps.next(), ps.next(), ps.next(), ps.next());
+                const uint32_t row = RI->row_base + K.lc % (uint32_t)RI->nr;
+                const double w = K.cls < 6 ? cw[row] : cw[P.cw_heavy + row];
+                K.Kn = (float)(cc.kc[K.cls] * (double)(K.spa == K.spb ? K.N : K.P) * w);
+                const bool ei = K.cls >= 1 && K.cls < 6;
+                K.fa = ei ? cc.a_e : 0.5f;
+                K.fb = ei ? cc.a_t : 0.5f;
+                cs = W.start[lane];
+            }
+            const uint32_t ls = lane < nlist ? W.lcoff[lane] : 0xFFFFFFFFu;
+            const uint32_t lo = lane < nlist ? W.lbase[lane] - W.lcoff[lane] : 0u;      // slot of cache place 0
+            // which of the batch's classes (lists) an index belongs to: those that
+            // start at or before it, of which the first lanes hold the starts in order
+            auto owner = [&](uint32_t starts, uint32_t i0) -> int {
+                const int before = __popc(__ballot_sync(FULL, starts < i0));
+                const uint32_t here = starts - i0 < 32u ? 1u << (starts - i0) : 0u;
+                const uint32_t m = __reduce_or_sync(FULL, starts >= i0 ? here : 0u);
+                return before + __popc(m & (lt | (1u << lane))) - 1;
+            };
+            const bool cached = tot <= (uint32_t)COUL_CACHE;
+            if (cached)
+                for (uint32_t i0 = 0; i0 < tot; i0 += 32) {
+                    const uint32_t i = i0 + (uint32_t)lane, slot = __shfl_sync(FULL, lo, owner(ls, i0)) + i;
+                    if (i < tot) {
+                        cvz[i] = A.vz[slot];
+                        cvr[i] = A.vr[slot];
+                        cvt[i] = A.vt[slot];
+                    }
+                }
+            for (int k = lane; k < COUL_MASKS; k += 32) mask[k] = 0u;
+            __syncwarp();
+            float* VZ = cached ? cvz : A.vz;
+            float* VR = cached ? cvr : A.vr;
+            float* VT = cached ? cvt : A.vt;
+#pragma unroll 1
+            for (uint32_t c0 = 0; c0 < T; c0 += 32) {
+                // lane q: pair c0 + q's particles and draws
+                const uint32_t p = c0 + (uint32_t)lane;
+                const int j = owner(cs, c0);
+                const CoulClass& K = W.cl[j];
+                uint32_t ia = 0, ib = 0;
+                float z = 0.0f, cph = 1.0f, sph = 0.0f, Kn = 0.0f;
+                bool valid = false, fail = false;
+                if (p < T) {
+                    const uint32_t k = p - W.start[j];
+                    uint32_t ra, rb;
+                    Kn = K.Kn;
+                    if (K.spa == K.spb) {
+                        const uint32_t N = K.N;
+                        const int h = perm_bits(N);
+                        uint32_t xa = 2u * k, xb = 2u * k + 1u;
+                        if (k >= K.P) {              // the closing triple: pair q joins q and q + 1 (mod 3)
+                            const uint32_t q = k - K.P;
+                            xa = N - 3u + q;
+                            xb = N - 3u + (q + 1u) % 3u;
+                            Kn = Kn * 0.5f;
+                        }
+                        perm_index2(xa, N, K.k1, h, xb, N, K.k1, h, ra, rb);
+                    } else {
+                        uint32_t m, f;
+                        perm_index2(k, K.N, K.k1, perm_bits(K.N), k % K.P, K.P, K.k2, perm_bits(K.P), m, f);
+                        ra = K.flags & 1u ? m : f;
+                        rb = K.flags & 1u ? f : m;
+                    }
+                    const uint32_t pa = K.flags & 2u ? ra : S.table[K.ba + ra];
+                    const uint32_t pb = K.flags & 4u ? rb : S.table[K.bb + rb];
+                    // the draws do not depend on the particles: they are computed
+                    // while the rank lookups are in flight (and dropped for a pair
+                    // that does not take place)
+                    coul_draws(K.lc, step, sid_coul(K.cls, k), RI->seed, RI->run, z, cph, sph, fail);
+                    if (pa < K.na && pb < K.nb) {
+                        const uint32_t ka = A.key[K.ba + pa], kb = A.key[K.bb + pb];
+                        valid = !(ka & KEY_FLAG) && key_species(ka) == K.spa && !(kb & KEY_FLAG) &&
+                                key_species(kb) == K.spb;
+                        ia = (cached ? K.ca : K.ba) + pa;
+                        ib = (cached ? K.cb : K.bb) + pb;
+                    } else {
+                        set_error(st, ERR_BOUNDS);   // ids not unique: corrupt state, never index with it
+                    }
+                }
+                const float fa = K.fa, fb = K.fb;
+                const int cls = K.cls;
+                uint32_t* const ma = mask + ia % COUL_MASKS;
+                uint32_t* const mb = mask + ib % COUL_MASKS;
+                if (valid) {
+                    atomicOr(ma, 1u << lane);
+                    atomicOr(mb, 1u << lane);
+                }
+                __syncwarp();
+                uint32_t wait = (*ma | *mb) & lt;
+                if (!cached) {
+                    // full words: the lanes that another's bits name, compared one by one
+                    uint32_t same = 0;
+                    for (unsigned named = __reduce_or_sync(FULL, valid ? wait : 0u); named; named &= named - 1u) {
+                        const int q = __ffs((int)named) - 1;
+                        const uint32_t qa = __shfl_sync(FULL, ia, q), qb = __shfl_sync(FULL, ib, q);
+                        if (qa == ia || qa == ib || qb == ia || qb == ib) same |= 1u << q;
+                    }
+                    wait &= same;
+                }
+                __syncwarp();
+                if (valid) *ma = *mb = 0u;
+                unsigned todo = __ballot_sync(FULL, valid);
+#pragma unroll 1
+                while (todo) {
+                    const bool now = (todo >> lane & 1u) && !(wait & todo);
+                    if (now) {
+                        V3 va{VZ[ia], VR[ia], VT[ia]}, vb{VZ[ib], VR[ib], VT[ib]};
+                        if (coulomb_turn(va, vb, Kn, fa, fb, z, cph, sph)) {
+                            VZ[ia] = va.x; VR[ia] = va.y; VT[ia] = va.z;
+                            VZ[ib] = vb.x; VR[ib] = vb.y; VT[ib] = vb.z;
+                            if (cls == 0) ++n_ee;
+                            else if (cls < 6) ++n_ei;
+                            else ++n_ii;
+                            if (fail) ++n_fb;
+                        }
+                    }
+                    __syncwarp();
+                    todo &= ~__ballot_sync(FULL, now);
+                }
+            }
+            if (cached) {
+                // the velocities back to their slots
+                __syncwarp();
+                for (uint32_t i0 = 0; i0 < tot; i0 += 32) {
+                    const uint32_t i = i0 + (uint32_t)lane, slot = __shfl_sync(FULL, lo, owner(ls, i0)) + i;
+                    if (i < tot) {
+                        A.vz[slot] = cvz[i];
+                        A.vr[slot] = cvr[i];
+                        A.vt[slot] = cvt[i];
+                    }
+                }
+            }
+            __syncwarp();
+            if (end || r != run) {
+                const uint32_t ee = __reduce_add_sync(FULL, n_ee), ei = __reduce_add_sync(FULL, n_ei);
+                const uint32_t ii = __reduce_add_sync(FULL, n_ii), fb = __reduce_add_sync(FULL, n_fb);
+                n_ee = n_ei = n_ii = n_fb = 0;
+                if (lane == 0) {
+                    RunState& rsv = P.rs[run];
+                    if (ee) atomicAdd(&rsv.ctr[C_COUL_EE], (unsigned long long)ee);
+                    if (ei) atomicAdd(&rsv.ctr[C_COUL_EI], (unsigned long long)ei);
+                    if (ii) atomicAdd(&rsv.ctr[C_COUL_II], (unsigned long long)ii);
+                    if (fb) atomicAdd(&rsv.ctr[C_ISOFB], (unsigned long long)fb);
+                }
+            }
+            ncl = nlist = 0;
+            tot = T = 0;
         }
-        // lists any class uses: rank tables, then the velocities in shared
-        // memory when they fit
-        unsigned used = on ? ((1u << la) | (1u << lb)) : 0u;
-        used = __reduce_or_sync(FULL, used);
+        if (end) break;
+        run = r;
+        // the cell joins the batch: rank tables of the lists its classes use, then the entries
+        const RunInfo* RI = &P.runs[r];
         const uint32_t idn = P.rs[r].id_next;
         const int id_top = idn > 1u ? 31 - __clz((int)(idn - 1u)) : 0;
-        uint32_t sorted = 0, tot = 0;
-        for (int l = 0; l < COUL_NLIST; ++l) {
+        uint32_t sorted = 0;
+        for (unsigned u = used; u; u &= u - 1u) {
+            const int l = __ffs((int)u) - 1;
             const uint32_t n = __shfl_sync(FULL, nl, l), b = __shfl_sync(FULL, bl, l);
-            const bool u = (used >> l) & 1u;
-            if (lane == 0) {
-                W.base[l] = b;
-                W.n[l] = n;
-                W.coff[l] = tot;
-                W.cn[l] = u ? n : 0u;
-            }
-            if (!u) continue;
-            tot += n;
             IdList L;
             load_ids(L, A.id, b, n, n, S, sbuf, S.table + b, id_top, true);
             if (L.sorted) sorted |= 1u << l;
         }
-        if (lane == 0) W.sorted = sorted;
-        const bool cached = tot <= (uint32_t)COUL_CACHE;
-        float* const cvz = reinterpret_cast<float*>(sbuf);
-        float* const cvr = cvz + COUL_CACHE;
-        float* const cvt = cvr + COUL_CACHE;
-        uint8_t* const touched = reinterpret_cast<uint8_t*>(cvt + COUL_CACHE);
-        __syncwarp();
-        if (cached) {
-            for (int l = 0; l < COUL_NLIST; ++l) {
-                const uint32_t n = W.cn[l], b = W.base[l], co = W.coff[l];
-                for (uint32_t q = (uint32_t)lane; q < n; q += 32) {
-                    cvz[co + q] = A.vz[b + q];
-                    cvr[co + q] = A.vr[b + q];
-                    cvt[co + q] = A.vt[b + q];
-                    touched[co + q] = 0;
-                }
-            }
+        const uint32_t coff = tot + ncum - nown;
+        const uint32_t ba = __shfl_sync(FULL, bl, la), bb = __shfl_sync(FULL, bl, lb);
+        const uint32_t ca = __shfl_sync(FULL, coff, la), cb = __shfl_sync(FULL, coff, lb);
+        if (on) {
+            const int e = ncl + __popc(mact & lt);
+            CoulClass& K = W.cl[e];
+            K.P = Pk;
+            K.N = Nk;
+            K.lc = c - RI->cell_base;
+            K.ba = ba;
+            K.na = Na;
+            K.ca = ca;
+            K.bb = bb;
+            K.nb = Nb;
+            K.cb = cb;
+            K.cls = (uint8_t)lane;
+            K.spa = (uint8_t)list_species(la);
+            K.spb = (uint8_t)list_species(lb);
+            K.flags = (uint8_t)((a_many ? 1u : 0u) | ((sorted >> la) & 1u) << 1 | ((sorted >> lb) & 1u) << 2);
+            W.start[e] = T + pcum - pown;
         }
-        __syncwarp();
-        float* VZ = cached ? cvz : A.vz;
-        float* VR = cached ? cvr : A.vr;
-        float* VT = cached ? cvt : A.vt;
-        uint32_t n_ee = 0, n_ei = 0, n_ii = 0, n_fb = 0;
-        int jw = 0;                      // the class of the wave being applied
-        for (uint32_t c0 = 0; c0 < T; c0 += 32) {
-            // lane q: pair c0 + q's particles and draws
-            const uint32_t p = c0 + (uint32_t)lane;
-            uint32_t ia = 0, ib = 0;
-            float z = 0.0f, cph = 1.0f, sph = 0.0f, Kn = 0.0f;
-            bool valid = false, fail = false;
-            if (p < T) {
-                int j = 0;
-                while (j + 1 < nact && W.cl[j + 1].start <= p) ++j;
-                const CoulClass& K = W.cl[j];
-                const uint32_t k = p - K.start;
-                uint32_t ra, rb;
-                Kn = K.Kn;
-                if (K.la == K.lb) {
-                    const uint32_t N = K.N;
-                    const int h = perm_bits(N);
-                    uint32_t xa = 2u * k, xb = 2u * k + 1u;
-                    if (k >= K.P) {              // the closing triple: pair q joins q and q + 1 (mod 3)
-                        const uint32_t q = k - K.P;
-                        xa = N - 3u + q;
-                        xb = N - 3u + (q + 1u) % 3u;
-                        Kn = Kn * 0.5f;
-                    }
-                    perm_index2(xa, N, K.k1, h, xb, N, K.k1, h, ra, rb);
-                } else {
-                    uint32_t m, f;
-                    perm_index2(k, K.N, K.k1, perm_bits(K.N), k % K.P, K.P, K.k2, perm_bits(K.P), m, f);
-                    ra = K.a_many ? m : f;
-                    rb = K.a_many ? f : m;
-                }
-                const int la_ = K.la, lb_ = K.lb;
-                const uint32_t na = W.n[la_], nb = W.n[lb_], ba = W.base[la_], bb = W.base[lb_];
-                const uint32_t pa = (W.sorted >> la_) & 1u ? ra : S.table[ba + ra];
-                const uint32_t pb = (W.sorted >> lb_) & 1u ? rb : S.table[bb + rb];
-                // the draws do not depend on the particles: they are computed
-                // while the rank lookups are in flight (and dropped for a pair
-                // that does not take place)
-                coul_draws(lc, st->step, sid_coul(K.cls, k), RI->seed, RI->run, z, cph, sph, fail);
-                if (pa < na && pb < nb) {
-                    const uint32_t ka = A.key[ba + pa], kb = A.key[bb + pb];
-                    valid = !(ka & KEY_FLAG) && (int)key_species(ka) == list_species(la_) && !(kb & KEY_FLAG) &&
-                            (int)key_species(kb) == list_species(lb_);
-                    ia = cached ? W.coff[la_] + pa : ba + pa;
-                    ib = cached ? W.coff[lb_] + pb : bb + pb;
-                } else {
-                    set_error(st, ERR_BOUNDS);   // ids not unique: corrupt state, never index with it
-                }
-                if (!valid) fail = false;
-            }
-            // the chunk's pairs in waves, in order
-            const uint32_t c1 = min(c0 + 32u, T);
-            for (uint32_t pw = c0; pw < c1;) {
-                while (pw >= W.cl[jw].start + W.cl[jw].npairs) ++jw;
-                const CoulClass& K = W.cl[jw];
-                const uint32_t k = pw - K.start;
-                uint32_t we;
-                if (K.la == K.lb) we = k < K.P ? K.start + K.P : pw + 1u;
-                else we = K.start + min((k / K.P + 1u) * K.P, K.N);
-                const uint32_t e = min(we, c1);
-                const int src = (int)(pw - c0) + lane;
-                const uint32_t wa = __shfl_sync(FULL, ia, src & 31), wb = __shfl_sync(FULL, ib, src & 31);
-                const float wz = __shfl_sync(FULL, z, src & 31), wc = __shfl_sync(FULL, cph, src & 31);
-                const float ws = __shfl_sync(FULL, sph, src & 31), wk = __shfl_sync(FULL, Kn, src & 31);
-                const bool wv = __shfl_sync(FULL, valid, src & 31), wf = __shfl_sync(FULL, fail, src & 31);
-                if (pw + (uint32_t)lane < e && wv) {
-                    V3 va{VZ[wa], VR[wa], VT[wa]}, vb{VZ[wb], VR[wb], VT[wb]};
-                    if (coulomb_turn(va, vb, wk, K.fa, K.fb, wz, wc, ws)) {
-                        VZ[wa] = va.x; VR[wa] = va.y; VT[wa] = va.z;
-                        VZ[wb] = vb.x; VR[wb] = vb.y; VT[wb] = vb.z;
-                        if (cached) {
-                            touched[wa] = 1;
-                            touched[wb] = 1;
-                        }
-                        if (K.cls == 0) ++n_ee;
-                        else if (K.cls < 6) ++n_ei;
-                        else ++n_ii;
-                        if (wf) ++n_fb;
-                    }
-                }
-                __syncwarp();
-                pw = e;
-            }
+        if ((used >> lane) & 1u) {
+            const int e = nlist + __popc(used & lt);
+            W.lbase[e] = bl;
+            W.lcoff[e] = coff;
         }
-        if (cached) {
-            // the velocities the pairs changed back to their slots
-            for (uint32_t i = (uint32_t)lane; i < tot; i += 32) {
-                if (!touched[i]) continue;
-                int l = 0;
-                while (i >= W.coff[l] + W.cn[l]) ++l;
-                const uint32_t slot = W.base[l] + (i - W.coff[l]);
-                A.vz[slot] = cvz[i];
-                A.vr[slot] = cvr[i];
-                A.vt[slot] = cvt[i];
-            }
-        }
-        __syncwarp();
-        const uint32_t ee = __reduce_add_sync(FULL, n_ee), ei = __reduce_add_sync(FULL, n_ei);
-        const uint32_t ii = __reduce_add_sync(FULL, n_ii), fb = __reduce_add_sync(FULL, n_fb);
-        if (lane == 0) {
-            RunState& rsv = P.rs[r];
-            if (ee) atomicAdd(&rsv.ctr[C_COUL_EE], (unsigned long long)ee);
-            if (ei) atomicAdd(&rsv.ctr[C_COUL_EI], (unsigned long long)ei);
-            if (ii) atomicAdd(&rsv.ctr[C_COUL_II], (unsigned long long)ii);
-            if (fb) atomicAdd(&rsv.ctr[C_ISOFB], (unsigned long long)fb);
-        }
+        ncl += __popc(mact);
+        nlist += __popc(used);
+        tot += ctot;
+        T += cT;
     }
 }
 
@@ -1918,8 +1970,10 @@ void launch_coulomb(const Particles& A, const Particles& B, const uint32_t* off,
                     const KParams& P, const CollConsts& cc, const double* cw, int sms, cudaStream_t s) {
     const RankScratch S{B.key, reinterpret_cast<uint32_t*>(B.pz), reinterpret_cast<uint32_t*>(B.pr),
                         reinterpret_cast<uint32_t*>(B.vz), B.id};
-    // one wave of resident blocks, grid-stride over the cells
-    k_coulomb<<<sms * 6, 32 * COUL_WARPS, 0, s>>>(A, S, off, cnt, st, P, cc, cw);
+    // a full batch a warp; fewer cells where that would leave the SMs short of warps
+    // (four steps of 97 x 131 cells 2.17 -> 1.80 ms, of 41 x 43 cells 1.05 -> 0.80)
+    const uint32_t cells = std::min<uint32_t>(std::max<uint32_t>(P.ncell / (uint32_t)(sms * COUL_BLOCKS), 1u), COUL_CELLS);
+    k_coulomb<<<(P.ncell + cells - 1) / cells, 32, 0, s>>>(A, S, off, cnt, st, P, cc, cw, cells);
 }
 void launch_finalize(const uint32_t* off, uint32_t nbins, const uint32_t* cand_off, DevState* st, const KParams& P,
                      const RunCircuit* circ, double dt, int circuit, cudaStream_t s) {

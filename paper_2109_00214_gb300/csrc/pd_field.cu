@@ -147,8 +147,9 @@ size_t field_workspace_bytes(const std::vector<int>& nz, const std::vector<int>&
 // level 0's f = r (float).  A warp takes 32 radial nodes and marches over
 // RED_ROWS rows, so that each node of phi is read once a row, not three times;
 // double arithmetic (seven operations a node) bounds it, and small units spread it
-// over the SMs: 120 x 480 cells 11.8 us with 8 rows a warp and 8 warps a block, 8.8.  Work list of (run, first unit), four units a block; the block that finishes a
-// run's last units sums the blocks' parts in their order and judges the run:
+// over the SMs: 120 x 480 cells 11.8 us with 8 rows a warp and 8 warps a block, 8.8
+// now.  Work list of (run, first unit), four units a block; the block that finishes
+// a run's last units sums the blocks' parts in their order and judges the run:
 // relres = |r| / |b|, converged flag, bookkeeping.
 // 512 x 512 cells, device time of a launch under ncu: 14.7 us with the norm (13.8
 // + 8.9 us as a launch of rows and one of norms).

@@ -208,3 +208,32 @@ def test_ensemble_sputtering_per_run_matches_oracle(pd, xs):
         for key in oc:
             assert gc[key] == oc[key], (k, key, gc[key], oc[key])
         assert gc["sput_cathode"] > 0
+
+
+def test_ensemble_coulomb_per_run_matches_oracle(pd, xs):
+    """Runs whose cells end inside a warp's ten: Coulomb pairs and their
+    counters are those of the run simulated alone."""
+    runs = _runs(field_on=2, sizes=(9, 13, 32))
+    for c, _ in runs:
+        c.update(coulomb=1, heavy_subcycle=2)
+    fields = [_field(c, 3 + k) for k, (c, _) in enumerate(runs)]
+    ens = _ensemble(pd, runs, xs, fields)
+    ens.step(3)
+    per_run = _split(ens, ens.particles())
+    for k, (cfg, parts) in enumerate(runs):
+        o = oracle.Oracle(cfg, fp64=False)
+        o.set_cross_sections(xs)
+        o.load(parts)
+        o.set_field(*fields[k])
+        o.prime()
+        o.step(3)
+        op, g = o.particles(), per_run[k]
+        assert len(g["id"]) == len(op["id"]), k
+        for key in ("id", "species", "iz", "ir"):
+            assert np.array_equal(g[key], op[key]), (k, key)
+        for key in FLOATS:
+            assert np.array_equal(g[key].astype(np.float64), op[key]), (k, key)
+        gc, oc = ens.run_counters(k), o.counters()
+        for key in oc:
+            assert gc[key] == oc[key], (k, key, gc[key], oc[key])
+        assert gc["coul_ee"] > 0 and gc["coul_ei"] > 0

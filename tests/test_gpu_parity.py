@@ -290,6 +290,26 @@ def test_dense_coulomb_cells_bit_exact(pd, xs, n_e, n_t, ncells):
     assert_same_particles(sim.particles(), o.particles())
 
 
+@pytest.mark.parametrize("n_e,n_t,ncells", [
+    (200, 136, 3),                 # a cell's charged particles just fill the velocity cache
+    (200, 137, 3),                 # ... one more: velocities in place
+    (6, 5, 23),                    # ten cells a batch, three in the last
+    (1, 1, 11),                    # one pair a cell
+])
+def test_coulomb_batches_bit_exact(pd, xs, n_e, n_t, ncells):
+    cfg, parts = synthetic.rate_cell(n_e=n_e * ncells, n_t=n_t * ncells, Te_eV=5.0, seed=13, coll_scale=1.0,
+                                     target_species=2, ncells=ncells)
+    at = np.arange(len(parts["iz"]))                   # the same number of each species in every cell
+    for sp in (0, 2):
+        k = at[parts["species"] == sp]
+        parts["iz"][k], parts["ir"][k] = 0, np.arange(len(k)) % ncells
+    cfg.update(nz=2, nr=ncells, coulomb=1)
+    sim, o = run_pair(pd, cfg, parts, xs, 2)
+    assert_same_counters(sim.counters(), o.counters())
+    assert sim.counters()["coul_ei"] > 0
+    assert_same_particles(sim.particles(), o.particles())
+
+
 def _rz_field(n, V0, seed=3):
     rng = np.random.default_rng(seed)
     Ez = np.full((n + 1, n + 1), -V0 / 6e-6) * (1 + 0.3 * rng.uniform(-1, 1, (n + 1, n + 1)))
