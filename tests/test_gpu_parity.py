@@ -560,6 +560,24 @@ def test_empty_and_capacity(pd, xs):
         sim3.synchronize()
 
 
+@pytest.mark.parametrize("lo,hi,nbins", [(0.0, 200.0, 1), (0.0, 300.0, 4096), (3.7, 3.7001, 5), (12.5, 14.0, 333),
+                                         (-1.0, 1e-3, 64), (0.0, 1e9, 7)])
+def test_spectrum_bins_match_oracle(pd, xs, lo, hi, nbins):
+    """Bins and ranges from one to all, wide and narrow; energies on the bins' edges."""
+    cfg, parts = synthetic.microbench(nz=16, nr=24, total=2e4, seed=3)
+    cfg.update(field_on=0)
+    e = np.flatnonzero(parts["species"] == 0)
+    edge = lo + (hi - lo) * np.arange(len(e)) / nbins
+    v = np.sqrt(np.maximum(edge, 0.0) * 2 * 1.602176634e-19 / 9.1093837015e-31)
+    for k in ("vr", "vt"):
+        parts[k][e[::2]] = 0.0
+    parts["vz"][e[::2]] = v[::2]                       # to a float's rounding
+    parts["vz"][e[::16]] = parts["vr"][e[::16]] = parts["vt"][e[::16]] = 0.0
+    sim, o = run_pair(pd, cfg, parts, xs, 0)
+    for sp in (0, 1, 2):
+        assert np.array_equal(sim.energy_spectrum(sp, lo, hi, nbins), o.energy_spectrum(sp, lo, hi, nbins))
+
+
 def test_species_diagnostics_match_oracle(pd, xs):
     n = 32
     cfg, parts = synthetic.rz_plume(n=n, total=2e4, seed=9)
