@@ -152,6 +152,7 @@ constexpr int RC = 8;                           // rows of 32 ids a warp sorts i
 constexpr uint32_t COMPARE_MAX = 64;            // ids whose ranks come from comparisons
 constexpr uint32_t RANK_BLOCK_MAX = 12288;      // longest list the large kernel sorts in shared memory
 constexpr int RT_THREADS = 1024;                // threads of a large-kernel block
+constexpr uint32_t RT_SEG = 128;                // ids of a warp in a block's sort, at least
 constexpr int RT_MID_THREADS = 256;             // threads of a mid-size-kernel block
 constexpr int RT_MID_BLOCKS_PER_SM = 5;
 constexpr uint32_t SENTINEL = 0xFFFFFFFFu;
@@ -392,7 +393,10 @@ __device__ void radix_table(uint32_t n, int top, uint32_t* xk, uint32_t* xv, uin
 // this kernel (entries cell << 3 | species bin 0..6; *nq of them, at most
 // max_q): one list per block at a time, NT threads, sorted in shared memory
 // up to MAXN ids and in the scratch buffers above that.  A list already in
-// ascending id order gets the identity.
+// ascending id order gets the identity.  Passes of the sort bound it: the digits
+// are those of id - (smallest id), one or two for most cells where the id itself
+// has three, and a warp takes at least RT_SEG ids (64 to 128 alike, 256: 97 us):
+// 6200 lists of 257 to 2048 ids 135 -> 90 us, the longer ones 20.6 -> 14.6 us.
 template <int NT, uint32_t MAXN>
 __global__ void __launch_bounds__(NT) k_rank_tables(const uint32_t* __restrict__ ids, RankScratch S,
                                                     const uint32_t* __restrict__ off, const uint32_t* __restrict__ cnt,
@@ -404,12 +408,10 @@ __global__ void __launch_bounds__(NT) k_rank_tables(const uint32_t* __restrict__
     extern __shared__ uint32_t s_buf[];                 // four arrays of MAXN
     __shared__ uint32_t s_cnt[NWARPS * 256];
     __shared__ uint32_t s_tot[256];
-    __shared__ uint32_t s_or;
+    __shared__ uint32_t s_lo[NWARPS], s_hi[NWARPS];
     const uint32_t nb = min(*nq, max_q);             // an overflow is flagged by k_ncand
     const uint32_t tid = threadIdx.x;
     const int lane = (int)(tid & 31u), w = (int)(tid >> 5);
-    if (tid == 0) s_or = 0u;
-    __syncthreads();
     for (uint32_t b = blockIdx.x; b < nb; b += gridDim.x) {
         const uint32_t e = q[b];
         const uint32_t bin = (e & 7u) * C + (e >> 3);
@@ -421,27 +423,37 @@ __global__ void __launch_bounds__(NT) k_rank_tables(const uint32_t* __restrict__
         uint32_t* yk = in_smem ? s_buf + 2 * MAXN : S.yk + slot0;
         uint32_t* yv = in_smem ? s_buf + 3 * MAXN : S.yv + slot0;
         uint32_t* table = S.table + slot0;
-        uint32_t orv = 0;
+        uint32_t lo = 0xFFFFFFFFu, hi = 0u;
         for (uint32_t k = tid; k < n; k += NT) {
             const uint32_t x = base[k];
             xk[k] = x;
-            orv |= x;
+            lo = min(lo, x);
+            hi = max(hi, x);
         }
-        orv = __reduce_or_sync(FULL, orv);
-        if (lane == 0 && orv) atomicOr(&s_or, orv);
+        lo = __reduce_min_sync(FULL, lo);
+        hi = __reduce_max_sync(FULL, hi);
+        if (lane == 0) {
+            s_lo[w] = lo;
+            s_hi[w] = hi;
+        }
         __syncthreads();
         bool asc = true;
         for (uint32_t k = tid; k + 1 < n; k += NT)
             if (!(xk[k] < xk[k + 1])) asc = false;
-        const uint32_t any = s_or;
         if (__syncthreads_and(asc)) {
             for (uint32_t r = tid; r < n; r += NT) table[r] = r;
         } else {
-            const int top = any ? 31 - __clz((int)any) : 0;
-            const int nw = (int)min((uint32_t)NWARPS, (n + 255u) / 256u);
+#pragma unroll
+            for (int v = 0; v < NWARPS; ++v) {
+                lo = min(lo, s_lo[v]);
+                hi = max(hi, s_hi[v]);
+            }
+            for (uint32_t k = tid; k < n; k += NT) xk[k] -= lo;
+            __syncthreads();
+            const int top = hi > lo ? 31 - __clz((int)(hi - lo)) : 0;
+            const int nw = (int)min((uint32_t)NWARPS, (n + RT_SEG - 1u) / RT_SEG);
             radix_table<true>(n, top, xk, xv, yk, yv, table, nw, s_cnt, s_tot, tid, lane, w);
         }
-        if (tid == 0) s_or = 0u;
         __syncthreads();
     }
 }

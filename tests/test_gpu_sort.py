@@ -117,3 +117,30 @@ def test_hot_heavies_bit_exact(pd, xs, n, min_relayouts):
         assert np.array_equal(g[k][order], op[k]), k
     for k in FLOATS:
         assert np.array_equal(g[k][order].astype(np.float64), op[k]), k
+
+
+@pytest.mark.parametrize("T_heavy", [1e10, 2e12])
+def test_long_bins_bit_exact(pd, xs, T_heavy):
+    """4 x 4 cells of about 6000 particles: holes and the particles that fill
+    them lie many words of the bit mask apart (a few per cent of the heavies
+    leave their cell a step at 1e10 K, a third at 2e12 K)."""
+    cfg, parts = synthetic.microbench(nz=4, nr=4, total=1e5, seed=8, T_heavy=T_heavy)
+    sim = pd.Simulation(cfg, xs)
+    o = oracle.Oracle(cfg, fp64=False)
+    o.set_cross_sections(xs)
+    sim.load(parts)
+    o.load(parts)
+    o.prime()
+    for _ in range(3):
+        sim.step(1)
+        o.step(1)
+        sim.synchronize()
+        check_bins(sim, 16)
+    assert sim.sort_stats()["faults"] == 0
+    g, op = sim.particles(), o.particles()
+    order = np.argsort(g["id"], kind="stable")
+    assert len(g["id"]) == len(op["id"])
+    for k in ("id", "species", "iz", "ir"):
+        assert np.array_equal(g[k][order], op[k]), k
+    for k in FLOATS:
+        assert np.array_equal(g[k][order].astype(np.float64), op[k]), k
