@@ -15,11 +15,11 @@
 //     K = the nodes, with one warp per tap; each block sums over the tiles it
 //     visits and writes a partial that a second kernel adds up in a fixed
 //     order (so the gradient does not depend on the launch).
-// The 1 -> 32 and 32 -> 1 layers (1/32 of the arithmetic) run on the CUDA
-// cores.  Storage: activations h_1..h_5 and the gradients with respect to
-// a_1..a_5 in bfloat16 (node-major, 32 channels = 64 bytes per node), the
-// input, output, targets and the output gradient in float, weights in
-// bfloat16 for the layers and in float (master copies) for Adam.
+// The 1 -> 32 layer, and the 32 -> 1 layer in training, run on the CUDA cores.
+// Storage: activations h_1..h_5 and the gradients with respect to a_1..a_5 in
+// bfloat16 (node-major, 32 channels = 64 bytes per node), the input, output,
+// targets and the output gradient in float, weights in bfloat16 for the layers and
+// in float (master copies) for Adam.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "pd.h"
+#include "pd_launch.cuh"
 #include "pd_net.h"
 
 namespace pd {
@@ -228,6 +229,7 @@ __global__ void __launch_bounds__(CONV_THREADS, 4) k_conv32(const bf16* __restri
                 wb[tap][kh][nt][0] = __ldg(p);
                 wb[tap][kh][nt][1] = __ldg(p + 4);
             }
+    if (!chained()) return;                                   // (the weights are older than the kernel before)
     float bv[2][2] = {};
     if (MODE == 0)
 #pragma unroll
@@ -328,13 +330,80 @@ __global__ void __launch_bounds__(CONV_THREADS, 4) k_conv32(const bf16* __restri
 }
 
 // ---------------------------------------------------------------------------
-// layer 6 (32 -> 1): a thread two nodes (rows r and r + 4) of a tile staged in
-// shared memory, sharing the weights' reads (read from global memory, the 36
-// 16-byte pieces of a node's window are on as many lines a lane: 513^2 nodes 35 ->
-// 17 us)
+// layer 6 (32 -> 1) on the tensor cores: a warp 16 columns by four rows.  The
+// three tap rows are three columns of one product, so that an input row's 16
+// nodes (six ldmatrix, six mma) give what it adds to the output rows above, beside
+// and below it; these meet by a shuffle and two additions.  The weights are
+// bfloat16 values already; products and sums are exact and in float as before.
+// 513^2 nodes, all layers: 115 us with a thread two nodes' 288 products on the CUDA
+// cores, 107 us.
 __global__ void __launch_bounds__(16 * TY) k_conv6(const bf16* __restrict__ h, float* __restrict__ y,
                                                    const float* __restrict__ w6, const float* __restrict__ b6,
                                                    const uint32_t* __restrict__ base, int B, int H, int W) {
+    if (!chained()) return;
+    static_assert(TY == 8 && CX == 32, "four warps: two column groups by two halves of the rows");
+    __shared__ __align__(16) bf16 xs[TILE_ELEMS];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int cg = (warp & 1) * 16, r0 = (warp >> 1) * (TY / 2);
+    uint32_t wb[3][2][2];                                     // [dx][channel half]: column g is tap row g
+#pragma unroll
+    for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+        for (int kh = 0; kh < 2; ++kh)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                float2 v = make_float2(0.0f, 0.0f);
+                if (g < 3) v = *(const float2*)(w6 + (3 * g + dx) * CH + kh * 16 + 8 * e + 2 * t);
+                const __nv_bfloat162 b = __floats2bfloat162_rn(v.x, v.y);
+                wb[dx][kh][e] = *(const uint32_t*)&b;
+            }
+    const float bias = b6[0];
+    const bf16* xl = xs + (r0 * (CX + 2) + cg + (lane & 15)) * HP + (lane >> 4) * 8;
+    const int tj = (W + CX - 1) / CX, ti = (H + TY - 1) / TY;
+    const long long ntiles = (long long)B * tj * ti;
+    for (long long q = blockIdx.x; q < ntiles; q += gridDim.x) {
+        const Tile tl = tile_at(q, tj, ti);
+        __syncthreads();
+        stage_halo(xs, h, base, tl, H, W);
+        copy_wait<0>();
+        __syncthreads();
+        if (tl.j0 + cg >= W) continue;
+        float o[3][2];                                        // open output rows: nodes g and g + 8 (lanes t = 0)
+#pragma unroll
+        for (int hi = 0; hi < TY / 2 + 2; ++hi) {
+            float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+                for (int kh = 0; kh < 2; ++kh) {
+                    uint32_t a[4];
+                    ldsm4(a, xl + (hi * (CX + 2) + dx) * HP + kh * 16);
+                    mma_bf16(c, a[0], a[1], a[2], a[3], wb[dx][kh][0], wb[dx][kh][1]);
+                }
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                const float below = __shfl_down_sync(0xFFFFFFFFu, c[2 * half], 1);      // tap row 2, of lane t = 1
+                if (hi >= 2) o[(hi - 2) % 3][half] += below;
+                if (hi >= 1 && hi - 1 < TY / 2) o[(hi - 1) % 3][half] += c[2 * half + 1];
+                if (hi < TY / 2) o[hi % 3][half] = c[2 * half];
+            }
+            if (hi < 2) continue;
+            const int i = tl.i0 + r0 + hi - 2;
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                const int j = tl.j0 + cg + g + 8 * half;
+                if (t == 0 && i < H && j < W) y[node_index(base, tl.b, H, W, i, j)] = o[(hi - 2) % 3][half] + bias;
+            }
+        }
+    }
+}
+
+// The same in training, a thread two nodes (rows r and r + 4), summed tap by tap:
+// the residual loss differentiates y twice, and its gradient (through bfloat16)
+// shows the last bit of y at 2e-5.
+__global__ void __launch_bounds__(16 * TY) k_conv6_train(const bf16* __restrict__ h, float* __restrict__ y,
+                                                         const float* __restrict__ w6, const float* __restrict__ b6,
+                                                         const uint32_t* __restrict__ base, int B, int H, int W) {
     __shared__ __align__(16) bf16 xs[(TY + 2) * (CX + 2) * HP];
     __shared__ __align__(16) float ws[9 * CH];
     for (int q = threadIdx.x; q < 9 * CH; q += blockDim.x) ws[q] = w6[q];
@@ -795,15 +864,19 @@ int tile_blocks(const pd_net* net, int B, int H, int W, int per_sm) {
     return (int)std::min(n, (long long)net->sms * per_sm);
 }
 
+// each layer's blocks start, and read its weights, while the layer before ends:
+// 513^2 nodes 107 -> 96 us.  Not in training: a step of 8 x 129^2 nodes 408 us,
+// 412 with these layers launched so, 435 with the back-propagation too.
 void forward_layers(pd_net* net, const float* x, float* y, int B, int H, int W, const uint32_t* base,
-                    cudaStream_t s) {
+                    cudaStream_t s, bool training) {
     const float* P = net->master;
     const int gc = tile_blocks(net, B, H, W, 4), ge = tile_blocks(net, B, H, W, 8);
     k_conv1<<<ge, 32 * TY, 0, s>>>(x, net->h[0], net->w1r, P + off_b(0), base, B, H, W);
     for (int l = 1; l <= 4; ++l)
-        k_conv32<0><<<gc, CONV_THREADS, CONV_SMEM, s>>>(net->h[l - 1], net->h[l], net->wk + (size_t)(l - 1) * 9 * CH * CH,
-                                                   P + off_b(l), nullptr, base, B, H, W);
-    k_conv6<<<ge, 16 * TY, 0, s>>>(net->h[4], y, net->w6r, P + off_b(5), base, B, H, W);
+        launch(!training, k_conv32<0>, gc, CONV_THREADS, CONV_SMEM, s, net->h[l - 1], net->h[l],
+               net->wk + (size_t)(l - 1) * 9 * CH * CH, P + off_b(l), nullptr, base, B, H, W);
+    if (training) k_conv6_train<<<ge, 16 * TY, 0, s>>>(net->h[4], y, net->w6r, P + off_b(5), base, B, H, W);
+    else launch(true, k_conv6, ge, 16 * TY, 0, s, net->h[4], y, net->w6r, P + off_b(5), base, B, H, W);
 }
 
 pd_status upload_weights(pd_net* net) {
@@ -819,7 +892,7 @@ namespace pd {
 int net_forward_at(pd_net* net, const float* x, float* y, int B, int H, int W, const uint32_t* base,
                    int64_t node_span, cudaStream_t stream) {
     if (!net || node_span > net->max_nodes) return 1;
-    forward_layers(net, x, y, B, H, W, base, stream);
+    forward_layers(net, x, y, B, H, W, base, stream, false);
     return cudaGetLastError() == cudaSuccess ? 0 : 1;
 }
 int64_t net_max_nodes(const pd_net* net) { return net ? net->max_nodes : 0; }
@@ -910,7 +983,7 @@ pd_status pd_net_get_params(pd_net* net, float* params) {
 pd_status pd_net_forward(pd_net* net, const float* x, int B, int H, int W, float* y) {
     if (!net || !x || !y) return PD_ERR_ARG;
     if (!shape_ok(net, B, H, W)) return net_fail(net, PD_ERR_ARG, "batch exceeds the network's node capacity");
-    forward_layers(net, x, y, B, H, W, nullptr, net->stream);
+    forward_layers(net, x, y, B, H, W, nullptr, net->stream, false);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? PD_OK : net_fail(net, PD_ERR_CUDA, cudaGetErrorString(e));
 }
@@ -966,7 +1039,7 @@ pd_status pd_net_loss_grad(pd_net* net, const float* x, const float* t, int B, i
     if (!shape_ok(net, B, H, W)) return net_fail(net, PD_ERR_ARG, "batch exceeds the network's node capacity");
     cudaStream_t s = net->stream;
     const long long total = (long long)B * H * W;
-    forward_layers(net, x, net->ybuf, B, H, W, nullptr, s);
+    forward_layers(net, x, net->ybuf, B, H, W, nullptr, s, true);
     const int lb = (int)std::min<long long>(LOSS_BLOCKS, (total + 255) / 256);
     k_loss<<<lb, 256, 0, s>>>(net->ybuf, t, net->g6, net->lpart, total);
     return backprop(net, x, net->g6, B, H, W, lb, 1.0 / (double)total, loss, grads);
@@ -978,7 +1051,7 @@ pd_status pd_net_loss_grad_rz(pd_net* net, const float* x, int B, int H, int W, 
         return net_fail(net, PD_ERR_ARG, "batch exceeds the network's node capacity, or a grid below 3 x 2 nodes");
     cudaStream_t s = net->stream;
     const long long total = (long long)B * H * W, n_int = (long long)B * (H - 2) * W;
-    forward_layers(net, x, net->ybuf, B, H, W, nullptr, s);
+    forward_layers(net, x, net->ybuf, B, H, W, nullptr, s, true);
     const int lb = (int)std::min<long long>(LOSS_BLOCKS, (total + 255) / 256);
     // r into g6, then dL/dy = -(2 / N) S r into ybuf (y is not needed after r)
     k_rz_resid<<<lb, 256, 0, s>>>(x, net->ybuf, net->g6, net->lpart, B, H, W);
