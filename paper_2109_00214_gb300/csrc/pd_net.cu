@@ -49,7 +49,7 @@ constexpr int CX = 32;               // columns of a convolution's tile (of TY r
 constexpr int CONV_THREADS = 128;    // a 32 -> 32 layer's block: two column groups by two channel halves
 constexpr int HP = 40;               // channel stride of a staged node (bf16): 80 bytes, conflict-free fragments
 constexpr int MAX_PART_BLOCKS = 384;  // (k_reduce holds a value's partials in 48 KB of shared memory, 32 values a block)
-constexpr int PART_STRIDE = 9 * CH * CH + CH;
+constexpr int PART_STRIDE = (NP + 31) / 32 * 32;   // a block's partial gradient: the whole parameter vector
 constexpr int LOSS_BLOCKS = 256;
 
 size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -625,7 +625,7 @@ __global__ void __launch_bounds__(320) k_wgrad1(const float* __restrict__ x, con
             for (int nd = 0; nd < TY * TX; ++nd) acc += gsm[nd][tid - 9 * CH];
         }
     }
-    part[(size_t)blockIdx.x * (9 * CH + CH) + tid] = acc;
+    part[(size_t)blockIdx.x * PART_STRIDE + tid] = acc;
 }
 
 // (a last block, beyond the gridDim.x - 1 that take tiles, sums the loss)
@@ -676,7 +676,7 @@ __global__ void __launch_bounds__(320) k_wgrad6(const float* __restrict__ g6, co
             for (int nd = 0; nd < TY * TX; ++nd) acc += gsm[nd];
         }
     }
-    if (tid <= 9 * CH) part[(size_t)blockIdx.x * (9 * CH + 1) + tid] = acc;
+    if (tid <= 9 * CH) part[(size_t)blockIdx.x * PART_STRIDE + tid] = acc;
 }
 
 // the same, each 8 x 8 matrix transposed
@@ -755,19 +755,20 @@ __global__ void __launch_bounds__(288) k_wgrad32(const bf16* __restrict__ h, con
     if (threadIdx.x < CH) P[9 * CH * CH + threadIdx.x] = bacc;
 }
 
-// out[k] = sum over blocks c (in order) of part[c * stride + k], k < count: a block
+// out[k] = sum over blocks c (in order) of part[c * PART_STRIDE + k], k < NP: a block
 // brings 32 values' partials into shared memory with all its loads in flight, a
 // warp adds them in order (the chain of additions waited for a load each: 304
-// partials of 9248 values 31 -> 10 us)
+// partials of 9248 values 31 -> 10 us).  One launch for all layers: a layer's fills
+// a quarter of the SMs for 10 us, six of them 60 us of a step: 8 x 129^2 nodes 411
+// -> 380 us a step (and, with no more blocks than tiles, 1 x 33 x 47 nodes 245 -> 192 us).
 constexpr int RED_COLS = 32;
-__global__ void __launch_bounds__(256) k_reduce(const float* __restrict__ part, int nblocks, int stride, int count,
-                                                float* out) {
+__global__ void __launch_bounds__(256) k_reduce(const float* __restrict__ part, int nblocks, float* out) {
     extern __shared__ float ps[];
     const int k0 = blockIdx.x * RED_COLS, lane = threadIdx.x & 31;
-    const bool in = k0 + lane < count;
+    const bool in = k0 + lane < NP;
 #pragma unroll 8
     for (int c = threadIdx.x >> 5; c < nblocks; c += 8)
-        ps[c * RED_COLS + lane] = in ? part[(size_t)c * stride + k0 + lane] : 0.0f;
+        ps[c * RED_COLS + lane] = in ? part[(size_t)c * PART_STRIDE + k0 + lane] : 0.0f;
     __syncthreads();
     if (threadIdx.x >= RED_COLS || !in) return;
     float s = 0.0f;
@@ -843,7 +844,11 @@ NetLayout net_layout(int64_t max_nodes) {
     return L;
 }
 
-int part_blocks(const pd_net* net) { return std::min(MAX_PART_BLOCKS, 2 * net->sms); }
+// blocks of the weight gradients over their tiles of TY x TX nodes
+int part_blocks(const pd_net* net, int B, int H, int W) {
+    const long long n = (long long)B * ((W + TX - 1) / TX) * ((H + TY - 1) / TY);
+    return (int)std::min<long long>(n, std::min(MAX_PART_BLOCKS, 2 * net->sms));
+}
 int elem_blocks(const pd_net* net, long long n) {
     const long long b = (n + 255) / 256;
     return (int)std::max(1LL, std::min(b, (long long)net->sms * 16));
@@ -992,34 +997,27 @@ pd_status pd_net_forward(pd_net* net, const float* x, int B, int H, int W, float
 
 namespace {
 
-// sum of `blocks` partials of n values each
-void reduce(const float* part, int blocks, int n, float* out, cudaStream_t s) {
-    k_reduce<<<(n + RED_COLS - 1) / RED_COLS, 256, (size_t)blocks * RED_COLS * 4, s>>>(part, blocks, n, n, out);
-}
-
 // back-propagation of the output gradient g6 (B H W floats) to the
 // parameter gradient, and the loss (of lb partials) and gradient out to the host
 // if asked
 pd_status backprop(pd_net* net, const float* x, const float* g6, int B, int H, int W, int lb, double inv_count,
                    double* loss, float* grads) {
     cudaStream_t s = net->stream;
-    const int pb = part_blocks(net);
+    const int pb = part_blocks(net, B, H, W);
     const int gc = tile_blocks(net, B, H, W, 4), ge = tile_blocks(net, B, H, W, 8);
     // layer 6
-    k_wgrad6<<<pb + 1, 320, 0, s>>>(g6, net->h[4], net->part, B, H, W, net->lpart, lb, inv_count, net->lsum);
-    reduce(net->part, pb, 9 * CH + 1, net->grad + off_w(5), s);
+    k_wgrad6<<<pb + 1, 320, 0, s>>>(g6, net->h[4], net->part + off_w(5), B, H, W, net->lpart, lb, inv_count, net->lsum);
     k_conv6_bwd<<<ge, 32 * TY, 0, s>>>(g6, net->h[4], net->g[4], net->w6r, B, H, W);
     // layers 5 .. 2
     for (int l = 4; l >= 1; --l) {
-        k_wgrad32<<<pb, 288, 0, s>>>(net->h[l - 1], net->g[l], net->part, B, H, W);
         // weights then biases: both contiguous in the parameter vector
-        reduce(net->part, pb, PART_STRIDE, net->grad + off_w(l), s);
+        k_wgrad32<<<pb, 288, 0, s>>>(net->h[l - 1], net->g[l], net->part + off_w(l), B, H, W);
         k_conv32<1><<<gc, CONV_THREADS, CONV_SMEM, s>>>(net->g[l], net->g[l - 1], net->wt + (size_t)(l - 1) * 9 * CH * CH,
                                                    nullptr, net->h[l - 1], nullptr, B, H, W);
     }
     // layer 1
-    k_wgrad1<<<pb, 320, 0, s>>>(x, net->g[0], net->part, B, H, W);
-    reduce(net->part, pb, 9 * CH + CH, net->grad + off_w(0), s);
+    k_wgrad1<<<pb, 320, 0, s>>>(x, net->g[0], net->part + off_w(0), B, H, W);
+    k_reduce<<<(NP + RED_COLS - 1) / RED_COLS, 256, (size_t)pb * RED_COLS * 4, s>>>(net->part, pb, net->grad);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return net_fail(net, PD_ERR_CUDA, cudaGetErrorString(e));
     net->have_grad = true;
