@@ -534,7 +534,7 @@ __global__ void __launch_bounds__(256) k_rz_resid_grad(const float* __restrict__
 }
 
 // the sum of a loss's n <= LOSS_BLOCKS partials in their order, by one block (a
-// chain of double additions, 8 us: it runs beside k_wgrad6's blocks)
+// chain of double additions, 8 us: it runs beside k_wgrad_edge's blocks)
 __device__ __forceinline__ void loss_sum(const double* __restrict__ part, int n, double inv_count, double* out,
                                          double* p) {
     if ((int)threadIdx.x < n) p[threadIdx.x] = part[threadIdx.x];
@@ -580,103 +580,77 @@ __global__ void __launch_bounds__(32 * TY) k_conv6_bwd(const float* __restrict__
 }
 
 // ---------------------------------------------------------------------------
-// weight gradients of the first and last layers (CUDA cores), over the same
-// 8 x 16 node tiles staged in shared memory: thread (tap, c) < 288 of a
-// 320-thread block sums over the tiles the block visits; the remaining
-// threads sum the bias gradients.  Partials: [block][288 + biases].
-__global__ void __launch_bounds__(320) k_wgrad1(const float* __restrict__ x, const bf16* __restrict__ g1,
-                                                float* part, int B, int H, int W) {
-    __shared__ float gsm[TY * TX][CH + 1];
-    __shared__ float xsm[(TY + 2) * (TX + 2)];
-    const int tid = threadIdx.x;
-    const int tap = tid / CH, co = tid % CH;
-    const int dy = tap < 9 ? tap_dy(tap) : 0, dx = tap < 9 ? tap_dx(tap) : 0;
-    const int tj = (W + TX - 1) / TX, ti = (H + TY - 1) / TY;
-    const long long ntiles = (long long)B * tj * ti, n = (long long)H * W;
-    float acc = 0.0f;
-    for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int b = (int)(tile / ((long long)tj * ti));
-        const int r = (int)(tile - (long long)b * tj * ti);
-        const int i0 = (r / tj) * TY, j0 = (r % tj) * TX;
-        __syncthreads();
-        for (int q = tid; q < TY * TX * 4; q += blockDim.x) {     // eight channels a load
-            const int nd = q >> 2, part4 = q & 3;
-            const int gi = i0 + nd / TX, gj = j0 + nd % TX;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (gi < H && gj < W) v = ((const uint4*)(g1 + ((size_t)b * n + (size_t)gi * W + gj) * CH))[part4];
-            const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                gsm[nd][part4 * 8 + 2 * e] = __uint_as_float(u[e] << 16);
-                gsm[nd][part4 * 8 + 2 * e + 1] = __uint_as_float(u[e] & 0xFFFF0000u);
-            }
-        }
-        for (int q = tid; q < (TY + 2) * (TX + 2); q += blockDim.x) {
-            const int gi = i0 + q / (TX + 2) - 1, gj = j0 + q % (TX + 2) - 1;
-            xsm[q] = (gi >= 0 && gi < H && gj >= 0 && gj < W) ? x[(size_t)b * n + (size_t)gi * W + gj] : 0.0f;
-        }
-        __syncthreads();
-        if (tid < 9 * CH) {
-#pragma unroll 32
-            for (int nd = 0; nd < TY * TX; ++nd)
-                acc += gsm[nd][co] * xsm[(nd / TX + dy + 1) * (TX + 2) + nd % TX + dx + 1];
-        } else {
-#pragma unroll 32
-            for (int nd = 0; nd < TY * TX; ++nd) acc += gsm[nd][tid - 9 * CH];
-        }
-    }
-    part[(size_t)blockIdx.x * PART_STRIDE + tid] = acc;
-}
-
-// (a last block, beyond the gridDim.x - 1 that take tiles, sums the loss)
-__global__ void __launch_bounds__(320) k_wgrad6(const float* __restrict__ g6, const bf16* __restrict__ h5,
-                                                float* part, int B, int H, int W, const double* __restrict__ lpart,
-                                                int lb, double inv_count, double* lsum) {
-    __shared__ float gsm[TY * TX];
-    __shared__ __align__(16) float hsm[(TY + 2) * (TX + 2)][CH + 1];
-    const int tid = threadIdx.x, nblk = (int)gridDim.x - 1;
-    if ((int)blockIdx.x == nblk) {
-        loss_sum(lpart, lb, inv_count, lsum, reinterpret_cast<double*>(&hsm[0][0]));
+// Weight gradients of the first and last layers (CUDA cores): each tap's sum over
+// the nodes of a node value at the tap's place (layer 1: x at p + tap, layer 6: g6
+// at p - tap) times 32 channel values at p (g1, h5).  A warp takes a row of an 8 x
+// 16 node tile, a lane a channel with its nine sums in registers, the node values
+// staged in shared memory and read as broadcasts; the rows' sums meet at the end
+// (a thread a tap and channel read two words of shared memory a product, which
+// bounded it, 21 us each at eight samples of 129^2 nodes: a step 380 -> 364 us).  Partials: 288
+// weights, then the bias gradients.  Layer 6: a last block sums the loss.
+template <int LAYER>
+__global__ void __launch_bounds__(32 * TY) k_wgrad_edge(const float* __restrict__ nodes, const bf16* __restrict__ chan,
+                                                        float* part, int B, int H, int W,
+                                                        const double* __restrict__ lpart, int lb, double inv_count,
+                                                        double* lsum) {
+    __shared__ float xs[(TY + 2) * (TX + 2)];
+    __shared__ __align__(16) float red[10][TY][CH];
+    const int lane = threadIdx.x & 31, row = threadIdx.x >> 5, nblk = (int)gridDim.x - (LAYER == 6 ? 1 : 0);
+    if (LAYER == 6 && (int)blockIdx.x == nblk) {
+        static_assert(LOSS_BLOCKS <= 32 * TY && sizeof(red) >= LOSS_BLOCKS * sizeof(double), "loss_sum");
+        loss_sum(lpart, lb, inv_count, lsum, reinterpret_cast<double*>(&red[0][0][0]));
         return;
     }
-    const int tap = tid / CH, ci = tid % CH;
-    const int dy = tap < 9 ? tap_dy(tap) : 0, dx = tap < 9 ? tap_dx(tap) : 0;
     const int tj = (W + TX - 1) / TX, ti = (H + TY - 1) / TY;
     const long long ntiles = (long long)B * tj * ti, n = (long long)H * W;
-    float acc = 0.0f;
+    float acc[10] = {};                                       // the taps, the bias
     for (long long tile = blockIdx.x; tile < ntiles; tile += nblk) {
         const int b = (int)(tile / ((long long)tj * ti));
         const int r = (int)(tile - (long long)b * tj * ti);
-        const int i0 = (r / tj) * TY, j0 = (r % tj) * TX;
-        __syncthreads();
-        for (int q = tid; q < TY * TX; q += blockDim.x) {
-            const int gi = i0 + q / TX, gj = j0 + q % TX;
-            gsm[q] = (gi < H && gj < W) ? g6[(size_t)b * n + (size_t)gi * W + gj] : 0.0f;
-        }
-        for (int q = tid; q < (TY + 2) * (TX + 2) * 4; q += blockDim.x) {     // eight channels a load
-            const int nd = q >> 2, part4 = q & 3;
-            const int gi = i0 + nd / (TX + 2) - 1, gj = j0 + nd % (TX + 2) - 1;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (gi >= 0 && gi < H && gj >= 0 && gj < W)
-                v = ((const uint4*)(h5 + ((size_t)b * n + (size_t)gi * W + gj) * CH))[part4];
-            const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+        const int i0 = (r / tj) * TY, j0 = (r % tj) * TX, i = i0 + row, nj = min(TX, W - j0);
+        float v[TX];
+        if (i < H) {
+            const bf16* src = chan + ((size_t)b * n + (size_t)i * W + j0) * CH + lane;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                hsm[nd][part4 * 8 + 2 * e] = __uint_as_float(u[e] << 16);
-                hsm[nd][part4 * 8 + 2 * e + 1] = __uint_as_float(u[e] & 0xFFFF0000u);
-            }
+            for (int j = 0; j < TX; ++j) v[j] = j < nj ? __bfloat162float(src[(size_t)j * CH]) : 0.0f;
         }
         __syncthreads();
-        if (tid < 9 * CH) {
-#pragma unroll 32
-            for (int nd = 0; nd < TY * TX; ++nd)
-                acc += gsm[nd] * hsm[(nd / TX + dy + 1) * (TX + 2) + nd % TX + dx + 1][ci];
-        } else if (tid == 9 * CH) {
-#pragma unroll 32
-            for (int nd = 0; nd < TY * TX; ++nd) acc += gsm[nd];
+        for (int q = threadIdx.x; q < (TY + 2) * (TX + 2); q += blockDim.x) {
+            const int gi = i0 + q / (TX + 2) - 1, gj = j0 + q % (TX + 2) - 1;
+            xs[q] = (gi >= 0 && gi < H && gj >= 0 && gj < W) ? nodes[(size_t)b * n + (size_t)gi * W + gj] : 0.0f;
         }
+        __syncthreads();
+        if (i >= H) continue;
+        const float* xr = xs + row * (TX + 2);
+#pragma unroll
+        for (int j = 0; j < TX; ++j) {
+#pragma unroll
+            for (int tap = 0; tap < 9; ++tap) {
+                const int y = LAYER == 1 ? tap / 3 : 2 - tap / 3, x = LAYER == 1 ? tap % 3 : 2 - tap % 3;
+                acc[tap] += v[j] * xr[y * (TX + 2) + j + x];
+            }
+            if (LAYER == 1) acc[9] += v[j];
+        }
+        if (LAYER == 6 && lane < TX) acc[9] += xr[TX + 2 + lane + 1];
     }
-    if (tid <= 9 * CH) part[(size_t)blockIdx.x * PART_STRIDE + tid] = acc;
+#pragma unroll
+    for (int k = 0; k < 10; ++k) red[k][row][lane] = acc[k];
+    __syncthreads();
+    float* out = part + (size_t)blockIdx.x * PART_STRIDE;
+    for (int q = threadIdx.x; q < (LAYER == 1 ? 10 : 9) * CH; q += blockDim.x) {
+        float t = 0.0f;
+#pragma unroll
+        for (int w = 0; w < TY; ++w) t += red[q / CH][w][q % CH];
+        out[q] = t;
+    }
+    if (LAYER == 6 && row == 0) {
+        float t = 0.0f;
+#pragma unroll
+        for (int w = 0; w < TY; ++w) t += red[9][w][lane];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
+        if (lane == 0) out[9 * CH] = t;
+    }
 }
 
 // the same, each 8 x 8 matrix transposed
@@ -1006,7 +980,8 @@ pd_status backprop(pd_net* net, const float* x, const float* g6, int B, int H, i
     const int pb = part_blocks(net, B, H, W);
     const int gc = tile_blocks(net, B, H, W, 4), ge = tile_blocks(net, B, H, W, 8);
     // layer 6
-    k_wgrad6<<<pb + 1, 320, 0, s>>>(g6, net->h[4], net->part + off_w(5), B, H, W, net->lpart, lb, inv_count, net->lsum);
+    k_wgrad_edge<6><<<pb + 1, 32 * TY, 0, s>>>(g6, net->h[4], net->part + off_w(5), B, H, W, net->lpart, lb, inv_count,
+                                               net->lsum);
     k_conv6_bwd<<<ge, 32 * TY, 0, s>>>(g6, net->h[4], net->g[4], net->w6r, B, H, W);
     // layers 5 .. 2
     for (int l = 4; l >= 1; --l) {
@@ -1016,7 +991,7 @@ pd_status backprop(pd_net* net, const float* x, const float* g6, int B, int H, i
                                                    nullptr, net->h[l - 1], nullptr, B, H, W);
     }
     // layer 1
-    k_wgrad1<<<pb, 320, 0, s>>>(x, net->g[0], net->part + off_w(0), B, H, W);
+    k_wgrad_edge<1><<<pb, 32 * TY, 0, s>>>(x, net->g[0], net->part + off_w(0), B, H, W, nullptr, 0, 0.0, nullptr);
     k_reduce<<<(NP + RED_COLS - 1) / RED_COLS, 256, (size_t)pb * RED_COLS * 4, s>>>(net->part, pb, net->grad);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return net_fail(net, PD_ERR_CUDA, cudaGetErrorString(e));
