@@ -233,7 +233,7 @@ def peaks():
 # it was taken on: TRAFFIC_SOURCE_SHA is the push_source_digest() of the
 # source at the capture, and `traffic` is null for any other source.
 TRAFFIC_PER_PARTICLE = {"push": 796.619e6 / 24898326}
-TRAFFIC_SOURCE_SHA = "4ea56a37e679cd6915a1f10f3105171b5066fd3f77c9b4c9d07c6f56dc5efaa0"
+TRAFFIC_SOURCE_SHA = "dcb1c292eddb73eaf7dbdb07f22ec3d7e329c3d9b219bdd824772da433b6e971"
 TRAFFIC_SOURCE = "ncu dram bytes per particle of a 2.49e7-particle launch, scaled"
 PUSH_SECTION_END = "// sort: holes, insertions, re-layout"
 
