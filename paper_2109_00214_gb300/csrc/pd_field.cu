@@ -26,7 +26,7 @@
 // inverse (formed on the host once; Gauss-Seidel sweeps instead when the
 // coarsest level has more than MG_DIRECT_MAX unknowns).  A level takes one
 // launch on the way down (smoothing, residual and restriction), one on the way
-// up (prolongation and smoothing); the levels of at most 34 x 34 nodes take one
+// up (prolongation and smoothing); the levels of at most 2048 nodes take one
 // launch together, and the residual with its norm the last of a cycle.
 //
 // Batched over runs: the per-cycle kernels take work lists of (run, tile) per
@@ -56,9 +56,13 @@ constexpr int TILE_WARPS = 4;          // tiles of a block of the smoothing kern
 constexpr int WIN_C = 64, PRE_H = 6, POST_H = 4;
 constexpr int K_SMALL = 20, K_LARGE = 32;
 constexpr int SMALL_TILES = 4 * 152;   // long windows from this many tiles on
-constexpr int TAIL_NODES = 34 * 34;    // levels from the first one with at most this many nodes: k_mg_tail
+// Levels from the first one with at most this many nodes (two of a color a thread):
+// k_mg_tail.  A level there takes 3-4 us of a cycle, its two launches 11: from 1156
+// nodes on, 224 x 96 cells 3.74 -> 3.65 ms, 448 x 256 3.15 -> 3.02 (57 x 25 and 57 x
+// 33 nodes).
+constexpr int TAIL_NODES = 2048;
 constexpr int TAIL_THREADS = 512;
-constexpr int TAIL_SLOTS = 2;          // nodes of a color a thread of k_mg_tail holds (at most 766 a level)
+constexpr int TAIL_SLOTS = 2;          // nodes of a color a thread of k_mg_tail holds (most levels: one)
 
 size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 
@@ -81,7 +85,7 @@ int coarse_unknowns(const int* a, const int* b, int n) { return (a[n - 1] - 1) *
 // most 1024 nodes)
 int tail_level(const int* a, const int* b, int n) {
     for (int l = 0; l < n; ++l)
-        if ((a[l] + 1) * (b[l] + 1) <= TAIL_NODES) return l;
+        if ((a[l] + 1) * (b[l] + 1) <= TAIL_NODES && (a[l] - 1) * ((b[l] + 2) / 2) <= TAIL_SLOTS * TAIL_THREADS) return l;
     return n - 1;
 }
 
@@ -1092,7 +1096,7 @@ int field_init(FieldSolver& fs, const std::vector<pd_config>& cfgs, const std::v
     for (int r = 0; r < R; ++r)
         for (int u = 0; u < red_units(cfgs[r].nz, cfgs[r].nr); u += RED_WARPS) tasks.push_back(make_int2(r, u));
     fs.red_len = (int)tasks.size() - fs.red_off;
-    // tail levels hold at most 34 x 34 nodes, the inverse 40 KB (10 KB are static)
+    // tail levels hold 24 KB and a third of that, the inverse 40 KB (10 KB are static)
     if (fs.tail_smem > 36 * 1024 && cudaFuncSetAttribute(k_mg_tail, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                          (int)fs.tail_smem) != cudaSuccess)
         return 1;
