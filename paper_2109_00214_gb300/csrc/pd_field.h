@@ -73,6 +73,7 @@ struct FieldSolver {
     // shared memory (k_mg_tail); the level lists hold only the levels above
     std::vector<int> tail_lev;
     TailRun* tails = nullptr;           // [nruns]
+    TailRun host_tail{};                // the first
     int max_tail = 0;                   // largest tail_lev over the runs
     size_t tail_smem = 0;               // dynamic shared memory of k_mg_tail
     int threads = 256;                  // threads per block of the node kernels (64..1024, a multiple of 32)
