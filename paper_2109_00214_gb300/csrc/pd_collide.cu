@@ -870,9 +870,7 @@ __device__ __forceinline__ uint32_t fe_round(uint32_t x, uint32_t k) {
 }
 // h of the permutation of [0, n): the least h >= 1 with 4^h >= n
 __device__ __forceinline__ int perm_bits(uint32_t n) {
-    int h = 1;
-    while ((1ull << (2 * h)) < (unsigned long long)n) ++h;
-    return h;
+    return n > 4u ? (33 - __clz((int)(n - 1u))) / 2 : 1;
 }
 // one pass of the four Feistel rounds on 2h bits
 __device__ __forceinline__ uint32_t feistel4(uint32_t y, const uint4& key, int h) {
@@ -890,35 +888,36 @@ __device__ __forceinline__ uint32_t feistel4(uint32_t y, const uint4& key, int h
 }
 // Indices x0 and x1 under two permutations (or the same one twice), each
 // walked back into its range [0, n) by repeating the rounds until the value
-// falls in it; the two walks advance side by side.  A walk ends within 4^h
-// steps, x lying in [0, n) itself (x is returned after 4^h, which it never
-// reaches).
+// falls in it, one walk after the other in one loop: a warp then takes as many
+// rounds as its longest pair of walks has (side by side it took twice the longest
+// walk's: k_coulomb 475 -> 417 us with that and 32-bit counts).
+// A walk ends within 4^h steps, x lying in [0, n) itself (x is returned after
+// 4^h, which it never reaches).
 __device__ void perm_index2(uint32_t x0, uint32_t n0, const uint4& key0, int h0, uint32_t x1, uint32_t n1,
                             const uint4& key1, int h1, uint32_t& out0, uint32_t& out1) {
-    const unsigned long long lim0 = 1ull << (2 * h0), lim1 = 1ull << (2 * h1);
-    const unsigned long long lim = lim0 > lim1 ? lim0 : lim1;
-    uint32_t y0 = x0, y1 = x1;
-    bool d0 = false, d1 = false;
     out0 = x0;
     out1 = x1;
-    for (unsigned long long it = 0; it < lim && !(d0 && d1); ++it) {
-        if (!d0) {
-            y0 = feistel4(y0, key0, h0);
-            if (y0 < n0) {
-                out0 = y0;
-                d0 = true;
-            } else if (it + 1 >= lim0) {
-                d0 = true;
+    uint4 key = key0;
+    uint32_t y = x0, n = n0;
+    int h = h0;
+    bool second = false;
+    uint32_t left = h0 < 16 ? 1u << (2 * h0) : 0xFFFFFFFFu;
+#pragma unroll 1
+    for (;;) {
+        y = feistel4(y, key, h);
+        const bool in = y < n;
+        if (in || --left == 0u) {
+            if (second) {
+                if (in) out1 = y;
+                return;
             }
-        }
-        if (!d1) {
-            y1 = feistel4(y1, key1, h1);
-            if (y1 < n1) {
-                out1 = y1;
-                d1 = true;
-            } else if (it + 1 >= lim1) {
-                d1 = true;
-            }
+            if (in) out0 = y;
+            second = true;
+            key = key1;
+            y = x1;
+            n = n1;
+            h = h1;
+            left = h1 < 16 ? 1u << (2 * h1) : 0xFFFFFFFFu;
         }
     }
 }
@@ -1084,9 +1083,9 @@ __device__ __forceinline__ int list_species(int l) { return l == 0 ? SP_E : SP_C
 // 826 us and 4060 instructions a cell with a warp a cell, its pairs in the
 // classes' waves of disjoint pairs (12.5 threads an instruction); 500 us and 2290
 // with batches and rounds; 450-475 us with blocks of one warp, at 22 an SM (20:
-// 490 us, 16: 530).  Of it the turns take 120 us, the rank tables 80, the
-// permutations 180 (their walks differ in length; tables of the permutations of
-// up to 16 places took as long to make).
+// 490 us, 16: 530), 417 us with shorter permutation walks.  Of it the turns take 120
+// us, the rank tables 80, the permutations about 120 (their walks differ in length;
+// tables of the permutations of up to 16 places took as long to make).
 __global__ void __launch_bounds__(32, COUL_BLOCKS) k_coulomb(Particles A, RankScratch S, const uint32_t* __restrict__ off,
                                                    const uint32_t* __restrict__ cnt, DevState* st, KParams P,
                                                    CollConsts cc, const double* __restrict__ cw, uint32_t cells) {
