@@ -726,16 +726,16 @@ pd_status issue_step(pd_sim* s, bool capturing) {
             launch_sort(a, s->st, P, s->sms, s->stream);
         }
         {
-            // the re-layout of the heavy bins (three kernels, a scan of three,
-            // and four more) returns at once unless a heavy bin overflowed
-            Timed t(s, K_SCAN_BINS, capturing, 10);
+            // the re-layout of the heavy bins (three kernels, a scan, and four
+            // more) returns at once unless a heavy bin overflowed
+            Timed t(s, K_SCAN_BINS, capturing, 7 + scan_launches(s->L.nbins_pad));
             launch_relayout(a, s->st, P, grid_for(s, s->tune.bincount_blocks_per_sm),
                             grid_for(s, s->tune.scatter_blocks_per_sm), s->stream, !s->sorted_valid);
         }
         {
-            // electron bins laid out (a scan of three, k_ebins), movers
-            // inserted (k_insert, k_insert_dense)
-            Timed t(s, K_SCATTER, capturing, 6);
+            // electron bins laid out (a scan, k_ebins), movers inserted
+            // (k_insert, k_insert_dense)
+            Timed t(s, K_SCATTER, capturing, 3 + scan_launches(s->L.ncell_pad));
             launch_insert(a, s->st, P, grid_for(s, s->tune.scatter_blocks_per_sm), s->stream);
         }
     }
@@ -746,7 +746,7 @@ pd_status issue_step(pd_sim* s, bool capturing) {
                      grid_for(s, s->tune.ncand_blocks_per_sm), s->stream);
     }
     {
-        Timed t(s, K_SCAN_CAND, capturing, 3);
+        Timed t(s, K_SCAN_CAND, capturing, scan_launches(s->L.ncell_pad));
         launch_scan(s->cand, s->cand_off, s->partial, s->L.ncell_pad, s->stream);
     }
     {

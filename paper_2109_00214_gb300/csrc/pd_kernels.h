@@ -7,6 +7,10 @@ namespace pd {
 constexpr int SCAN_THREADS = 256;
 constexpr uint32_t SCAN_TILE = SCAN_THREADS * 8;   // elements per scan block
 
+// scans of at most this many blocks take two launches (no k_scan_partials)
+constexpr uint32_t SCAN_DIRECT = 1024;
+inline int scan_launches(uint32_t n_padded) { return n_padded / SCAN_TILE <= SCAN_DIRECT ? 2 : 3; }
+
 inline uint32_t scan_padded(uint64_t n) { return (uint32_t)((n + SCAN_TILE - 1) / SCAN_TILE * SCAN_TILE); }
 
 // external circuit of one run
@@ -48,12 +52,12 @@ struct SortArgs {
 // heavy bins: counts, holes closed, slots borrowed by full bins (three launches)
 void launch_sort(const SortArgs& a, DevState* st, const KParams& P, int sms, cudaStream_t s);
 // a new layout of the heavy bins when one overflowed (every kernel returns at
-// once otherwise; ten launches).  first: no particle is in a bin yet (the
+// once otherwise; seven launches and a scan).  first: no particle is in a bin yet (the
 // first step after the loads), so the layout is written into A directly
 void launch_relayout(const SortArgs& a, DevState* st, const KParams& P, int grid_bins, int grid_slots,
                      cudaStream_t s, bool first);
 // the electron bins packed after the heavy bins, then every mover into its
-// bin (six launches)
+// bin (three launches and a scan)
 void launch_insert(const SortArgs& a, DevState* st, const KParams& P, int grid_dense, cudaStream_t s);
 // heavy bins that may borrow slots from their neighbours in one step (more
 // lay the bins out anew)
@@ -68,8 +72,6 @@ void launch_deposit(const Particles& A, long long* rho_e, long long* rho_h, DevS
 // (cond: when not null, the scan runs only if *cond is nonzero)
 void launch_scan(const uint32_t* in, uint32_t* out, uint32_t* partial, uint32_t n_padded, cudaStream_t s,
                  const uint32_t* cond = nullptr);
-// the same over the population counts of the input words
-void launch_scan_popc(const uint32_t* in, uint32_t* out, uint32_t* partial, uint32_t n_padded, cudaStream_t s);
 // diagnostics of one run
 // live particles of every run and species, out[run * NSP + species] (zeroed by the caller)
 void launch_species_count_all(const Particles& A, DevState* st, const KParams& P, unsigned long long* out, int grid,
