@@ -63,6 +63,10 @@ constexpr int SMALL_TILES = 4 * 152;   // long windows from this many tiles on
 constexpr int TAIL_NODES = 2048;
 constexpr int TAIL_THREADS = 512;
 constexpr int TAIL_SLOTS = 2;          // nodes of a color a thread of k_mg_tail holds (most levels: one)
+// Dynamic shared memory k_mg_tail may take: levels of up to 2048 nodes 24 KB, the
+// coarser ones a third of that, their coefficients, an inverse 40 KB at most; the
+// most of any grid is 73.7 KB (160 x 768 cells, from 40 x 192 of them on).
+constexpr size_t TAIL_SMEM_MAX = 80 * 1024;
 
 size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 
@@ -1103,9 +1107,10 @@ int field_init(FieldSolver& fs, const std::vector<pd_config>& cfgs, const std::v
     for (int r = 0; r < R; ++r)
         for (int u = 0; u < red_units(cfgs[r].nz, cfgs[r].nr); u += RED_WARPS) tasks.push_back(make_int2(r, u));
     fs.red_len = (int)tasks.size() - fs.red_off;
-    // tail levels hold 24 KB and a third of that, the inverse 40 KB (10 KB are static)
-    if (fs.tail_smem > 36 * 1024 && cudaFuncSetAttribute(k_mg_tail, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                         (int)fs.tail_smem) != cudaSuccess)
+    // The limit is the kernel's, shared by every solver of the process: always the
+    // same value, so that no solver lowers it under another's launches.
+    if (fs.tail_smem > TAIL_SMEM_MAX) return 1;
+    if (cudaFuncSetAttribute(k_mg_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TAIL_SMEM_MAX) != cudaSuccess)
         return 1;
     fs.tasks = (int2*)take(tasks.size() * sizeof(int2) + 8);
     if (o > bytes) return 1;
