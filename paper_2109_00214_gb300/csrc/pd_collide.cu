@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(NT) k_rank_tables(const uint32_t* __restrict__
                                                     const uint32_t* __restrict__ q,
                                                     const uint32_t* nq, uint32_t max_q, uint32_t C,
                                                     const DevState* st) {
-    if (st->error) return;                           // a fault was flagged: the state is not stepped further
+    if (block_faulted(st)) return;                   // a fault was flagged: the state is not stepped further
     constexpr int NWARPS = NT / 32;
     extern __shared__ uint32_t s_buf[];                 // four arrays of MAXN
     __shared__ uint32_t s_cnt[NWARPS * 256];
@@ -1393,7 +1393,7 @@ __global__ void __launch_bounds__(32 * COLL_WARPS, 4) k_collide(
     const uint4* __restrict__ nc, const uint4* __restrict__ nc2, const uint32_t* __restrict__ cand_off,
     const uint32_t* __restrict__ active, DevState* st, long long* rho_e, long long* rho_h,
     const float* __restrict__ xsE, const float* __restrict__ xs, KParams P, CollConsts cc, uint32_t big_blocks) {
-    if (st->error) return;                           // a fault was flagged: the state is not stepped further
+    if (block_faulted(st)) return;                   // a fault was flagged: the state is not stepped further
     __shared__ __align__(16) uint32_t s_sort[COLL_WARPS][COLL_SORT_WORDS + 2 * RANK_WARP_MAX];
     __shared__ uint32_t s_ctr[COLL_WARPS][OUT_N];
     __shared__ uint32_t s_nsp[COLL_WARPS];           // electrons each warp of a block's batch made
@@ -1713,7 +1713,7 @@ __device__ __forceinline__ float rayleigh(const float* __restrict__ ray, float U
 
 __global__ void __launch_bounds__(256) k_inject(Particles A, const float2* __restrict__ E, DevState* st, KParams P,
                                                 const InjectConsts* __restrict__ icv, const float* __restrict__ ray) {
-    if (st->error) return;                           // a fault was flagged: the state is not stepped further
+    if (block_faulted(st)) return;                   // a fault was flagged: the state is not stepped further
     __shared__ uint32_t ne_s[64], nn_s[64], pre_s[65];
     __shared__ unsigned long long slot0_s;
     const int run = blockIdx.x;
@@ -1820,7 +1820,7 @@ constexpr size_t SPUT_SMEM = SPUT_MAX * sizeof(unsigned long long);
 
 __global__ void __launch_bounds__(SPUT_THREADS) k_sputter(Particles M, uint32_t* mm, DevState* st, KParams P,
                                                           const float* __restrict__ ray, uint32_t* in_cnt) {
-    if (st->error) return;                           // a fault was flagged: the state is not stepped further
+    if (block_faulted(st)) return;                   // a fault was flagged: the state is not stepped further
     extern __shared__ unsigned long long s_key[];    // ion id << 32 | record index
     __shared__ uint32_t s_cnt, s_el[2], s_wsum[SPUT_THREADS / 32];
     __shared__ unsigned long long s_base;

@@ -268,6 +268,12 @@ __device__ __forceinline__ int run_of(const KParams& P, uint32_t gcell) {
 
 __device__ __forceinline__ void set_error(DevState* st, uint32_t bits) { atomicOr(&st->error, bits); }
 
+// Whether a fault was flagged, the same answer in every thread of the block (a
+// barrier).  Another block of the same launch may flag one at any moment, so warps
+// that read the word each for themselves can part: those that go on then meet
+// barriers without the others, and read shared memory that the others were to fill.
+__device__ __forceinline__ bool block_faulted(const DevState* st) { return __syncthreads_or(st->error != 0u) != 0; }
+
 // sigma(eps): linear interpolation on the grid E_k = 2^e (1 + j/64); the
 // bracketing index comes from the exponent and top six mantissa bits of eps.
 __device__ __forceinline__ float xs_lookup(const float* __restrict__ E, const float* __restrict__ s, float eps) {

@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(256, FIELD ? 3 : 4) k_push4(Particles A, const
                                                long long* rho_h, uint32_t* out_cnt, uint32_t* in_cnt,
                                                uint32_t* mv, uint32_t* mm, Particles M, DevState* st, KParams P) {
     __shared__ RunInfo s_runs[MULTI ? MAX_RUNS_SMEM : 1];
-    if (st->error) return;                           // a fault was flagged: the state is not stepped further
+    if (block_faulted(st)) return;                   // a fault was flagged: the state is not stepped further
     if (MULTI) {
         for (int r = threadIdx.x; r < P.nruns; r += blockDim.x) s_runs[r] = P.runs[r];
         __syncthreads();
@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(256) k_bins(Particles A, const uint32_t* __res
                                               const uint32_t* __restrict__ mv, uint32_t* act, int* net, uint4* bigq,
                                               uint32_t bigq_cap, uint32_t* ovq, uint32_t* ovbits, uint32_t b0,
                                               uint32_t nbins, DevState* st) {
-    if (st->error) return;                           // a fault was flagged: the state is not stepped further
+    if (block_faulted(st)) return;                   // a fault was flagged: the state is not stepped further
     long long dlive = 0;
     for (uint32_t b = b0 + blockIdx.x * blockDim.x + threadIdx.x; b < nbins; b += gridDim.x * blockDim.x) {
         const uint32_t o = out_cnt[b], in = in_cnt[b];
@@ -815,7 +815,7 @@ __device__ __forceinline__ void species_rates(const DevState* st, uint32_t since
 __global__ void __launch_bounds__(256) k_relayout_want(const uint32_t* __restrict__ cnt,
                                                        const uint32_t* __restrict__ act, const int* __restrict__ net,
                                                        uint32_t nbins, uint32_t ncell, DevState* st) {
-    if (!st->relayout || st->error) return;
+    if (!st->relayout || block_faulted(st)) return;
     const uint32_t since = st->since;
     __shared__ float s_rate[NSP], s_mean[NSP];
     species_rates(st, since, ncell, s_rate, s_mean);
@@ -864,7 +864,7 @@ __global__ void __launch_bounds__(256) k_relayout_want(const uint32_t* __restric
 __global__ void __launch_bounds__(256) k_relayout_caps(const uint32_t* __restrict__ cnt, uint32_t* cap,
                                                        uint32_t* act, int* net, uint32_t nbins, uint32_t nbins_pad,
                                                        uint32_t ncell, DevState* st, KParams P) {
-    if (!st->relayout || st->error) return;
+    if (!st->relayout || block_faulted(st)) return;
     const uint32_t since = st->since;
     __shared__ float s_rate[NSP], s_mean[NSP];
     species_rates(st, since, ncell, s_rate, s_mean);
@@ -1272,7 +1272,7 @@ __global__ void __launch_bounds__(256, 4) k_push_rz(Particles A, const float2* _
                                                                 uint32_t* mv, uint32_t* mm, Particles M, DevState* st,
                                                                 KParams P) {
     __shared__ RunInfo s_runs[MULTI ? MAX_RUNS_SMEM : 1];
-    if (st->error) return;                           // a fault was flagged: the state is not stepped further
+    if (block_faulted(st)) return;                   // a fault was flagged: the state is not stepped further
     if (MULTI) {
         for (int r = threadIdx.x; r < P.nruns; r += blockDim.x) s_runs[r] = P.runs[r];
         __syncthreads();

@@ -237,3 +237,34 @@ def test_ensemble_coulomb_per_run_matches_oracle(pd, xs):
         for key in oc:
             assert gc[key] == oc[key], (k, key, gc[key], oc[key])
         assert gc["coul_ee"] > 0 and gc["coul_ei"] > 0
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+def test_a_fault_in_one_run_is_reported(pd, xs, value):
+    """Non-finite velocities in one of 32 runs: the push flags the fault while
+    other blocks of the launch start.  The steps report it, and an ensemble
+    beside it goes on as its runs do alone."""
+    runs = []
+    for k in range(32):
+        cfg, parts = synthetic.rz_plume(n=16 + k % 16, total=3e3, seed=20 + k)
+        cfg.update(field_on=2, inject_on=0, run=k)
+        runs.append((cfg, parts))
+    fields = [_field(c, 3 + k) for k, (c, _) in enumerate(runs)]
+    good = _ensemble(pd, runs, xs, fields)
+    bad = [(c, {k: v.copy() for k, v in p.items()}) for c, p in runs]
+    bad[3][1]["vz"][:] = value
+    ens = _ensemble(pd, bad, xs, fields)
+    ens.step(2)
+    with pytest.raises(pd.PdError, match="NONFINITE"):
+        ens.synchronize()
+    good.step(2)
+    per_run = _split(good, good.particles())
+    for k in (3, 31):
+        sim = pd.Simulation(runs[k][0], xs)
+        sim.load(runs[k][1])
+        sim.set_field(*fields[k])
+        sim.step(2)
+        p = sim.particles()
+        order = np.argsort(p["id"], kind="stable")
+        for key in ("id", "species", "iz", "ir") + FLOATS:
+            assert np.array_equal(per_run[k][key], p[key][order]), (k, key)

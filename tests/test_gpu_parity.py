@@ -560,6 +560,22 @@ def test_empty_and_capacity(pd, xs):
         sim3.synchronize()
 
 
+def test_capacity_overrun_in_large_cells_is_reported(pd, xs):
+    """512 cells of some 340 candidates, a block each, whose spawns fit for a few
+    cells only: the others flag the overrun while blocks are still starting."""
+    cfg, parts = synthetic.heavy_cells(n_e=512 * 60, n_cu=512 * 60, n_cup=512 * 60, ncells=512,
+                                       coll_scale=7.5e4 * 300 / 60 ** 2)
+    sim = pd.Simulation(dict(cfg, capacity=len(parts["species"]) + 4096), xs)
+    sim.load(parts)
+    sim.step(2)
+    with pytest.raises(pd.PdError, match="CAPACITY"):
+        sim.synchronize()
+    cfg["capacity"] = 1 << 21
+    sim, o = run_pair(pd, cfg, parts, xs, 1)           # with room: as the oracle
+    assert_same_counters(sim.counters(), o.counters())
+    assert sim.counters()["cand_total"] > 512 * 256
+
+
 @pytest.mark.parametrize("lo,hi,nbins", [(0.0, 200.0, 1), (0.0, 300.0, 4096), (3.7, 3.7001, 5), (12.5, 14.0, 333),
                                          (-1.0, 1e-3, 64), (0.0, 1e9, 7)])
 def test_spectrum_bins_match_oracle(pd, xs, lo, hi, nbins):
