@@ -594,6 +594,18 @@ def test_spectrum_bins_match_oracle(pd, xs, lo, hi, nbins):
         assert np.array_equal(sim.energy_spectrum(sp, lo, hi, nbins), o.energy_spectrum(sp, lo, hi, nbins))
 
 
+@pytest.mark.parametrize("total", [5e2, 4e5])
+@pytest.mark.parametrize("nbins", [2048, 4095, 4096])
+def test_spectrum_of_many_bins_matches_oracle(pd, xs, total, nbins):
+    """Few slots a block for the bins (counted in global memory) and many (in a
+    block's own bins)."""
+    cfg, parts = synthetic.microbench(nz=16, nr=24, total=total, seed=5)
+    cfg.update(field_on=0)
+    sim, o = run_pair(pd, cfg, parts, xs, 0)
+    for sp in (0, 1):
+        assert np.array_equal(sim.energy_spectrum(sp, 0.0, 150.0, nbins), o.energy_spectrum(sp, 0.0, 150.0, nbins))
+
+
 def test_species_diagnostics_match_oracle(pd, xs):
     n = 32
     cfg, parts = synthetic.rz_plume(n=n, total=2e4, seed=9)
