@@ -392,7 +392,9 @@ void pd_net_destroy(pd_net* net);
 pd_status pd_net_set_params(pd_net* net, const float* params);
 pd_status pd_net_get_params(pd_net* net, float* params);
 /* Inference on a batch of B samples of H x W nodes stored one after another
- * (x, y: device float arrays of B H W values). */
+ * (x, y: device float arrays of B H W values).  The output that the losses below
+ * are formed from is summed in another order: it may differ from y in the last
+ * bits. */
 pd_status pd_net_forward(pd_net* net, const float* x, int B, int H, int W, float* y);
 /* Forward and back-propagation of the loss against targets t (device,
  * B H W floats): *loss (host, may be null) receives the loss and grads

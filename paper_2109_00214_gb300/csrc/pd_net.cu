@@ -6,16 +6,17 @@
 // layers, forward and back-propagation alike, are implicit GEMMs on the
 // tensor cores (mma.sync m16n8k16, bfloat16 operands, float accumulators):
 //   forward / input gradient: M = 16 nodes of a tile row, N = 32 output
-//     channels, K = 9 taps x 32 input channels; a block stages the layer's
-//     weights once and 8 x 32 node tiles with their halo in shared memory.  The
-//     input
-//     gradient is the same convolution over the output gradient with the
-//     weights mirrored in the tap and transposed in the channels.
+//     channels, K = 9 taps x 32 input channels; a warp keeps the weights of its
+//     16 output channels in registers, a block stages 8 x 32 node tiles with
+//     their halo in shared memory.  The input gradient is the same convolution
+//     over the output gradient with the weights mirrored in the tap and
+//     transposed in the channels.
 //   weight gradient: per tap, M = 32 output channels, N = 32 input channels,
 //     K = the nodes, with one warp per tap; each block sums over the tiles it
 //     visits and writes a partial that a second kernel adds up in a fixed
 //     order (so the gradient does not depend on the launch).
-// The 1 -> 32 layer, and the 32 -> 1 layer in training, run on the CUDA cores.
+// The 1 -> 32 layer, and the 32 -> 1 layer in training, run on the CUDA cores (the
+// latter in inference on the tensor cores: k_conv6).
 // Storage: activations h_1..h_5 and the gradients with respect to a_1..a_5 in
 // bfloat16 (node-major, 32 channels = 64 bytes per node), the input, output,
 // targets and the output gradient in float, weights in bfloat16 for the layers and
@@ -334,9 +335,13 @@ __global__ void __launch_bounds__(CONV_THREADS, 4) k_conv32(const bf16* __restri
 // three tap rows are three columns of one product, so that an input row's 16
 // nodes (six ldmatrix, six mma) give what it adds to the output rows above, beside
 // and below it; these meet by a shuffle and two additions.  The weights are
-// bfloat16 values already; products and sums are exact and in float as before.
-// 513^2 nodes, all layers: 115 us with a thread two nodes' 288 products on the CUDA
-// cores, 107 us.
+// bfloat16 values already, so the products are exact.  Each mma adds its 16 from
+// zero and float additions join them: an mma does not round its addition to a
+// running sum to nearest, and with the sum kept in it the layer's error against 64
+// bits was 0.75 to 1.35 times that of a sum term by term, where it is now 0.45 to
+// 0.95 (513^2 nodes, all layers: 96.4 -> 98.3 us).
+// 513^2 nodes, all layers, before the launches overlapped: 115 us with a thread two
+// nodes' 288 products on the CUDA cores, 107 us.
 __global__ void __launch_bounds__(16 * TY) k_conv6(const bf16* __restrict__ h, float* __restrict__ y,
                                                    const float* __restrict__ w6, const float* __restrict__ b6,
                                                    const uint32_t* __restrict__ base, int B, int H, int W) {
@@ -377,8 +382,11 @@ __global__ void __launch_bounds__(16 * TY) k_conv6(const bf16* __restrict__ h, f
 #pragma unroll
                 for (int kh = 0; kh < 2; ++kh) {
                     uint32_t a[4];
+                    float p[4] = {0.0f, 0.0f, 0.0f, 0.0f};
                     ldsm4(a, xl + (hi * (CX + 2) + dx) * HP + kh * 16);
-                    mma_bf16(c, a[0], a[1], a[2], a[3], wb[dx][kh][0], wb[dx][kh][1]);
+                    mma_bf16(p, a[0], a[1], a[2], a[3], wb[dx][kh][0], wb[dx][kh][1]);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) c[e] += p[e];
                 }
 #pragma unroll
             for (int half = 0; half < 2; ++half) {
@@ -400,7 +408,8 @@ __global__ void __launch_bounds__(16 * TY) k_conv6(const bf16* __restrict__ h, f
 
 // The same in training, a thread two nodes (rows r and r + 4), summed tap by tap:
 // the residual loss differentiates y twice, and its gradient (through bfloat16)
-// shows the last bit of y at 2e-5.
+// shows the last bit of y at 2e-5.  So the y of a loss and the y of inference differ
+// in the last bits.
 __global__ void __launch_bounds__(16 * TY) k_conv6_train(const bf16* __restrict__ h, float* __restrict__ y,
                                                          const float* __restrict__ w6, const float* __restrict__ b6,
                                                          const uint32_t* __restrict__ base, int B, int H, int W) {

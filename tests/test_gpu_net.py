@@ -91,6 +91,65 @@ def test_tile_edges_match_the_oracle(pd, torch, B, H, W):
     net.close()
 
 
+@pytest.mark.parametrize("B,H,W", [(1, 1, 1), (2, 9, 33), (1, 129, 65)])
+def test_inference_and_training_form_the_same_output(pd, torch, B, H, W):
+    """The last layer's sum on the tensor cores (inference) against the one tap
+    by tap (training): with inference's output as the target the loss is the mean
+    square of their difference.  Products of bfloat16 values are exact, so each
+    side is off by the rounding of its additions: 289 of at most 2^-24 S tap by
+    tap, S the sum of the terms' magnitudes; 18 products of 16 terms each, whose
+    aligned addition drops up to 2^-22 S, and three more additions."""
+    rng = np.random.default_rng(B + H * W)
+    p = _params(6)
+    x = torch.from_numpy(rng.standard_normal((B, H, W)).astype(np.float32)).cuda()
+    net = pd.Net(B * H * W, params=p)
+    y = net.forward(x)
+    loss, _ = net.loss_grad(x, y)
+    p[-289:] = np.abs(p[-289:])                        # the terms' magnitudes (activations are not negative)
+    net.set_params(p)
+    S = net.forward(x).double().cpu().numpy()
+    net.close()
+    assert np.sqrt(loss) <= (289 + 18 * 4 + 3) * 2.0 ** -24 * np.sqrt((S ** 2).mean())
+    assert S.mean() > 0
+
+
+@pytest.mark.parametrize("seed,B,H,W,positive,spread", [(1, 1, 513, 513, False, 0.0), (4, 2, 65, 65, True, 0.0),
+                                                        (5, 1, 257, 257, False, 2.0)])
+def test_last_layer_no_further_off_than_term_by_term(pd, torch, seed, B, H, W, positive, spread):
+    """The last layer alone against float64: a first layer of one tap and identity
+    layers after it give known bfloat16 activations.  Inference's sum on the
+    tensor cores is no further from the exact one than the training form, which
+    adds term by term in float (weights of both signs, of one, and of uneven size)."""
+    rng = np.random.default_rng(seed)
+    offs = np.cumsum([0] + [k for pair in cnn.layer_sizes() for k in pair])
+    p = np.zeros(offs[-1], np.float32)
+
+    def bf(a):
+        return torch.tensor(np.asarray(a, np.float32)).bfloat16().float().numpy()
+
+    w1, b1 = bf(0.7 * rng.standard_normal(32)), (0.5 * rng.standard_normal(32)).astype(np.float32)
+    w6 = bf(rng.standard_normal((9, 32)) * np.sqrt(2 / 288))
+    b6 = np.float32(0.05 * rng.standard_normal())
+    w6 = np.abs(w6) if positive else w6
+    if spread:
+        w6 = bf(w6 * np.exp(spread * rng.standard_normal((9, 32))))
+    p[offs[0] + 4 * 32:offs[0] + 5 * 32], p[offs[1]:offs[1] + 32] = w1, b1
+    for l in range(1, 5):
+        p[offs[2 * l] + 4 * 1024:offs[2 * l] + 5 * 1024] = np.eye(32, dtype=np.float32).ravel()
+    p[offs[10]:offs[11]], p[offs[11]] = w6.ravel(), b6
+    x = rng.standard_normal((B, H, W)).astype(np.float32)
+    h = bf(np.maximum(b1 + w1 * x[..., None].astype(np.float64), 0.0)).astype(np.float64)
+    h = np.pad(h, ((0, 0), (1, 1), (1, 1), (0, 0)))
+    y = np.float64(b6) + sum(h[:, t // 3:t // 3 + H, t % 3:t % 3 + W] @ w6[t].astype(np.float64) for t in range(9))
+    net = pd.Net(B * H * W, params=p)
+    xd, t = torch.from_numpy(x).cuda(), torch.from_numpy(y.astype(np.float32)).cuda()
+    inference = float(((net.forward(xd).double() - t.double()) ** 2).mean())
+    training, _ = net.loss_grad(xd, t)                 # its mean square from the same targets
+    net.close()
+    assert 0.0 < training < 1e-10 * (y ** 2).max()     # the activations are the known ones
+    assert inference <= training
+
+
 def test_gradient_check_fails_for_a_wrong_gradient(pd, torch):
     """The comparison above has teeth: the GPU gradient is far from the
     oracle's gradient of a perturbed problem (targets shifted)."""
