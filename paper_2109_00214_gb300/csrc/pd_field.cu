@@ -938,10 +938,8 @@ int field_init(FieldSolver& fs, const std::vector<pd_config>& cfgs, const std::v
     // every array starts at zero (the electrode rows of the corrections stay zero)
     if (cudaMemsetAsync(ws, 0, bytes, s) != cudaSuccess) return 1;
     fs.nruns = R;
-    fs.nlev.assign(R, 0);
     fs.host_lev.assign((size_t)R * MG_MAX_LEVELS, MGLevel{});
     fs.host_top.assign(R, MGTop{});
-    fs.max_levels = 0;
     fs.max_tail = 0;
     fs.tail_smem = 0;
     fs.tail_lev.assign(R, 0);
@@ -953,8 +951,6 @@ int field_init(FieldSolver& fs, const std::vector<pd_config>& cfgs, const std::v
         const pd_config& c = cfgs[r];
         int a[MG_MAX_LEVELS], b[MG_MAX_LEVELS], n;
         level_dims(c.nz, c.nr, a, b, n);
-        fs.nlev[r] = n;
-        fs.max_levels = std::max(fs.max_levels, n);
         fs.tail_lev[r] = tail_level(a, b, n);
         fs.max_tail = std::max(fs.max_tail, fs.tail_lev[r]);
         fs.max_nodes0 = std::max(fs.max_nodes0, (c.nz + 1) * (c.nr + 1));

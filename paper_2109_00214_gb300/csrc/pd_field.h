@@ -47,8 +47,6 @@ struct TailRun {
 
 struct FieldSolver {
     int nruns = 0;
-    int max_levels = 0;                 // deepest hierarchy over the runs
-    std::vector<int> nlev;              // levels of each run
     std::vector<MGLevel> host_lev;      // [run * MG_MAX_LEVELS + l]
     MGLevel* lev = nullptr;             // device copy of host_lev
     std::vector<MGTop> host_top;        // [run]

@@ -23,14 +23,6 @@ __device__ __forceinline__ unsigned long long warp_sum_ull(unsigned long long v)
     return v;
 }
 
-// histogram increment with one atomic per distinct bin in the warp
-__device__ __forceinline__ void warp_count(uint32_t* count, uint32_t bin, bool on) {
-    const unsigned m = __ballot_sync(FULL_MASK, on);
-    if (!on) return;
-    const unsigned g = __match_any_sync(m, bin);
-    if ((threadIdx.x & 31) == (unsigned)(__ffs(g) - 1)) atomicAdd(&count[bin], (uint32_t)__popc(g));
-}
-
 // Fixed-point CIC deposit, Eq. (9)-(10): w = rn(f * 2^16) per axis, corner
 // weights (2^16 - w_z)(2^16 - w_r), w_z (2^16 - w_r), (2^16 - w_z) w_r, w_z w_r
 // (they sum to 2^32).  Lanes holding the same key (species and cell) are
