@@ -7,14 +7,16 @@
 //              Lists of more than RANK_WARP_MAX ids that active cells use
 //              are queued for k_rank_tables.
 //   k_rank_tables  rank tables of the queued lists, one block per list.
-//   k_collide  one warp per active cell.  Candidate m draws from the stream
+//   k_collide  one warp per active cell, or a block per cell of BIG_CELL
+//              candidates or more.  Candidate m draws from the stream
 //              (cell, step, k<<28 | m): the electron and target ranks (in
 //              ascending-id order inside the cell), the acceptance number and
-//              the channel number.  The candidates that share no particle
-//              with an earlier one are applied side by side, a lane each,
-//              the others in order.  Spawned electrons go to the slots
+//              the channel number.  A batch (a candidate a thread) is applied in
+//              rounds: in each, the candidates whose earlier sharers of a particle
+//              are through, side by side.  Spawned electrons go to the slots
 //              reserved for the cell at n_alive + 2 * (candidates of the
 //              cells before it); unused reserved slots are marked dead.
+//   k_coulomb  one warp per batch of cells: the Coulomb pairs (see there).
 //   k_finalize slot / id bookkeeping and the RC circuit update.
 // Compiled with -fmad=false (decision arithmetic is rounded op by op).
 #include <algorithm>
@@ -850,11 +852,12 @@ __device__ __forceinline__ int collide_pair(Particles& A, int k, uint32_t ie, ui
 // A pair's particles and random numbers do not depend on any velocity: the
 // particles come from keyed permutations of the id ranks, and each pair
 // draws from a stream of its own (twelve uniforms for Z, then the azimuth).
-// So a cell's warp first derives them for 32 pairs at a time, flattened over
-// all the cell's classes, and then applies the pairs in waves that the
-// sequential definition allows to run side by side: the regular pairs of a
-// species with itself (disjoint), each pair of an odd count's closing triple
-// alone, and each round of N_fewer pairs of two species (disjoint) in turn.
+// So a warp first derives them for 32 pairs at a time, flattened over all the
+// classes of a batch of cells, and then applies the pairs in rounds: in each, the
+// pairs whose earlier sharers of a particle are through (by the sequential
+// definition the regular pairs of a species with itself share none, the three of
+// an odd count's closing triple do, and each pair of two species does with the
+// one N_fewer pairs before it).
 // ---------------------------------------------------------------------
 
 // Pseudo-random permutation of [0, n): four Feistel rounds (Luby and Rackoff)

@@ -260,9 +260,10 @@ __global__ void __launch_bounds__(256) k_spectrum(Particles A, DevState* st, KPa
     extern __shared__ unsigned int bins[];
     const unsigned long long n = st->n_slots;
     // Few slots and many bins: clearing and adding up a block's bins costs more than
-    // it spares.  The line is a 64th of the bins a slot of a block (32 slots and 2048
-    // bins): 2e4 particles by 4096 bins 39 -> 31 us a call, by 1024 as before.  From
-    // 2e5 particles on, all in one bin, an eighth would cost 40 -> 78 us.
+    // it spares, and the particles go straight to the histogram.  The line is 64 bins
+    // for each slot of a block's share: 2e4 particles by 4096 bins 39 -> 31 us a call,
+    // by 1024 as before; at eight bins a slot 2e5 particles in one of 2048 bins would
+    // take 78 us for 40.
     const bool direct = n * 64u < (unsigned long long)nbins * gridDim.x;
     for (int b = threadIdx.x; b < nbins && !direct; b += blockDim.x) bins[b] = 0u;
     __syncthreads();
